@@ -186,6 +186,17 @@ __device__ __forceinline__ void mma_ts_el(uint32_t d_tmem, uint32_t a_tmem, uint
         "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, p;\n\t}"
         ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate) : "memory");
 }
+// The same with an output mask: rows whose half of the tile is switched off (lanes 0-63 by off_lo, 64-127 by off_hi, all
+// ones = off) keep their accumulator.
+__device__ __forceinline__ void mma_ts_el_rows(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc,
+                                               uint32_t off_lo, uint32_t off_hi, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p, e;\n\t.reg .b64 db;\n\tsetp.ne.b32 p, %7, 0;\n\t"
+        "mov.b64 db, {%2, %3};\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, {%5, %5, %6, %6}, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(off_lo), "r"(off_hi), "r"(accumulate) : "memory");
+}
 __device__ __forceinline__ void tc_commit_el(uint32_t bar) {
     asm volatile(
         "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
@@ -292,10 +303,82 @@ struct Cfg {
     static constexpr uint32_t kOffK = 0;
     static constexpr uint32_t kOffV = kOffK + kStages * kTileBytes;
     static constexpr uint32_t kOffBar = kOffV + kStages * kTileBytes;
-    static constexpr uint32_t kSmemBytes = kOffBar + 512 + 1024;    // barriers + slack to align the base to 1 KiB
+    static constexpr uint32_t kOffPlan = kOffBar + 512;
+    static constexpr uint32_t kSmemBytes = kOffPlan + 1024;         // barriers + slack to align the base to 1 KiB
 };
 
-template <int D>
+// Step plan of the 64-token block forms, in shared memory behind the barriers: per row half a bitmap of its listed key
+// blocks, the number of entries before each bitmap word, and the entries themselves, two bytes each.
+constexpr int kPlanMaxKeyBlocks = 12288;
+constexpr uint32_t kPlanBlockMask = 0x3FFF, kPlanPad = 0x3FFF;   // a pad entry points past every token: its tiles read as zero
+constexpr int kPlanRowBit = 14;                                  // bit 14 + r: listed by row half r
+inline uint32_t plan_bytes(int nkb) { return uint32_t(ceil_div(nkb, 32)) * 12 + uint32_t(nkb + 2) * 2 + 4; }
+
+// Builds the plan of one CTA: the union of the lists of its row halves (one list when the tile is one query block).
+// Returns the number of entries, or -1 when a list is malformed (an index outside [0, nkb) or not ascending).
+template <bool kPairs>
+__device__ __forceinline__ int build_plan(const AttnArgs& a, const int32_t* list0, int n0, const int32_t* list1, int n1,
+                                          uint32_t* words, uint16_t* plan, int* total) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int bad = 0;
+    if (!kPairs) {
+        for (int i = tid; i < n0; i += kThreads) {
+            const int J = list0[i];
+            if (J < 0 || J >= a.nkb || (i > 0 && J <= list0[i - 1])) bad = 1;
+            plan[i] = uint16_t((uint32_t(J) & kPlanBlockMask) | (1u << kPlanRowBit));
+        }
+        if (tid == 0) plan[n0] = uint16_t(kPlanPad);
+        return __syncthreads_or(bad) ? -1 : n0;
+    }
+    const int nw = (a.nkb + 31) >> 5;
+    uint32_t *map0 = words, *map1 = words + nw, *before = words + 2 * nw;
+    for (int i = tid; i < 2 * nw; i += kThreads) words[i] = 0u;
+    __syncthreads();
+    for (int i = tid; i < n0 + n1; i += kThreads) {
+        const bool second = i >= n0;
+        const int32_t* l = second ? list1 : list0;
+        const int k = second ? i - n0 : i;
+        const int J = l[k];
+        if (J < 0 || J >= a.nkb || (k > 0 && J <= l[k - 1])) bad = 1;
+        else atomicOr((second ? map1 : map0) + (J >> 5), 1u << (J & 31));
+    }
+    if (__syncthreads_or(bad)) return -1;
+    if (warp == 0) {
+        int base = 0;
+        for (int w0 = 0; w0 < nw; w0 += 32) {
+            const int n = w0 + lane < nw ? __popc(map0[w0 + lane] | map1[w0 + lane]) : 0;
+            int incl = n;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int up = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += up;
+            }
+            if (w0 + lane < nw) before[w0 + lane] = base + incl - n;
+            base += __shfl_sync(0xffffffffu, incl, 31);
+        }
+        if (lane == 0) { *total = base; plan[base] = uint16_t(kPlanPad); }
+    }
+    __syncthreads();
+    for (int w = warp; w < nw; w += kThreads / 32) {
+        const uint32_t m0 = map0[w], m1 = map1[w], both = m0 | m1;
+        if ((both >> lane) & 1u)
+            plan[before[w] + __popc(both & ((1u << lane) - 1u))] =
+                uint16_t(uint32_t(w * 32 + lane) | (((m0 >> lane) & 1u) << kPlanRowBit) | (((m1 >> lane) & 1u) << (kPlanRowBit + 1)));
+    }
+    __syncthreads();
+    return *total;
+}
+
+// BQ, BK: token counts of the mask's query and key blocks (128 or 64).  The tile is 128 x 128 tokens in every form:
+//   BQ = 64: two query blocks share a CTA (neighbours in the execution order, which puts rows with like lists side by
+//            side); the CTA walks the union of their lists.  A row half that does not list a block has those scores at
+//            -inf and its accumulator rows masked out of that product, so nothing of the block (not even an infinity
+//            in V) reaches it.
+//   BK = 64: a step is two listed blocks, brought by a copy each.
+// Why a union and not 64-row products: those run at half the tensor rate.  Wan-1.3B-shaped layer with 64-token blocks
+// (12 heads, 32760 tokens, 36 % of the tiles): 10.13 ms on the mma.sync kernel, 2.51 ms here; the unions hold about 15 % more
+// tiles than the lists.
+template <int D, int BQ, int BK>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapV, const AttnArgs a) {
     using C = Cfg<D>;
@@ -308,10 +391,49 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int b = blockIdx.z, h = blockIdx.y;
     const int64_t bh = int64_t(b) * a.H + h;
-    const int I = a.order[bh * a.nqb + blockIdx.x];
-    const int T = a.counts[bh * a.nqb + I];           // steps = listed key blocks
+    constexpr bool kPairs = BQ == 64, kPlanned = BQ == 64 || BK == 64;
+    constexpr int kPerStep = kBlock / BK;             // listed key blocks in a step
+    const int x0 = kPairs ? 2 * blockIdx.x : blockIdx.x;
+    const int I = a.order[bh * a.nqb + x0];
+    int T = a.counts[bh * a.nqb + I];                 // steps = listed key blocks
     const int32_t* list = a.lists + (bh * a.nqb + I) * int64_t(a.nkb);
-    const int q0 = I * kBlock;
+    const int q0 = I * BQ;
+    // rows 64..127 of a paired tile: the next query block in the order (none: as if skipped)
+    const int I2 = kPairs && x0 + 1 < a.nqb ? a.order[bh * a.nqb + x0 + 1] : -1;
+    const int T2 = I2 >= 0 ? a.counts[bh * a.nqb + I2] : -1;
+    const int q0_2 = I2 * BQ;
+    uint16_t* plan = nullptr;
+    int n_listed = 0;                                 // entries of the plan
+
+    if (kPlanned) {
+        __shared__ int plan_total;
+        if (T > a.nkb || T2 > a.nkb) {                // counts that cannot come from compaction
+            if (tid == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_CHECK, 20, max(T, T2), blockIdx.x);
+            return;
+        }
+        if (T <= 0 && T2 <= 0) {                      // nothing to attend to: O = 0, LSE = -inf where a block is listed empty
+            const bool second = kPairs && tid >= BQ;
+            const int row = second ? q0_2 + tid - BQ : q0 + tid;
+            if (tid < kBlock && (second ? T2 : T) == 0 && row < a.N) {
+                __nv_bfloat16* op = a.O + b * a.os[0] + h * a.os[1] + int64_t(row) * a.os[2];
+#pragma unroll
+                for (int c = 0; c < D / 8; ++c) *reinterpret_cast<uint4*>(op + c * 8) = make_uint4(0, 0, 0, 0);
+                a.LSE[bh * a.N + row] = -INFINITY;
+            }
+            return;
+        }
+        unsigned char* area = smem_dyn + (((smem_u32(smem_dyn) + 1023u) & ~1023u) - smem_u32(smem_dyn)) + C::kOffPlan;
+        uint32_t* words = reinterpret_cast<uint32_t*>(area);
+        plan = reinterpret_cast<uint16_t*>(area + (kPairs ? ((a.nkb + 31) >> 5) * 12 : 0));
+        n_listed = build_plan<kPairs>(a, list, max(T, 0), a.lists + (bh * a.nqb + max(I2, 0)) * int64_t(a.nkb), max(T2, 0),
+                                      words, plan, &plan_total);
+        if (n_listed < 0) {
+            if (tid == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_CHECK, 21, I, blockIdx.x);
+            return;
+        }
+    }
+    const int T1 = T;                                 // listed key blocks of the (first) query block
+    if (kPlanned) T = (n_listed + kPerStep - 1) / kPerStep;
 
     if (T < 0) return;                      // skipped query block (region-restricted form): output untouched
     if (T > a.nkb) {                        // a count that cannot come from compaction: stop before reading a list that long
@@ -385,18 +507,21 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
                 if (u >= 0 && !mbar_wait(bar_sfull(u & 1), uint32_t(u >> 1) & 1u, abortp, 100, limit)) {
                     set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 1, i, blockIdx.x); break;
                 }
-                const int J = list[i];
-                if (J < 0 || J >= a.nkb || (i > 0 && J <= list[i - 1])) {      // malformed list: stop before touching memory
+                const int J = kPlanned ? 0 : list[i];
+                if (!kPlanned && (J < 0 || J >= a.nkb || (i > 0 && J <= list[i - 1]))) {   // malformed list: stop before touching memory
                     set_status(a.hdr, CARNATOR_ERR_DEVICE_CHECK, 21, i, blockIdx.x); *abortp = 1; break;
                 }
                 // Test of the time-out path only: the first K tile of the first query block in the order is never
                 // requested, so the wait for it runs out and the CTA takes the abort-and-drain path.
                 if (i == 0 && a.hdr->debug_withhold != 0 && blockIdx.x == 0 && bh == 0) continue;
                 mbar_expect_tx(bar_kfull(s), C::kTileBytes);
-                const int key0 = J * kBlock;
 #pragma unroll
-                for (int x = 0; x < C::kBoxes; ++x)
-                    tma_load_4d(sK + s * C::kTileBytes + x * C::kBoxBytes, &mapK, bar_kfull(s), x * 64, key0, h, b);
+                for (int kh = 0; kh < kPerStep; ++kh) {
+                    const int key0 = kPlanned ? int(plan[i * kPerStep + kh] & kPlanBlockMask) * BK : J * kBlock;
+#pragma unroll
+                    for (int x = 0; x < C::kBoxes; ++x)
+                        tma_load_4d(sK + s * C::kTileBytes + x * C::kBoxBytes + kh * BK * 128, &mapK, bar_kfull(s), x * 64, key0, h, b);
+                }
                 armed = i;
             }
             if (*abortp) {      // copies in flight must land before the CTA gives its shared memory back
@@ -413,13 +538,16 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
                 if (u >= 0 && !mbar_wait(bar_pvdone(u & 1), uint32_t(u >> 1) & 1u, abortp, 100, limit)) {
                     set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 2, i, blockIdx.x); break;
                 }
-                const int J = list[i];
-                if (J < 0 || J >= a.nkb) { *abortp = 1; break; }                  // reported by the K producer
+                const int J = kPlanned ? 0 : list[i];
+                if (!kPlanned && (J < 0 || J >= a.nkb)) { *abortp = 1; break; }   // reported by the K producer
                 mbar_expect_tx(bar_vfull(s), C::kTileBytes);
-                const int key0 = J * kBlock;
 #pragma unroll
-                for (int x = 0; x < C::kBoxes; ++x)
-                    tma_load_4d(sV + s * C::kTileBytes + x * C::kBoxBytes, &mapV, bar_vfull(s), x * 64, key0, h, b);
+                for (int kh = 0; kh < kPerStep; ++kh) {
+                    const int key0 = kPlanned ? int(plan[i * kPerStep + kh] & kPlanBlockMask) * BK : J * kBlock;
+#pragma unroll
+                    for (int x = 0; x < C::kBoxes; ++x)
+                        tma_load_4d(sV + s * C::kTileBytes + x * C::kBoxBytes + kh * BK * 128, &mapV, bar_vfull(s), x * 64, key0, h, b);
+                }
                 armed = i;
             }
             if (*abortp) {
@@ -460,8 +588,14 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
                         const uint32_t v_lo = v_lo0 + uint32_t(s) * (C::kTileBytes >> 4), p_t = tmem + kColP, d_o = tmem + kColO;
                         const uint32_t acc0 = ip > 0 ? 1u : 0u;
 #pragma unroll
-                        for (int kk = 0; kk < kBlock / 16; ++kk)
-                            mma_ts_el(d_o, p_t + kk * 8, v_lo + kk * (2048 >> 4), hi_v, idesc_pv, kk > 0 ? 1u : acc0);
+                        for (int kk = 0; kk < kBlock / 16; ++kk) {
+                            if (kPairs) {       // O starts at zero; rows that do not list the block keep what they have
+                                const uint32_t e = plan[ip * kPerStep + kk / (BK / 16)] >> kPlanRowBit;
+                                mma_ts_el_rows(d_o, p_t + kk * 8, v_lo + kk * (2048 >> 4), hi_v, idesc_pv, (e & 1u) - 1u, (e >> 1) - 1u, 1u);
+                            } else {
+                                mma_ts_el(d_o, p_t + kk * 8, v_lo + kk * (2048 >> 4), hi_v, idesc_pv, kk > 0 ? 1u : acc0);
+                            }
+                        }
                         tc_commit_el(bar_pvdone(g));
                         ++ip; progress = true;
                     }
@@ -523,7 +657,9 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
         const int quarter = warp & 3, wg = warp >> 2;
         const int r_loc = quarter * 32 + lane;                      // query row within the tile
         const uint32_t lane_base = uint32_t(quarter * 32) << 16;
-        const int row = q0 + r_loc;
+        const bool second = kPairs && quarter >= 2;                 // warp-uniform: rows of the pair's second query block
+        const int row = second ? q0_2 + r_loc - BQ : q0 + r_loc;
+        const bool row_in = row < a.N && (!kPairs || (second ? T2 : T1) >= 0);   // rows of a skipped query block are left alone
         {
             // The query tile goes into tensor memory as the A operand of Q K^T (row = lane, two bf16 per column), so
             // those products read only the K tile from shared memory.  Group g brings half of the head dimension.
@@ -533,7 +669,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
                 uint32_t r[32];
 #pragma unroll
                 for (int v = 0; v < 8; ++v) {
-                    const uint4 u = row < a.N ? *reinterpret_cast<const uint4*>(qp + c * 64 + v * 8) : make_uint4(0, 0, 0, 0);
+                    const uint4 u = row_in ? *reinterpret_cast<const uint4*>(qp + c * 64 + v * 8) : make_uint4(0, 0, 0, 0);
                     r[4 * v] = u.x; r[4 * v + 1] = u.y; r[4 * v + 2] = u.z; r[4 * v + 3] = u.w;
                 }
                 tmem_st32(tmem + lane_base + kColQ + wg * (D / 4) + c * 32, r);
@@ -542,10 +678,15 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
                 uint32_t r[16];
 #pragma unroll
                 for (int v = 0; v < 4; ++v) {
-                    const uint4 u = row < a.N ? *reinterpret_cast<const uint4*>(qp + v * 8) : make_uint4(0, 0, 0, 0);
+                    const uint4 u = row_in ? *reinterpret_cast<const uint4*>(qp + v * 8) : make_uint4(0, 0, 0, 0);
                     r[4 * v] = u.x; r[4 * v + 1] = u.y; r[4 * v + 2] = u.z; r[4 * v + 3] = u.w;
                 }
                 tmem_st16(tmem + lane_base + kColQ + wg * 16, r);
+            }
+            if (kPairs) {       // the products into O are masked by rows, so none of them can be the one that starts it
+                const uint32_t zero[32] = {};
+#pragma unroll
+                for (int c = 0; c < D / 64; ++c) tmem_st32(tmem + lane_base + kColO + wg * (D / 2) + c * 32, zero);
             }
             tmem_wait_st();
             tc_fence_before();
@@ -554,7 +695,12 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
         float m_w = -INFINITY, l_w = 0.f;                           // this group's reference and partial row sum
         bool ok = true;
         // lists ascend, so only the last listed block can be the ragged one: read it once, off the per-step path
-        const int nvalid_last = a.N - list[T - 1] * kBlock;
+        int nvalid_last;
+        if (!kPlanned) nvalid_last = a.N - list[T - 1] * kBlock;
+        else {
+            const int left = min(BK, a.N - int(plan[n_listed - 1] & kPlanBlockMask) * BK);
+            nvalid_last = ((n_listed - 1) % kPerStep) * BK + left;
+        }
         for (int i = wg; i < T; i += 2) {
             const int rs = i % kRefSlots;
             const uint32_t sph = uint32_t(i >> 1) & 1u;
@@ -576,6 +722,21 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
 #pragma unroll
                     for (int e = 0; e < 32; ++e)
                         if (c * 32 + e >= nvalid) s[c][e] = -INFINITY;
+            }
+            // 64-token blocks: the halves of the step that this warp's rows list (a pad entry is listed by nobody)
+            bool on0 = true, on1 = true;
+            if (kPlanned) {
+                const int bit = kPlanRowBit + (second ? 1 : 0);
+                on0 = (plan[i * kPerStep] >> bit) & 1;
+                on1 = (plan[i * kPerStep + kPerStep - 1] >> bit) & 1;
+                if (!on0) {
+#pragma unroll
+                    for (int e = 0; e < 64; ++e) s[e >> 5][e & 31] = -INFINITY;
+                }
+                if (!on1) {
+#pragma unroll
+                    for (int e = 64; e < 128; ++e) s[e >> 5][e & 31] = -INFINITY;
+                }
             }
             // row maximum of the raw scores (the scale is positive), four independent chains
             float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
@@ -608,7 +769,8 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
                 ok = mbar_wait_warp(bar_pvdone(wg ^ 1), uint32_t((i - 1) >> 1) & 1u, abortp, 0, limit);
                 if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 9, i, blockIdx.x); break; }
                 tc_fence_after();
-                const float f = ex2_approx(r_prev - r_now);          // 1 for rows that did not move
+                // 1 for rows that did not move (rows of a pair may both times be at -inf: nothing listed so far)
+                const float f = !kPairs || grow ? ex2_approx(r_prev - r_now) : 1.f;
 #pragma unroll
                 for (int c = 0; c < D / 32; ++c) {
                     float o[32];
@@ -625,6 +787,10 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
             const uint64_t neg_m2 = pack2(-r_now, -r_now), scale2 = pack2(a.scale_log2, a.scale_log2);
             uint64_t part2[2] = {pack2(0.f, 0.f), pack2(0.f, 0.f)};
             uint32_t pk[4][16];
+            if (kPairs && !on0 && !on1) {        // warp-uniform: nothing of this step belongs to these rows (their reference may be -inf)
+#pragma unroll
+                for (int e = 0; e < 64; ++e) pk[e >> 4][e & 15] = 0u;
+            } else {
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
 #pragma unroll
@@ -635,6 +801,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
                     part2[e & 1] = add2(part2[e & 1], pack2(p0, p1));
                     pk[c][e] = pack_bf16(p0, p1);
                 }
+            }
             }
             if (!p_free) {      // the one P buffer is free once P V of step i-1 (the other group's) has read it
                 ok = mbar_wait_warp(bar_pvdone(wg ^ 1), uint32_t((i - 1) >> 1) & 1u, abortp, 0, limit);
@@ -667,8 +834,10 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
             tc_fence_after();
             const float m0 = fin[0][0][r_loc], m1 = fin[1][0][r_loc];
             const float r_fin = fmaxf(m0, m1);
-            const float l_tot = fin[0][1][r_loc] * ex2_approx(m0 - r_fin) + fin[1][1][r_loc] * ex2_approx(m1 - r_fin);
-            const float inv = 1.f / l_tot;
+            float l_tot = fin[0][1][r_loc] * ex2_approx(m0 - r_fin) + fin[1][1][r_loc] * ex2_approx(m1 - r_fin);
+            if (kPairs && (second ? T2 : T1) <= 0) l_tot = 0.f;
+            // rows of a pair that list nothing: O = 0, LSE = -inf
+            const float inv = !kPairs || l_tot > 0.f ? 1.f / l_tot : 0.f;
             // each group writes half of the head dimension
             __nv_bfloat16* op = a.O + b * a.os[0] + h * a.os[1] + int64_t(row) * a.os[2] + wg * (D / 2);
 #pragma unroll
@@ -676,7 +845,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
                 float o[32];
                 tmem_ld32(tmem + lane_base + kColO + wg * (D / 2) + c * 32, o);      // warp-collective: every lane takes part
                 tmem_wait_ld();
-                if (row < a.N) {
+                if (row_in) {
 #pragma unroll
                     for (int v = 0; v < 4; ++v) {
                         uint4 u;
@@ -688,7 +857,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
                     }
                 }
             }
-            if (wg == 0 && row < a.N) a.LSE[bh * a.N + row] = (r_fin + log2f(l_tot)) * kLn2;
+            if (wg == 0 && row_in) a.LSE[bh * a.N + row] = !kPairs || l_tot > 0.f ? (r_fin + log2f(l_tot)) * kLn2 : -INFINITY;
         }
     }
 
@@ -801,17 +970,26 @@ inline bool tma_strides_ok(const carnator_shape* s, const int64_t st[3]) {
     return (s->B == 1 || st[0] > 0) && (s->H == 1 || st[1] > 0);
 }
 
+// Shapes for which the caller may ask for this kernel by name: 128-token blocks.
 inline bool tcgen05_supported(const carnator_shape* s) {
     return s->block_q == tc::kBlock && s->block_k == tc::kBlock && (s->D == 64 || s->D == 128) &&
            tma_strides_ok(s, s->k_stride) && tma_strides_ok(s, s->v_stride);
 }
 
-template <int D>
+// Shapes that run on it when the library chooses.  The forms with 64-token blocks keep a plan of the listed key blocks in
+// shared memory, 2.4 bytes a block beside 194 KB of tiles at D = 128; beyond 12288 key blocks the portable kernel stays.
+inline bool tcgen05_takes(const carnator_shape* s) {
+    if (s->block_q == tc::kBlock && s->block_k == tc::kBlock) return tcgen05_supported(s);
+    return (s->D == 64 || s->D == 128) && ceil_div(s->N, s->block_k) <= tc::kPlanMaxKeyBlocks &&
+           tma_strides_ok(s, s->k_stride) && tma_strides_ok(s, s->v_stride);
+}
+
+template <int D, int BQ, int BK>
 inline carnator_status launch_tc(const AttnArgs& a, const CUtensorMap& mk, const CUtensorMap& mv,
                                  cudaStream_t stream, char* err, size_t errlen) {
-    using C = tc::Cfg<D>;
-    auto kern = tc::attn_tcgen05_kernel<D>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::kSmemBytes));
+    const uint32_t smem = tc::Cfg<D>::kSmemBytes + (BQ == 64 || BK == 64 ? tc::plan_bytes(a.nkb) : 0u);
+    auto kern = tc::attn_tcgen05_kernel<D, BQ, BK>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) { snprintf(err, errlen, "cudaFuncSetAttribute(tcgen05): %s", cudaGetErrorString(e)); return CARNATOR_ERR_CUDA; }
     // The register hand-over inside the kernel only completes if the CTA owns enough registers: check what the
     // compiler allocated instead of finding out on the device.
@@ -822,23 +1000,32 @@ inline carnator_status launch_tc(const AttnArgs& a, const CUtensorMap& mk, const
         snprintf(err, errlen, "attn_tcgen05_kernel was built with %d registers per thread: too few for its setmaxnreg split", fa.numRegs);
         return CARNATOR_ERR_UNSUPPORTED;
     }
-    dim3 grid(a.nqb, a.H, a.B);
-    kern<<<grid, tc::kThreads, C::kSmemBytes, stream>>>(mk, mv, a);
+    dim3 grid(BQ == 64 ? ceil_div(a.nqb, 2) : a.nqb, a.H, a.B);
+    kern<<<grid, tc::kThreads, smem, stream>>>(mk, mv, a);
     e = cudaGetLastError();
     if (e != cudaSuccess) { snprintf(err, errlen, "attn_tcgen05_kernel: %s", cudaGetErrorString(e)); return CARNATOR_ERR_CUDA; }
     return CARNATOR_OK;
 }
 
+template <int D>
+inline carnator_status launch_tc_blocks(const AttnArgs& a, const CUtensorMap& mk, const CUtensorMap& mv,
+                                        cudaStream_t stream, char* err, size_t errlen) {
+    if (a.block_q == 128) return a.block_k == 128 ? launch_tc<D, 128, 128>(a, mk, mv, stream, err, errlen)
+                                                  : launch_tc<D, 128, 64>(a, mk, mv, stream, err, errlen);
+    return a.block_k == 128 ? launch_tc<D, 64, 128>(a, mk, mv, stream, err, errlen)
+                            : launch_tc<D, 64, 64>(a, mk, mv, stream, err, errlen);
+}
+
 inline carnator_status launch_tcgen05(const AttnArgs& a, const carnator_shape* s, cudaStream_t stream,
                                       char* err, size_t errlen, long long* launches) {
     CUtensorMap mk, mv;      // Q is read with plain loads (once per CTA, into tensor memory)
-    if (!tc::make_map(&mk, a.K, a.B, a.H, a.N, s->D, a.ks, tc::kBlock) ||
-        !tc::make_map(&mv, a.V, a.B, a.H, a.N, s->D, a.vs, tc::kBlock)) {
+    if (!tc::make_map(&mk, a.K, a.B, a.H, a.N, s->D, a.ks, a.block_k) ||
+        !tc::make_map(&mv, a.V, a.B, a.H, a.N, s->D, a.vs, a.block_k)) {
         snprintf(err, errlen, "cuTensorMapEncodeTiled failed or is unavailable");
         return CARNATOR_ERR_CUDA;
     }
-    carnator_status st = (s->D == 128) ? launch_tc<128>(a, mk, mv, stream, err, errlen)
-                                       : launch_tc<64>(a, mk, mv, stream, err, errlen);
+    carnator_status st = (s->D == 128) ? launch_tc_blocks<128>(a, mk, mv, stream, err, errlen)
+                                       : launch_tc_blocks<64>(a, mk, mv, stream, err, errlen);
     if (st == CARNATOR_OK) *launches = 1;
     return st;
 }

@@ -464,7 +464,7 @@ extern "C" carnator_status carnator_sparse_attn_compacted(const void* Q, const v
     a.block_q = s->block_q; a.block_k = s->block_k;
     a.scale_log2 = effective_scale(s) * kLog2e;
 
-    const bool use_tc = tc_ok && s->attn_impl != CARNATOR_IMPL_PORTABLE;
+    const bool use_tc = s->attn_impl == CARNATOR_IMPL_TCGEN05 || (s->attn_impl == CARNATOR_IMPL_AUTO && tcgen05_takes(s));
     if (use_tc) {
         long long n = 0;
         st = launch_tcgen05(a, s, stream, g_cuda_error, sizeof(g_cuda_error), &n);

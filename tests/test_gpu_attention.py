@@ -323,3 +323,68 @@ def test_host_buffer_call_equals_device_call(name, kw):
     O_dev = O[:, :, : w.N].contiguous().view(torch.int16).cpu()
     assert torch.equal(hO, O_dev)
     assert torch.equal(hL, L[:, :, : w.N].cpu())
+
+
+# 64-token blocks on the tensor-core kernel: pairs of query blocks over the union of their lists, two key blocks to a step.
+# Sizes at the edges: one block, an odd number of query blocks, an odd number of listed blocks, a ragged tail of 1 / 63 / 64.
+@pytest.mark.parametrize("D,bq,bk,N,density", [(128, 64, 64, 40, 1.0), (128, 64, 64, 64 * 7, 0.3), (128, 64, 64, 64 * 12 + 1, 0.5),
+                                               (64, 64, 64, 64 * 9 + 63, 0.2), (128, 64, 64, 64 * 70 + 5, 0.1), (64, 64, 64, 2500, 0.9),
+                                               (128, 64, 128, 1300, 0.4), (64, 64, 128, 129, 0.6), (64, 128, 64, 1000, 0.3),
+                                               (128, 128, 64, 64 * 33 + 1, 0.5), (128, 128, 64, 64, 1.0)])
+def test_blocks_of_64_on_the_tensor_core_kernel(D, bq, bk, N, density):
+    rng = np.random.default_rng(N * 3 + D + bq)
+    B, H = 2, 2
+    Qb, Kb, Vb = (rand_bits(rng, (B, H, N, D)) for _ in range(3))
+    nqb, nkb = -(-N // bq), -(-N // bk)
+    mask = (rng.random((B, H, nqb, nkb)) < density).astype(np.uint8)
+    mask[0, 0, :: 3] = 0                                         # empty rows beside listed ones
+    mask[1, 1, nqb - 1] = 0
+    mask[1, 1, nqb - 1, nkb - 1] = 1                             # a row that sees only the last block
+    rec = (rng.random((B, nqb)) < 0.2).astype(np.uint8)
+    rec[0, 0] = 0
+    launches = cn.kernel_launches()
+    O, L, ws, shape = _run(Qb, Kb, Vb, N, 0, 1, 1, N, bq, bk, mask, rec, cn.IMPL_AUTO)
+    assert cn.kernel_launches() > launches
+    O_ref, L_ref = orc.attention_full(Qb, Kb, Vb, N, bq, bk, 1.0 / np.sqrt(D), mask, rec)
+    check_attention(o_to_host(O), L.cpu().numpy(), O_ref, L_ref, f"D{D} bq{bq} bk{bk} N{N}")
+    eff = (mask != 0) | (rec != 0)[:, None, :, None]
+    assert cn.compacted_tiles(shape, ws) == int(eff.sum())
+
+
+@pytest.mark.parametrize("bk", [64, 128])
+def test_query_blocks_that_share_a_tile_do_not_see_each_others_keys(bk):
+    """Two 64-token query blocks share a tile.  Infinities and NaN in the K and V of a block must reach only the rows that
+    list it, in whatever order the blocks come, and rows of a skipped query block stay as they were."""
+    rng = np.random.default_rng(77)
+    B, H, N, D, bq = 1, 1, 64 * 11, 128, 64
+    Qb, Kb, Vb = (rand_bits(rng, (B, H, N, D)) for _ in range(3))
+    nqb, nkb = -(-N // bq), -(-N // bk)
+    mask = (rng.random((B, H, nqb, nkb)) < 0.6).astype(np.uint8)
+    bad = [0, nkb // 2]
+    mask[0, 0, ::2, bad] = 0
+    mask[0, 0, 1::2, bad] = 1
+    mask[0, 0, 4] = 0                                            # empty: O = 0, LSE = -inf beside a row with NaN
+    Q, K, V = to_dev(Qb), to_dev(Kb), to_dev(Vb)
+    for n, J in enumerate(bad):
+        V[:, :, J * bk:(J + 1) * bk] = float("nan") if n else float("inf")
+        K[:, :, J * bk + 1] = float("inf") if n else float("nan")
+    shape = cn.make_shape(B, H, N, D, 0, 1, 1, N, bq, bk, Q, K, V)
+    active = torch.ones((B, nqb), dtype=torch.uint8, device="cuda")
+    active[0, 6] = 0
+    ones = torch.ones((B, nkb), dtype=torch.uint8, device="cuda")
+    out = []
+    for impl in (cn.IMPL_PORTABLE, cn.IMPL_AUTO):
+        shape.attn_impl = impl
+        O = torch.full((B, H, N, D), 3.0, dtype=torch.bfloat16, device="cuda")
+        L = torch.full((B, H, N), -7.0, dtype=torch.float32, device="cuda")
+        ws = cn.sparse_attn_region(Q, K, V, torch.from_numpy(mask).cuda(), active, ones, shape, O, L)
+        assert cn.query_status(ws) == cn.OK
+        out.append((O.float(), L))
+    (O0, L0), (O1, L1) = out
+    assert torch.equal(O0.isnan(), O1.isnan()) and torch.equal(L0.isnan(), L1.isnan())
+    assert torch.equal(L0.isneginf(), L1.isneginf())
+    clean = np.repeat((mask[0, 0][:, bad] == 0).all(1), bq)[:N]
+    assert torch.isfinite(O1[0, 0, torch.from_numpy(clean).cuda()]).all()
+    assert bool((O1[0, 0, 6 * bq:7 * bq] == 3.0).all()) and bool((L1[0, 0, 6 * bq:7 * bq] == -7.0).all())
+    ok = torch.isfinite(O0)
+    assert float((O0[ok] - O1[ok]).abs().max()) <= 2e-2
