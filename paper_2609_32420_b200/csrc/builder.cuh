@@ -17,6 +17,7 @@ struct PoolArgs {
     int nb[2];
     float* out[2];     // [B,H,nb,D]
     int N, H;
+    WsHeader* hdr;
 };
 
 __device__ __forceinline__ uint4 ld_stream16(const void* p) {
@@ -26,17 +27,31 @@ __device__ __forceinline__ uint4 ld_stream16(const void* p) {
     return v;
 }
 
+// Programmatic dependent launch: the next kernel of a call starts while this one drains, and waits here for its results.
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// A CTA takes 32 KB of consecutive tokens, one block at D = 128 and two at D = 64, with all eight 16-byte loads of a thread
+// in flight at once (with four loads, and 16 KB per CTA at D = 64, 218 MB took 46 us).
+// The first CTA clears the workspace header for the kernels behind it.
 template <int D>
 __global__ void __launch_bounds__(256) pool_kernel(PoolArgs a) {
     constexpr int TPR = D / 8;          // threads per token row (16 B each)
-    constexpr int RPP = 256 / TPR;      // token rows per pass
+    constexpr int TPB = 2 * D;          // threads per block of tokens
+    constexpr int RPP = TPB / TPR;      // token rows per pass (16)
+    constexpr int BPC = 256 / TPB;      // blocks per CTA
+    constexpr int U = 128 / RPP;        // passes of a 128-token block
+    grid_launch_dependents();
+    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x < sizeof(WsHeader) / 4)
+        reinterpret_cast<int32_t*>(a.hdr)[threadIdx.x] = 0;
     const int which = blockIdx.z & 1;
     const int b = blockIdx.z >> 1;
     const int h = blockIdx.y;
-    const int I = blockIdx.x;
+    const int part = threadIdx.x / TPB, t = threadIdx.x % TPB;
+    const int I = blockIdx.x * BPC + part;
     // select with ternaries: dynamic indexing of the argument struct would force a local copy
     const int nb = which ? a.nb[1] : a.nb[0];
-    if (I >= nb) return;
+    if (int(blockIdx.x) * BPC >= nb) return;
     const int block = which ? a.block[1] : a.block[0];
     const __nv_bfloat16* X = which ? a.X[1] : a.X[0];
     float* out = which ? a.out[1] : a.out[0];
@@ -44,42 +59,38 @@ __global__ void __launch_bounds__(256) pool_kernel(PoolArgs a) {
     const int64_t sh = which ? a.stride[1][1] : a.stride[0][1];
     const int64_t sn = which ? a.stride[1][2] : a.stride[0][2];
     const int tok0 = I * block;
-    const int nvalid = min(block, a.N - tok0);
-    const int r = threadIdx.x / TPR, c = threadIdx.x % TPR;
+    const int nvalid = I < nb ? min(block, a.N - tok0) : 0;
+    const int r = t / TPR, c = t % TPR;
     const __nv_bfloat16* base = X + b * sb + h * sh + int64_t(tok0) * sn + c * 8;
 
+    uint4 v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int row = r + u * RPP;
+        v[u] = (row < nvalid) ? ld_stream16(base + int64_t(row) * sn) : make_uint4(0, 0, 0, 0);
+    }
     float acc[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-
-    // rows r, r+RPP, ...; issue up to four independent 16-byte loads before using them
-    for (int row0 = r; row0 < nvalid; row0 += 4 * RPP) {
-        uint4 v[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            int row = row0 + u * RPP;
-            v[u] = (row < nvalid) ? ld_stream16(base + int64_t(row) * sn) : make_uint4(0, 0, 0, 0);
-        }
+    for (int u = 0; u < U; ++u) {
+        const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                acc[2 * e]     += __uint_as_float(w[e] << 16);
-                acc[2 * e + 1] += __uint_as_float(w[e] & 0xFFFF0000u);
-            }
+        for (int e = 0; e < 4; ++e) {
+            acc[2 * e]     += __uint_as_float(w[e] << 16);
+            acc[2 * e + 1] += __uint_as_float(w[e] & 0xFFFF0000u);
         }
     }
 
-    __shared__ float red[RPP][D + 4];
+    __shared__ float red[BPC][RPP][D + 4];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) red[r][c * 8 + e] = acc[e];
+    for (int e = 0; e < 8; ++e) red[part][r][c * 8 + e] = acc[e];
     __syncthreads();
-    if (threadIdx.x < D) {
+    if (t < D && I < nb) {
         float s = 0.f;
 #pragma unroll
-        for (int rr = 0; rr < RPP; ++rr) s += red[rr][threadIdx.x];
-        out[((int64_t(b) * a.H + h) * nb + I) * D + threadIdx.x] = s / float(nvalid);
+        for (int rr = 0; rr < RPP; ++rr) s += red[part][rr][t];
+        out[((int64_t(b) * a.H + h) * nb + I) * D + t] = s / float(nvalid);
     }
 }
 
@@ -180,6 +191,12 @@ __device__ __forceinline__ T block_sum(T v, T* scratch /* >= 8 */) {
     return t;
 }
 
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
 struct SelectArgs {
     const float* scores;   // [B,H,nqb,nkb]
     uint8_t* mask;         // [B,H,nqb,nkb]
@@ -193,7 +210,7 @@ struct SelectArgs {
 };
 
 // One CTA (256 threads) per (b,h,I).  Dynamic shared memory: npad uint64 sort keys + nkb keep bytes
-// (+ npad doubles for the cumulative-mass mode).
+// (+ npad doubles for the cumulative-mass mode).  Cumulative-mass rows of more than 1024 key blocks.
 __global__ void __launch_bounds__(256) select_kernel(SelectArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned long long* keys = reinterpret_cast<unsigned long long*>(smem_raw);
@@ -303,7 +320,244 @@ __global__ void __launch_bounds__(256) select_kernel(SelectArgs a) {
     for (int J = tid; J < a.nkb; J += nt) a.mask[row + J] = keep[J];
 }
 
-// Top-k mode without a sort: one warp per (b,h,I).  Each lane keeps the order-preserving keys of the
+// Selection of one row by one warp, the row's scores at `s` (shared or global memory), without a sort: each lane keeps the
+// order-preserving keys of the blocks J = lane, lane + 32, ... in registers and the warp searches the threshold key bit by bit.
+//   top-k: the largest T that at least n_admit keys reach; equal keys are admitted in ascending block order.
+//   cumulative mass: blocks are admitted in descending order as long as the mass kept before them is below the target, so T
+//   is the largest key for which the forced mass plus the mass of the keys >= T reaches the target; the search narrows an
+//   interval of keys and ends when one block is left in it (about 12 of the 32 bits).  The masses are fp64, as in the sort
+//   that select_kernel does.
+template <int NPL>   // keys per lane: nkb <= 32 * NPL
+__device__ __forceinline__ void select_row(const SelectArgs& a, const float* s, int I, uint8_t* mask_row) {
+    const int lane = threadIdx.x & 31;
+    const Geometry& g = a.g;
+    const int nkb = a.nkb;
+    const int text_cols = (g.text_dense && g.n_text > 0) ? (g.n_text + g.bk - 1) / g.bk : 0;
+    // Always-kept key blocks of the frame window: blocks are runs of consecutive tokens, so the blocks that touch frames
+    // [f_lo, f_hi] are the interval of blocks that touch tokens [n_text + f_lo hw, n_text + (f_hi + 1) hw).
+    int j_lo = 1, j_hi = 0;
+    if (g.window >= 0) {
+        const int q_lo = max(I * g.bq, g.n_text), q_hi = min(g.N, (I + 1) * g.bq) - 1;
+        if (q_hi >= q_lo) {
+            const int f_lo = max(0, (q_lo - g.n_text) / g.hw - g.window);
+            const int f_hi = min(g.T - 1, (q_hi - g.n_text) / g.hw + g.window);
+            j_lo = (g.n_text + f_lo * g.hw) / g.bk;
+            j_hi = (min(g.N, g.n_text + (f_hi + 1) * g.hw) - 1) / g.bk;
+        }
+    }
+    if (g.text_dense && g.n_text > 0 && I * g.bq < g.n_text) { j_lo = 0; j_hi = nkb - 1; }
+
+    uint32_t key[NPL], forced = 0u;      // bit q: block q * 32 + lane is always kept (its key is 0 and never competes)
+    static_assert(NPL <= 32, "one word of always-kept bits per lane");
+    float smax = -INFINITY;
+#pragma unroll
+    for (int q = 0; q < NPL; ++q) {
+        const int J = q * 32 + lane;
+        key[q] = 0u;
+        if (J < nkb) {
+            const float v = s[J];
+            smax = fmaxf(smax, v);
+            if (J < text_cols || (J >= j_lo && J <= j_hi)) forced |= 1u << q;
+            else key[q] = ordered_bits(v);
+        }
+    }
+    const int nforced = __reduce_add_sync(0xffffffffu, __popc(forced));
+    const int nfree = nkb - nforced;
+
+    // bits above the first one in which two competing keys differ are the same in every such key
+    uint32_t k_or = 0u, k_and = 0xFFFFFFFFu;
+#pragma unroll
+    for (int q = 0; q < NPL; ++q) { k_or |= key[q]; k_and &= key[q] ? key[q] : 0xFFFFFFFFu; }
+    k_or = __reduce_or_sync(0xffffffffu, k_or);
+    k_and = __reduce_and_sync(0xffffffffu, k_and);
+    const int top = 31 - __clz(int((k_or ^ k_and) | 1u));
+    uint32_t T = (top >= 31) ? 0u : (k_and & ~((2u << top) - 1u));
+
+    int need_eq = 0;                     // blocks with key == T that are admitted, lowest index first
+    bool any = true;                     // false: nothing is admitted by score
+    if (a.mode == CARNATOR_MODE_TOPK) {
+        int n_admit = a.count_includes_forced ? max(0, a.k_all - nforced) : topk_count_dev(a.keep_ratio, nfree);
+        n_admit = min(n_admit, nfree);
+        any = n_admit > 0;
+        bool exact = !any;               // a threshold that exactly n_admit keys reach: no tie to break
+#pragma unroll 1
+        for (int bit = top; bit >= 0 && !exact; --bit) {
+            const uint32_t cand = T | (1u << bit);
+            int c = 0;
+#pragma unroll
+            for (int q = 0; q < NPL; ++q) c += (key[q] >= cand) ? 1 : 0;
+            c = __reduce_add_sync(0xffffffffu, c);
+            if (c >= n_admit) { T = cand; exact = c == n_admit; }
+        }
+        if (exact) need_eq = nkb;        // every key >= T
+        else {
+            int gt = 0;
+#pragma unroll
+            for (int q = 0; q < NPL; ++q) gt += (key[q] > T) ? 1 : 0;
+            need_eq = n_admit - __reduce_add_sync(0xffffffffu, gt);
+        }
+    } else {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) smax = fmaxf(smax, __shfl_xor_sync(0xffffffffu, smax, o));
+        double e[NPL], all = 0.0, kept = 0.0;
+#pragma unroll
+        for (int q = 0; q < NPL; ++q) {
+            const int J = q * 32 + lane;
+            e[q] = 0.0;
+            if (J < nkb) {
+                e[q] = a.values_are_mass ? double(s[J]) : exp(double(s[J]) - double(smax));
+                all += e[q];
+                if ((forced >> q) & 1u) kept += e[q];
+            }
+        }
+        all = warp_sum(all);
+        kept = warp_sum(kept) / all;
+#pragma unroll
+        for (int q = 0; q < NPL; ++q) e[q] /= all;
+        const double target = double(a.mass);
+        // mass kept by the blocks whose key reaches c (or passes it); a NaN anywhere reads as "target reached"
+        auto mass_from = [&](uint32_t c) {
+            double m = 0.0;
+#pragma unroll
+            for (int q = 0; q < NPL; ++q) m += (key[q] >= c && key[q] != 0u) ? e[q] : 0.0;
+            return kept + warp_sum(m);
+        };
+        any = nfree > 0 && kept < target;
+        if (any && mass_from(1u) < target) {       // even all of them fall short: all are admitted
+            T = 1u; need_eq = nkb;
+        } else if (any) {
+            int inside = nfree;                    // blocks with keys in [T, T + 2^(bit+1))
+#pragma unroll 1
+            for (int bit = top; bit >= 0 && inside > 1; --bit) {
+                const uint32_t cand = T | (1u << bit);
+                int c = 0;
+#pragma unroll
+                for (int q = 0; q < NPL; ++q) c += (key[q] >= cand && (key[q] - cand) >> bit == 0u) ? 1 : 0;
+                c = __reduce_add_sync(0xffffffffu, c);
+                if (!(mass_from(cand) < target)) { T = cand; inside = c; } else inside -= c;
+            }
+            // the interval's last block (or its equal keys) is the one that reaches the target: T becomes its key
+            uint32_t low = 0xFFFFFFFFu;
+#pragma unroll
+            for (int q = 0; q < NPL; ++q) if (key[q] >= T && key[q] != 0u) low = min(low, key[q]);
+            T = __reduce_min_sync(0xffffffffu, low);
+            double over = 0.0, eq = 0.0;
+#pragma unroll
+            for (int q = 0; q < NPL; ++q) {
+                over += key[q] > T ? e[q] : 0.0;
+                eq = key[q] == T ? e[q] : eq;
+            }
+            over = kept + warp_sum(over);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) eq = fmax(eq, __shfl_xor_sync(0xffffffffu, eq, o));
+            need_eq = 0;
+            for (double run = over; run < target && need_eq < nfree && eq > 0.0; run += eq) ++need_eq;
+            if (eq == 0.0 && over < target) need_eq = nkb;
+        }
+    }
+    int seen = 0;
+#pragma unroll
+    for (int q = 0; q < NPL; ++q) {
+        const int J = q * 32 + lane;
+        const bool eq = any && key[q] == T && key[q] != 0u;
+        const unsigned bal = __ballot_sync(0xffffffffu, eq);
+        const bool keep = ((forced >> q) & 1u) || (any && key[q] > T) || (eq && seen + __popc(bal & ((1u << lane) - 1u)) < need_eq);
+        seen += __popc(bal);
+        if (J < nkb) mask_row[J] = keep ? 1 : 0;
+    }
+}
+
+// Rows whose scores lie in global memory (the exact builder's masses): one warp per (b,h,I).
+template <int NPL>
+__global__ void __launch_bounds__(256) select_rows_kernel(SelectArgs a, int rows) {
+    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (warp >= rows) return;
+    select_row<NPL>(a, a.scores + int64_t(warp) * a.nkb, warp % a.nqb, a.mask + int64_t(warp) * a.nkb);
+}
+
+// M2 + M3 for layers of up to 1024 key blocks: a CTA takes R query blocks of a head, computes their scores in fp32 (the
+// same sequence of FFMAs over the head dimension as score_kernel) into shared memory, and each of its R warps selects one
+// row there.  The key-block means come 128 at a time, 64 elements of the head dimension per step, through two cp.async
+// buffers; rows of 68 floats keep the 16-byte reads free of bank conflicts.  What this saves against score_kernel and a
+// selection kernel is a launch and the scores' way through memory.  Whole calls, before and after: 12 heads, 61 blocks, top-k
+// 34.1 -> 21.9 us; 48 heads, 139 blocks, cumulative mass 209 -> 72 us (of which the sort of every row took 153).
+constexpr int kScoreKeys = 128, kScoreLd = 68;
+template <int D, int R>
+constexpr size_t score_select_smem(int nkb) {
+    return size_t(2 * kScoreKeys * kScoreLd + R * D) * 4 + size_t(R) * ((nkb + 3) & ~3) * 4;
+}
+__device__ __forceinline__ void cp16(float* dst, const float* src, bool valid) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+                 ::"r"(uint32_t(__cvta_generic_to_shared(dst))), "l"(src), "r"(valid ? 16 : 0) : "memory");
+}
+template <int D, int R, int NPL>
+__global__ void __launch_bounds__(R * 32) score_select_kernel(const float* __restrict__ qbar, const float* __restrict__ kbar,
+                                                              float* __restrict__ scores_out, float scale, SelectArgs a) {
+    extern __shared__ __align__(16) float ssm[];
+    constexpr int NT = R * 32, NG = NT / kScoreKeys, RG = R / NG;      // threads, row groups, rows per thread (4)
+    float* const sK = ssm;                                             // [2][128][68]
+    float* const sQ = sK + 2 * kScoreKeys * kScoreLd;                  // [R][D]
+    float* const sS = sQ + R * D;                                      // [R][nkb_pad]
+    const int nkb = a.nkb, nkb_pad = (nkb + 3) & ~3;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int I0 = blockIdx.x * R;
+    const int64_t bh = int64_t(blockIdx.z) * a.H + blockIdx.y;
+    const float* K = kbar + bh * nkb * D;
+    const int steps = ((nkb + kScoreKeys - 1) / kScoreKeys) * (D / 64);
+    auto load = [&](int st) {
+        const int j0 = (st / (D / 64)) * kScoreKeys, d0 = (st % (D / 64)) * 64;
+        for (int i = tid; i < kScoreKeys * 16; i += NT) {
+            const int j = i >> 4, c = (i & 15) * 4;
+            const bool in = j0 + j < nkb;
+            cp16(sK + (st & 1) * kScoreKeys * kScoreLd + j * kScoreLd + c, K + int64_t(in ? j0 + j : 0) * D + d0 + c, in);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    grid_wait();                                                       // the means are complete
+    for (int i = tid; i < R * (D / 4); i += NT) {
+        const int r = i / (D / 4), c = (i % (D / 4)) * 4;
+        cp16(sQ + r * D + c, qbar + (bh * a.nqb + min(I0 + r, a.nqb - 1)) * D + c, true);
+    }
+    load(0);
+    float acc[RG];
+    const int key = tid & (kScoreKeys - 1), r0 = (tid / kScoreKeys) * RG;
+    for (int st = 0; st < steps; ++st) {
+        if (st + 1 < steps) { load(st + 1); asm volatile("cp.async.wait_group 1;" ::: "memory"); }
+        else asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        const int d0 = (st % (D / 64)) * 64;
+        if (d0 == 0) {
+#pragma unroll
+            for (int r = 0; r < RG; ++r) acc[r] = 0.f;
+        }
+        const float* kr = sK + (st & 1) * kScoreKeys * kScoreLd + key * kScoreLd;
+        const float* qr = sQ + r0 * D + d0;
+#pragma unroll 4
+        for (int d = 0; d < 64; d += 4) {
+            const float4 k4 = *reinterpret_cast<const float4*>(kr + d);
+#pragma unroll
+            for (int r = 0; r < RG; ++r) {
+                const float4 q4 = *reinterpret_cast<const float4*>(qr + r * D + d);
+                acc[r] = fmaf(q4.x, k4.x, acc[r]); acc[r] = fmaf(q4.y, k4.y, acc[r]);
+                acc[r] = fmaf(q4.z, k4.z, acc[r]); acc[r] = fmaf(q4.w, k4.w, acc[r]);
+            }
+        }
+        const int J = (st / (D / 64)) * kScoreKeys + key;
+        if (d0 + 64 == D && J < nkb) {
+#pragma unroll
+            for (int r = 0; r < RG; ++r) sS[(r0 + r) * nkb_pad + J] = scale * acc[r];
+        }
+        __syncthreads();
+    }
+    const int I = I0 + warp;
+    if (I >= a.nqb) return;
+    const float* row = sS + warp * nkb_pad;
+    if (scores_out)
+        for (int J = lane; J < nkb; J += 32) scores_out[(bh * a.nqb + I) * nkb + J] = row[J];
+    select_row<NPL>(a, row, I, a.mask + (bh * a.nqb + I) * nkb);
+}
+
+// Top-k rows of more than 1024 key blocks.  One warp per (b,h,I).  Each lane keeps the order-preserving keys of the
 // blocks J = lane, lane+32, ... in registers; the k-th largest key is found bit by bit (largest T with
 // #(key >= T) >= k), then equal keys are admitted in ascending block order until k is reached.
 template <int NPL>   // keys per lane: nkb <= 32 * NPL

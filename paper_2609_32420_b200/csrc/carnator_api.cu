@@ -113,6 +113,43 @@ carnator_status allow_smem(K kernel, size_t bytes) {
     return CARNATOR_OK;
 }
 
+// Launch that may begin before the kernel ahead of it in the stream has ended (that kernel calls grid_launch_dependents,
+// this one grid_wait before it reads anything of it).
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A... args) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+template <int D, int R, int NPL>
+carnator_status launch_score_select_r(const BuildWs& w, float* scores_opt, float scale, int B, const SelectArgs& sa, cudaStream_t stream) {
+    const size_t smem = score_select_smem<D, R>(sa.nkb);
+    carnator_status st = allow_smem(score_select_kernel<D, R, NPL>, smem);
+    if (st != CARNATOR_OK) return st;
+    const cudaError_t e = launch_dependent(score_select_kernel<D, R, NPL>, dim3(ceil_div(sa.nqb, R), sa.H, B), dim3(R * 32), smem, stream,
+                                           w.qbar, w.kbar, scores_opt, scale, sa);
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    return e == cudaSuccess ? CARNATOR_OK : cuda_fail(e, "score_select_kernel");
+}
+// Sixteen rows a CTA, unless that leaves SMs without one (twice over, so that a CTA's loads run under another's selection).
+template <int D, int NPL>
+carnator_status launch_score_select_d(const BuildWs& w, float* scores_opt, float scale, int B, const SelectArgs& sa, int sms, cudaStream_t stream) {
+    if (int64_t(B) * sa.H * ceil_div(sa.nqb, 16) < 2 * int64_t(sms)) return launch_score_select_r<D, 8, NPL>(w, scores_opt, scale, B, sa, stream);
+    return launch_score_select_r<D, 16, NPL>(w, scores_opt, scale, B, sa, stream);
+}
+carnator_status launch_score_select(const BuildWs& w, float* scores_opt, float scale, int B, int D, const SelectArgs& sa, int sms, cudaStream_t stream) {
+    if (sa.nkb <= 32 * 8) return D == 128 ? launch_score_select_d<128, 8>(w, scores_opt, scale, B, sa, sms, stream)
+                                          : launch_score_select_d<64, 8>(w, scores_opt, scale, B, sa, sms, stream);
+    return D == 128 ? launch_score_select_d<128, 32>(w, scores_opt, scale, B, sa, sms, stream)
+                    : launch_score_select_d<64, 32>(w, scores_opt, scale, B, sa, sms, stream);
+}
+constexpr int kMaxKeyBlocksInRegisters = 32 * 32;     // a selecting warp holds its row's keys in registers
+
 }  // namespace
 
 namespace {
@@ -219,9 +256,6 @@ extern "C" carnator_status carnator_build_connectivity(const void* Q, const void
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     float* scores = pooled_scores_opt ? pooled_scores_opt : w.scores;
 
-    // header and the per-head pooled-block counters are contiguous: one clear
-    CUDA_TRY(cudaMemsetAsync(w.hdr, 0, align256(sizeof(WsHeader)) + align256(size_t(s->B) * s->H * 4), stream));
-
     PoolArgs pa;
     pa.X[0] = static_cast<const __nv_bfloat16*>(Q);
     pa.X[1] = static_cast<const __nv_bfloat16*>(K);
@@ -229,7 +263,7 @@ extern "C" carnator_status carnator_build_connectivity(const void* Q, const void
     pa.block[0] = s->block_q; pa.block[1] = s->block_k;
     pa.nb[0] = nqb; pa.nb[1] = nkb;
     pa.out[0] = w.qbar; pa.out[1] = w.kbar;
-    pa.N = s->N; pa.H = s->H;
+    pa.N = s->N; pa.H = s->H; pa.hdr = w.hdr;
     SelectArgs sa;
     sa.scores = scores; sa.mask = mask;
     sa.nqb = nqb; sa.nkb = nkb; sa.npad = next_pow2(nkb); sa.H = s->H;
@@ -251,6 +285,8 @@ extern "C" carnator_status carnator_build_connectivity(const void* Q, const void
     const bool fused_pays = int64_t(s->B) * s->H * ceil_div(nqb, kFusedRows) >= int64_t(sms);
     if (fused_able && (choice == 2 || (choice == 0 && fused_pays))) {
         // one persistent kernel: pooling, pooled scores and selection; the scores stay on chip
+        // header and the per-head pooled-block counters are contiguous: one clear
+        CUDA_TRY(cudaMemsetAsync(w.hdr, 0, align256(sizeof(WsHeader)) + align256(size_t(s->B) * s->H * 4), stream));
         FusedArgs fa;
         fa.pool = pa; fa.sel = sa;
         fa.scores_out = pooled_scores_opt; fa.done = w.done; fa.hdr = w.hdr;
@@ -272,11 +308,15 @@ extern "C" carnator_status carnator_build_connectivity(const void* Q, const void
     }
     // M1
     {
-        dim3 grid(nqb > nkb ? nqb : nkb, s->H, 2 * s->B);
+        const int blocks = s->D == 64 ? 2 : 1;      // a CTA's share
+        dim3 grid(ceil_div(nqb > nkb ? nqb : nkb, blocks), s->H, 2 * s->B);
         if (s->D == 128) pool_kernel<128><<<grid, 256, 0, stream>>>(pa);
         else pool_kernel<64><<<grid, 256, 0, stream>>>(pa);
         LAUNCH_CHECK("pool_kernel");
     }
+    // M2 and M3
+    if (nkb <= kMaxKeyBlocksInRegisters)
+        return launch_score_select(w, pooled_scores_opt, effective_scale(s), s->B, s->D, sa, sms, stream);
     // M2
     {
         dim3 grid(ceil_div(nkb, 64), ceil_div(nqb, 64), s->B * s->H);
@@ -292,10 +332,7 @@ extern "C" carnator_status carnator_build_connectivity(const void* Q, const void
             const int rows = s->B * s->H * nqb;
             const int grid = ceil_div(rows, 8);
             const size_t tbl = size_t(nkb) * sizeof(int2);     // key-block frame table (<= 32 KiB)
-            if (nkb <= 32 * 8) select_topk_kernel<8><<<grid, 256, tbl, stream>>>(sa, rows);
-            else if (nkb <= 32 * 20) select_topk_kernel<20><<<grid, 256, tbl, stream>>>(sa, rows);
-            else if (nkb <= 32 * 32) select_topk_kernel<32><<<grid, 256, tbl, stream>>>(sa, rows);
-            else select_topk_kernel<128><<<grid, 256, tbl, stream>>>(sa, rows);
+            select_topk_kernel<128><<<grid, 256, tbl, stream>>>(sa, rows);
         } else {
             // cumulative-mass mode needs the sorted order: shared-memory bitonic sort, one CTA per row
             size_t smem = size_t(sa.npad) * 8 * 2 + ((nkb + 15) & ~15);
@@ -369,11 +406,17 @@ extern "C" carnator_status carnator_build_connectivity_exact(const void* Q, cons
     sa.count_includes_forced = 1; sa.k_all = nkb; sa.values_are_mass = 1;
     sa.g.N = s->N; sa.g.n_text = s->n_text; sa.g.hw = s->Hg * s->Wg > 0 ? s->Hg * s->Wg : 1; sa.g.T = s->T;
     sa.g.bq = s->block_q; sa.g.bk = s->block_k; sa.g.window = p->window_frames; sa.g.text_dense = p->text_dense;
-    const size_t smem = size_t(sa.npad) * 8 * 2 + ((nkb + 15) & ~15);
-    st = allow_smem(select_kernel, 72 * 1024);
-    if (st != CARNATOR_OK) return st;
-    dim3 grid(nqb, s->H, s->B);
-    select_kernel<<<grid, 256, smem, stream>>>(sa);
+    if (nkb <= kMaxKeyBlocksInRegisters) {
+        const int rows = s->B * s->H * nqb;
+        if (nkb <= 32 * 8) select_rows_kernel<8><<<ceil_div(rows, 8), 256, 0, stream>>>(sa, rows);
+        else select_rows_kernel<32><<<ceil_div(rows, 8), 256, 0, stream>>>(sa, rows);
+    } else {
+        const size_t smem = size_t(sa.npad) * 8 * 2 + ((nkb + 15) & ~15);
+        st = allow_smem(select_kernel, 72 * 1024);
+        if (st != CARNATOR_OK) return st;
+        dim3 grid(nqb, s->H, s->B);
+        select_kernel<<<grid, 256, smem, stream>>>(sa);
+    }
     LAUNCH_CHECK("select_kernel");
     return CARNATOR_OK;
 }

@@ -164,3 +164,39 @@ def test_full_size_masks_on_sampled_heads(name, keep):
     Kb = wl.gen_tensor(w, "K", "history", threads=nthreads)
     n_excused = _compare(w, Qb, Kb, heads=heads, what=f"{name} keep={w.build.keep_ratio}")
     assert n_excused <= 8
+
+
+# One kernel scores and selects for up to 1024 key blocks (a warp holds 8 or 32 keys a lane), two take more: the edges of those
+# ranges, ragged last blocks and query tiles, both CTA sizes (8 and 16 rows), unequal block sizes.
+@pytest.mark.parametrize("mode", [wl.MODE_TOPK, wl.MODE_CUMMASS], ids=["topk", "mass"])
+@pytest.mark.parametrize("B,H,N,n_text,D,bq,bk,window", [
+    (1, 1, 50, 0, 128, 64, 64, -1), (1, 1, 64 * 31 + 1, 7, 64, 128, 64, -1), (2, 3, 64 * 33, 0, 128, 64, 64, 0),
+    (1, 48, 64 * 129 - 1, 100, 64, 64, 64, 1), (1, 2, 64 * 256, 0, 64, 128, 64, -1), (1, 1, 64 * 257, 0, 128, 128, 64, 1),
+    (1, 1, 64 * 1024, 0, 64, 128, 64, -1), (1, 1, 64 * 1024 + 1, 0, 64, 128, 64, 0), (1, 2, 128 * 40 + 5, 0, 128, 128, 128, 2)])
+def test_score_and_selection_at_the_edges_of_their_ranges(B, H, N, n_text, D, bq, bk, window, mode):
+    rng = np.random.default_rng(N + D + mode)
+    T = 4 if (N - n_text) % 4 == 0 else 1
+    hw = (N - n_text) // T
+    Qb, Kb = (rng.standard_normal((B, H, N, D)).astype(np.float32) for _ in range(2))
+    Qb, Kb = ((x.view(np.uint32) >> 16).astype(np.uint16) for x in (Qb, Kb))
+    if N >= 4 * bk:
+        Kb[:, :, 2 * bk:3 * bk] = Kb[:, :, :bk]                 # equal scores: the lower index comes first
+    Q, K = to_dev(Qb), to_dev(Kb)
+    shape = cn.make_shape(B, H, N, D, n_text, T, 1, hw, bq, bk, Q, K)
+    p = cn.BuildParams()
+    p.mode, p.keep_ratio, p.mass, p.window_frames, p.text_dense, p.count_includes_forced = mode, 0.3, 0.8, window, 1, 0
+    nqb, nkb = -(-N // bq), -(-N // bk)
+    scores = torch.empty((B, H, nqb, nkb), dtype=torch.float32, device="cuda")
+    cn.debug_set_builder_path(cn.BUILDER_THREE_KERNELS)
+    try:
+        ws = torch.full((cn.build_workspace_bytes(shape, p),), 0xFF, dtype=torch.uint8, device="cuda")   # a workspace that was something else
+        mask, ws = cn.build_connectivity(Q, K, shape, p, pooled_scores=scores, ws=ws)
+        assert cn.query_status(ws) == cn.OK
+        mask2, _ = cn.build_connectivity(Q, K, shape, p)
+    finally:
+        cn.debug_set_builder_path(cn.BUILDER_AUTO)
+    assert torch.equal(mask, mask2)
+    ref = orc.build_connectivity(Qb, Kb, N, n_text, T, 1, hw, bq, bk, 1.0 / np.sqrt(D), mode, 0.3, 0.8, window, 1, 0)
+    s = scores.cpu().numpy()
+    assert np.abs(s - ref[1]).max() <= 2e-5
+    check_mask(mask.cpu().numpy(), ref[0], ref[1], ref[2], ref[3], topk_mode=(mode == wl.MODE_TOPK), what=f"N={N}")
