@@ -324,9 +324,8 @@ __global__ void __launch_bounds__(256) select_kernel(SelectArgs a) {
 // order-preserving keys of the blocks J = lane, lane + 32, ... in registers and the warp searches the threshold key bit by bit.
 //   top-k: the largest T that at least n_admit keys reach; equal keys are admitted in ascending block order.
 //   cumulative mass: blocks are admitted in descending order as long as the mass kept before them is below the target, so T
-//   is the largest key for which the forced mass plus the mass of the keys >= T reaches the target; the search narrows an
-//   interval of keys and ends when one block is left in it (about 12 of the 32 bits).  The masses are fp64, as in the sort
-//   that select_kernel does.
+//   is the largest key for which the forced mass plus the mass of the keys >= T reaches the target.  The masses are fp64, as
+//   in select_kernel.
 template <int NPL>   // keys per lane: nkb <= 32 * NPL
 __device__ __forceinline__ void select_row(const SelectArgs& a, const float* s, int I, uint8_t* mask_row) {
     const int lane = threadIdx.x & 31;
@@ -411,11 +410,12 @@ __device__ __forceinline__ void select_row(const SelectArgs& a, const float* s, 
             }
         }
         all = warp_sum(all);
-        kept = warp_sum(kept) / all;
+        const double inv = 1.0 / all;
+        kept = warp_sum(kept) * inv;
 #pragma unroll
-        for (int q = 0; q < NPL; ++q) e[q] /= all;
+        for (int q = 0; q < NPL; ++q) e[q] *= inv;
         const double target = double(a.mass);
-        // mass kept by the blocks whose key reaches c (or passes it); a NaN anywhere reads as "target reached"
+        // mass kept once the blocks with keys >= c are in; comparisons are written so that a NaN reads as "target reached"
         auto mass_from = [&](uint32_t c) {
             double m = 0.0;
 #pragma unroll
@@ -423,36 +423,43 @@ __device__ __forceinline__ void select_row(const SelectArgs& a, const float* s, 
             return kept + warp_sum(m);
         };
         any = nfree > 0 && kept < target;
-        if (any && mass_from(1u) < target) {       // even all of them fall short: all are admitted
-            T = 1u; need_eq = nkb;
-        } else if (any) {
-            int inside = nfree;                    // blocks with keys in [T, T + 2^(bit+1))
+        if (any) {
+            // First on masses in units of 2^-30, whose warp sum is one instruction; the outcome is then checked in fp64.
+            const uint32_t T0 = T;
+            const uint32_t goal = uint32_t(fmax(1.0, ceil((target - kept) * 1073741824.0)));
+            uint32_t fine[NPL];
+#pragma unroll
+            for (int q = 0; q < NPL; ++q) fine[q] = uint32_t(e[q] * 1073741824.0 + 0.5);
 #pragma unroll 1
-            for (int bit = top; bit >= 0 && inside > 1; --bit) {
+            for (int bit = top; bit >= 0; --bit) {
                 const uint32_t cand = T | (1u << bit);
-                int c = 0;
+                uint32_t m = 0u;
 #pragma unroll
-                for (int q = 0; q < NPL; ++q) c += (key[q] >= cand && (key[q] - cand) >> bit == 0u) ? 1 : 0;
-                c = __reduce_add_sync(0xffffffffu, c);
-                if (!(mass_from(cand) < target)) { T = cand; inside = c; } else inside -= c;
+                for (int q = 0; q < NPL; ++q) m += key[q] >= cand ? fine[q] : 0u;
+                if (__reduce_add_sync(0xffffffffu, m) >= goal) T = cand;
             }
-            // the interval's last block (or its equal keys) is the one that reaches the target: T becomes its key
-            uint32_t low = 0xFFFFFFFFu;
-#pragma unroll
-            for (int q = 0; q < NPL; ++q) if (key[q] >= T && key[q] != 0u) low = min(low, key[q]);
-            T = __reduce_min_sync(0xffffffffu, low);
-            double over = 0.0, eq = 0.0;
-#pragma unroll
-            for (int q = 0; q < NPL; ++q) {
-                over += key[q] > T ? e[q] : 0.0;
-                eq = key[q] == T ? e[q] : eq;
+            double over = mass_from(T + 1u);
+            if (!(over < target) || mass_from(T) < target) {       // not so in fp64: the same search on the masses themselves
+                T = T0;
+                for (int bit = top; bit >= 0; --bit)
+                    if (!(mass_from(T | (1u << bit)) < target)) T |= 1u << bit;
+                over = mass_from(T + 1u);
             }
-            over = kept + warp_sum(over);
+            if (mass_from(T) < target) need_eq = nkb;              // even all of them fall short: all are admitted (T is below every key)
+            else {
+                // the blocks with the threshold's key are admitted one by one, as long as the mass before them is short
+                int ties = 0;
+                double p = 0.0;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) eq = fmax(eq, __shfl_xor_sync(0xffffffffu, eq, o));
-            need_eq = 0;
-            for (double run = over; run < target && need_eq < nfree && eq > 0.0; run += eq) ++need_eq;
-            if (eq == 0.0 && over < target) need_eq = nkb;
+                for (int q = 0; q < NPL; ++q) if (key[q] == T && key[q] != 0u) { ++ties; p = e[q]; }
+                ties = __reduce_add_sync(0xffffffffu, ties);
+                need_eq = 1;
+                if (ties > 1) {
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) p = fmax(p, __shfl_xor_sync(0xffffffffu, p, o));
+                    for (double run = over + p; run < target && need_eq < ties; run += p) ++need_eq;
+                }
+            }
         }
     }
     int seen = 0;
@@ -480,7 +487,7 @@ __global__ void __launch_bounds__(256) select_rows_kernel(SelectArgs a, int rows
 // row there.  The key-block means come 128 at a time, 64 elements of the head dimension per step, through two cp.async
 // buffers; rows of 68 floats keep the 16-byte reads free of bank conflicts.  What this saves against score_kernel and a
 // selection kernel is a launch and the scores' way through memory.  Whole calls, before and after: 12 heads, 61 blocks, top-k
-// 34.1 -> 21.9 us; 48 heads, 139 blocks, cumulative mass 209 -> 72 us (of which the sort of every row took 153).
+// 34.1 -> 20.6 us; 48 heads, 139 blocks, cumulative mass 209 -> 61 us (the sort of every row took 153).
 constexpr int kScoreKeys = 128, kScoreLd = 68;
 template <int D, int R>
 constexpr size_t score_select_smem(int nkb) {

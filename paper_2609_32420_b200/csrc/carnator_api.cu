@@ -143,10 +143,16 @@ carnator_status launch_score_select_d(const BuildWs& w, float* scores_opt, float
     return launch_score_select_r<D, 16, NPL>(w, scores_opt, scale, B, sa, stream);
 }
 carnator_status launch_score_select(const BuildWs& w, float* scores_opt, float scale, int B, int D, const SelectArgs& sa, int sms, cudaStream_t stream) {
-    if (sa.nkb <= 32 * 8) return D == 128 ? launch_score_select_d<128, 8>(w, scores_opt, scale, B, sa, sms, stream)
-                                          : launch_score_select_d<64, 8>(w, scores_opt, scale, B, sa, sms, stream);
-    return D == 128 ? launch_score_select_d<128, 32>(w, scores_opt, scale, B, sa, sms, stream)
-                    : launch_score_select_d<64, 32>(w, scores_opt, scale, B, sa, sms, stream);
+    // keys per lane: what a row needs costs instructions whether the row is that long or not
+#define CARNATOR_SCORE_SELECT(NPL) \
+    if (sa.nkb <= 32 * NPL) return D == 128 ? launch_score_select_d<128, NPL>(w, scores_opt, scale, B, sa, sms, stream) \
+                                            : launch_score_select_d<64, NPL>(w, scores_opt, scale, B, sa, sms, stream);
+    CARNATOR_SCORE_SELECT(5)
+    CARNATOR_SCORE_SELECT(8)
+    CARNATOR_SCORE_SELECT(20)
+    CARNATOR_SCORE_SELECT(32)
+#undef CARNATOR_SCORE_SELECT
+    return CARNATOR_ERR_UNSUPPORTED;
 }
 constexpr int kMaxKeyBlocksInRegisters = 32 * 32;     // a selecting warp holds its row's keys in registers
 
@@ -409,6 +415,7 @@ extern "C" carnator_status carnator_build_connectivity_exact(const void* Q, cons
     if (nkb <= kMaxKeyBlocksInRegisters) {
         const int rows = s->B * s->H * nqb;
         if (nkb <= 32 * 8) select_rows_kernel<8><<<ceil_div(rows, 8), 256, 0, stream>>>(sa, rows);
+        else if (nkb <= 32 * 20) select_rows_kernel<20><<<ceil_div(rows, 8), 256, 0, stream>>>(sa, rows);
         else select_rows_kernel<32><<<ceil_div(rows, 8), 256, 0, stream>>>(sa, rows);
     } else {
         const size_t smem = size_t(sa.npad) * 8 * 2 + ((nkb + 15) & ~15);

@@ -166,12 +166,13 @@ def test_full_size_masks_on_sampled_heads(name, keep):
     assert n_excused <= 8
 
 
-# One kernel scores and selects for up to 1024 key blocks (a warp holds 8 or 32 keys a lane), two take more: the edges of those
+# One kernel scores and selects for up to 1024 key blocks (a warp holds 5, 8, 20 or 32 keys a lane), two take more: the edges of those
 # ranges, ragged last blocks and query tiles, both CTA sizes (8 and 16 rows), unequal block sizes.
 @pytest.mark.parametrize("mode", [wl.MODE_TOPK, wl.MODE_CUMMASS], ids=["topk", "mass"])
 @pytest.mark.parametrize("B,H,N,n_text,D,bq,bk,window", [
     (1, 1, 50, 0, 128, 64, 64, -1), (1, 1, 64 * 31 + 1, 7, 64, 128, 64, -1), (2, 3, 64 * 33, 0, 128, 64, 64, 0),
-    (1, 48, 64 * 129 - 1, 100, 64, 64, 64, 1), (1, 2, 64 * 256, 0, 64, 128, 64, -1), (1, 1, 64 * 257, 0, 128, 128, 64, 1),
+    (1, 48, 64 * 129 - 1, 100, 64, 64, 64, 1), (1, 2, 64 * 256, 0, 64, 128, 64, -1), (1, 2, 64 * 160, 0, 64, 128, 64, -1), (1, 1, 64 * 161, 9, 64, 128, 64, 0),
+    (1, 1, 64 * 640 - 3, 0, 128, 128, 64, 1), (1, 1, 64 * 257, 0, 128, 128, 64, 1),
     (1, 1, 64 * 1024, 0, 64, 128, 64, -1), (1, 1, 64 * 1024 + 1, 0, 64, 128, 64, 0), (1, 2, 128 * 40 + 5, 0, 128, 128, 128, 2)])
 def test_score_and_selection_at_the_edges_of_their_ranges(B, H, N, n_text, D, bq, bk, window, mode):
     rng = np.random.default_rng(N + D + mode)
