@@ -391,6 +391,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int b = blockIdx.z, h = blockIdx.y;
     const int64_t bh = int64_t(b) * a.H + h;
+    grid_wait();                            // launched while the compaction drains
     constexpr bool kPairs = BQ == 64, kPlanned = BQ == 64 || BK == 64;
     constexpr int kPerStep = kBlock / BK;             // listed key blocks in a step
     const int x0 = kPairs ? 2 * blockIdx.x : blockIdx.x;
@@ -1001,8 +1002,7 @@ inline carnator_status launch_tc(const AttnArgs& a, const CUtensorMap& mk, const
         return CARNATOR_ERR_UNSUPPORTED;
     }
     dim3 grid(BQ == 64 ? ceil_div(a.nqb, 2) : a.nqb, a.H, a.B);
-    kern<<<grid, tc::kThreads, smem, stream>>>(mk, mv, a);
-    e = cudaGetLastError();
+    e = launch_dependent(kern, grid, dim3(tc::kThreads), smem, stream, mk, mv, a);
     if (e != cudaSuccess) { snprintf(err, errlen, "attn_tcgen05_kernel: %s", cudaGetErrorString(e)); return CARNATOR_ERR_CUDA; }
     return CARNATOR_OK;
 }

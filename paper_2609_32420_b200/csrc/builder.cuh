@@ -27,10 +27,6 @@ __device__ __forceinline__ uint4 ld_stream16(const void* p) {
     return v;
 }
 
-// Programmatic dependent launch: the next kernel of a call starts while this one drains, and waits here for its results.
-__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 // A CTA takes 32 KB of consecutive tokens, one block at D = 128 and two at D = 64, with all eight 16-byte loads of a thread
 // in flight at once (with four loads, and 16 KB per CTA at D = 64, 218 MB took 46 us).
 // The first CTA clears the workspace header for the kernels behind it.

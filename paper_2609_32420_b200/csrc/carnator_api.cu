@@ -113,19 +113,6 @@ carnator_status allow_smem(K kernel, size_t bytes) {
     return CARNATOR_OK;
 }
 
-// Launch that may begin before the kernel ahead of it in the stream has ended (that kernel calls grid_launch_dependents,
-// this one grid_wait before it reads anything of it).
-template <typename... P, typename... A>
-cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A... args) {
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = stream;
-    cfg.attrs = at; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
-}
-
 template <int D, int R, int NPL>
 carnator_status launch_score_select_r(const BuildWs& w, float* scores_opt, float scale, int B, const SelectArgs& sa, cudaStream_t stream) {
     const size_t smem = score_select_smem<D, R>(sa.nkb);
@@ -458,14 +445,28 @@ static carnator_status compact_impl(const uint8_t* mask, const uint8_t* recomput
     if (st != CARNATOR_OK) return st;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     const int nqb = ceil_div(s->N, s->block_q), nkb = ceil_div(s->N, s->block_k);
-    if (nqb > 12000) return CARNATOR_ERR_UNSUPPORTED;   // order kernel keeps one head's counts in shared memory
-    CUDA_TRY(cudaMemsetAsync(w.hdr, 0, sizeof(WsHeader), stream));
-    const int rows = s->B * s->H * nqb;
-    compact_rows_kernel<<<ceil_div(rows, 8), 256, 0, stream>>>(mask, recompute_rows, s->B, s->H, nqb, nkb, w.counts, w.lists,
-                                                               active_q, context_k);
-    LAUNCH_CHECK("compact_rows_kernel");
-    order_rows_kernel<<<s->B * s->H, 256, size_t(nqb) * 4, stream>>>(w.counts, nqb, w.order, w.hdr);
-    LAUNCH_CHECK("order_rows_kernel");
+    if (nqb > kMaxQueryBlocks) return CARNATOR_ERR_UNSUPPORTED;
+    CompactArgs ca;
+    ca.mask = mask; ca.recompute = recompute_rows; ca.active_q = active_q; ca.context_k = context_k;
+    ca.counts = w.counts; ca.lists = w.lists; ca.order = w.order; ca.hdr = w.hdr;
+    ca.H = s->H; ca.nqb = nqb; ca.nkb = nkb;
+    ca.ctas = 1;
+    while (ca.ctas < 8 && int64_t(nqb) * nkb > int64_t(kCompactPairsPerCta) * ca.ctas) ca.ctas *= 2;
+    const bool pairs = s->block_q == 64;
+    const size_t smem = compact_smem(nqb, pairs);
+    auto kern = pairs ? compact_order_kernel<true> : compact_order_kernel<false>;
+    if (smem > 48 * 1024) {
+        st = allow_smem(kern, smem);
+        if (st != CARNATOR_OK) return st;
+    }
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = unsigned(ca.ctas); at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(unsigned(s->B) * s->H * ca.ctas); cfg.blockDim = dim3(kCompactThreads);
+    cfg.dynamicSmemBytes = smem; cfg.stream = stream; cfg.attrs = at; cfg.numAttrs = 1;
+    CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, ca));
+    g_launches.fetch_add(1, std::memory_order_relaxed);
     return CARNATOR_OK;
 }
 
@@ -550,6 +551,8 @@ extern "C" carnator_status carnator_compacted_tiles(const carnator_shape* s, con
     st = attn_ws_check(s, const_cast<void*>(ws), ws_bytes, &w);
     if (st != CARNATOR_OK) return st;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
+    count_tiles_kernel<<<1, 1024, 0, stream>>>(w.counts, int64_t(s->B) * s->H * ceil_div(s->N, s->block_q), w.hdr);
+    LAUNCH_CHECK("count_tiles_kernel");
     WsHeader h;
     CUDA_TRY(cudaMemcpyAsync(&h, w.hdr, sizeof(WsHeader), cudaMemcpyDeviceToHost, stream));
     CUDA_TRY(cudaStreamSynchronize(stream));

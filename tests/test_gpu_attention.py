@@ -388,3 +388,42 @@ def test_query_blocks_that_share_a_tile_do_not_see_each_others_keys(bk):
     assert bool((O1[0, 0, 6 * bq:7 * bq] == 3.0).all()) and bool((L1[0, 0, 6 * bq:7 * bq] == -7.0).all())
     ok = torch.isfinite(O0)
     assert float((O0[ok] - O1[ok]).abs().max()) <= 2e-2
+
+
+@pytest.mark.parametrize("bq,bk,N,H", [(128, 128, 128 * 3, 5), (128, 128, 128 * 129, 2), (128, 64, 64 * 400 + 3, 1), (64, 64, 64, 1),
+                                       (64, 64, 64 * 301, 2), (64, 128, 64 * 513, 1)])
+def test_compacted_lists_and_order(bq, bk, N, H):
+    """Lists, counts and order for one CTA per head up to a cluster of eight: every row's list is its mask, the order is a
+    permutation, longest list first (128-token query blocks), or pairs of like rows, longest pair first, the odd row last."""
+    rng = np.random.default_rng(N + bq)
+    B, D = 2, 64
+    nqb, nkb = -(-N // bq), -(-N // bk)
+    mask = (rng.random((B, H, nqb, nkb)) < rng.random((B, H, nqb, 1))).astype(np.uint8)
+    rec = (rng.random((B, nqb)) < 0.1).astype(np.uint8)
+    mask[:, :, nqb // 2] = 0
+    rec[:, nqb // 2] = 0
+    shape = cn.make_shape(B, H, N, D, 0, 1, 1, N, bq, bk)
+    ws = torch.full((cn.attn_workspace_bytes(shape),), 0xAB, dtype=torch.uint8, device="cuda")
+    cn.compact_mask(torch.from_numpy(mask).cuda(), torch.from_numpy(rec).cuda(), shape, ws=ws)
+    eff = (mask != 0) | (rec != 0)[:, None, :, None]
+    assert cn.query_status(ws) == cn.OK and cn.compacted_tiles(shape, ws) == int(eff.sum())
+    rows = B * H * nqb
+    al = lambda x: (x + 255) // 256 * 256
+    w = ws.cpu().numpy()
+    counts, order = (w[256 + k * al(rows * 4):][:rows * 4].view(np.int32).reshape(B * H, nqb) for k in range(2))
+    lists = w[256 + 2 * al(rows * 4):][:rows * nkb * 4].view(np.int32).reshape(B * H, nqb, nkb)
+    np.testing.assert_array_equal(counts, eff.sum(-1).reshape(B * H, nqb))
+    for bh in range(B * H):
+        for I in range(nqb):
+            np.testing.assert_array_equal(lists[bh, I, :counts[bh, I]], np.flatnonzero(eff.reshape(B * H, nqb, nkb)[bh, I]))
+        c, o = counts[bh], order[bh]
+        assert sorted(o.tolist()) == list(range(nqb))
+        if bq == 128:
+            np.testing.assert_array_equal(o, np.argsort(-c, kind="stable"))
+            continue
+        kind = np.where(c == nkb, 0, np.where(c > 0, 1, 2))
+        seq = np.lexsort((np.arange(nqb), kind))
+        pairs = {tuple(seq[i:i + 2]) for i in range(0, nqb, 2)}
+        assert {tuple(o[i:i + 2]) for i in range(0, nqb, 2)} == pairs
+        longest = [c[o[i:i + 2]].max() for i in range(0, nqb - 1, 2)]
+        assert longest == sorted(longest, reverse=True)
