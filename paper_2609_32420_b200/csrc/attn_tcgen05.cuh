@@ -8,22 +8,23 @@
 //   warps 0-3  softmax group 0, warps 4-7 softmax group 1: the groups take the 128-key steps in turn; within
 //              a group warp w owns tensor-memory lanes 32w..32w+31 = query rows.  Both also run the epilogue.
 //   warp 8     TMA producer for the K tiles (one lane)
-//   warp 9     tensor-memory allocation, issue of every matrix product (the warp stays converged, an elected lane issues)
+//   warp 9     tensor-memory allocation, issue of Q K^T
 //   warp 10    TMA producer for the V tiles (one lane)
-//   warp 11    idle
+//   warp 11    issue of P V
 // The third warpgroup gives most of its registers to the softmax groups (setmaxnreg), which hold a full
 // 128-column score row per thread.
-// One warp issues all the matrix products: two threads issuing at once each ran at half the rate, and the
-// pipe then executes in a known order.  The warp runs its loop converged and elects the issuing lane per instruction
-// (elect.sync) instead of sending one lane into a branch: the descriptors then live in uniform registers and a batch
-// takes a third fewer cycles to queue while the softmax warps on the same scheduler are busy.  Each batch ends in
+// The two issuing warps run their loops converged and elect the issuing lane per instruction (elect.sync) instead of
+// sending one lane into a branch: the descriptors then live in uniform registers and a batch
+// takes a third fewer cycles to queue while the softmax warps on the same scheduler are busy.  Each waits for its own
+// operands and nothing else; one warp that polled for both kinds of product took 1 to 3 % longer (Wan-14B-shaped layer
+// 24.7 against 24.4 ms, five-frame clip 416 against 396 us, 64-token blocks 2.48 against 2.39 ms).  Each batch ends in
 // one tcgen05.commit (a commit costs the issuer about as much as two MMAs): "S_g full" also releases the K slot,
 // "P V done" also releases the V slot and the P buffer.
 // Tensor memory (512 columns): S0 | S1 (128 fp32 columns each, one per softmax group), P (64 columns of packed
 // bf16), Q (D / 2 columns of packed bf16), O (D fp32 columns).  The query tile is written there once by the
 // softmax groups (straight from global memory) and serves as the A operand of every Q K^T, so those products
 // read only the K tile from shared memory, whose bandwidth the TMA writes and the operand reads share.  A group
-// signals as soon as it has pulled its scores into registers, so Q K^T of its next step runs underneath its own
+// signals when it no longer needs its scores in tensor memory, so Q K^T of its next step runs underneath its own
 // exponentials; it keeps its probabilities in registers until they are complete and stores them in one go, by
 // which time P V of the previous step has long read the one P buffer.  P V is issued in step order.
 // Every wait on an mbarrier is bounded; on expiry the role records CARNATOR_ERR_DEVICE_TIMEOUT in
@@ -42,7 +43,7 @@ constexpr int kSBufs = 2;              // score buffers in tensor memory, one pe
 constexpr int kRefSlots = 3;           // hand-over slots of the shared reference maximum
 constexpr int kStages = 3;             // ring slots for K tiles and for V tiles
 constexpr int kSoftmaxWarps = 8;       // two warpgroups taking the steps in turn
-constexpr int kThreads = (kSoftmaxWarps + 4) * 32;   // third warpgroup: two TMA producers, the MMA issuer, one idle warp
+constexpr int kThreads = (kSoftmaxWarps + 4) * 32;   // third warpgroup: two TMA producers, two MMA issuers
 constexpr int kWarpTmaK = 8, kWarpMma = 9, kWarpTmaV = 10;
 constexpr int kTmemCols = 512;         // S0 | S1 | P | Q | O
 constexpr uint32_t kColP = 2 * kBlock;        // packed bf16 probabilities: 64 columns, one buffer for both groups
@@ -215,6 +216,16 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
         : "r"(taddr) : "memory");
 #pragma unroll
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr) : "memory");
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 __device__ __forceinline__ float ex2_approx(float x) {
     float y;
@@ -455,7 +466,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
     const uint32_t sK = smem_base + C::kOffK;
     const uint32_t sV = smem_base + C::kOffV;
     const uint32_t bars = smem_base + C::kOffBar;
-    const uint32_t bar_q = bars, bar_o = bars + 8, bar_drain = bars + 16;
+    const uint32_t bar_q = bars, bar_o = bars + 8, bar_drain = bars + 16, bar_drain2 = bars + 24;
     auto bar_kfull = [&](int s) { return bars + 32 + 8 * s; };       // up to 4 stages each
     auto bar_vfull = [&](int s) { return bars + 96 + 8 * s; };
     auto bar_sfull = [&](int s) { return bars + 160 + 8 * s; };      // S_g holds fresh scores
@@ -464,18 +475,20 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
     auto bar_ref = [&](int s, int q) { return bars + 224 + 8 * (s * 4 + q); };   // r_pub slot s, lane quarter q
     auto bar_fin = [&](int q) { return bars + 320 + 8 * q; };
     auto bar_pvdone = [&](int s) { return bars + 352 + 8 * s; };     // P V of the step that used score buffer s has completed
+    auto bar_pva = [&](int s) { return bars + 368 + 8 * s; };
+    auto bar_pfullb = [&](int s) { return bars + 384 + 8 * s; };
     volatile int* abortp = &abort_flag;
     // every bounded wait of this CTA gives up after `limit` (2 s unless the workspace header asks for less)
     const unsigned long long limit = a.hdr->wait_limit_ns ? a.hdr->wait_limit_ns : kDefaultWaitNs;
 
     if (tid == 0) {
         abort_flag = 0;
-        mbar_init(bar_q, kSoftmaxWarps); mbar_init(bar_o, 1); mbar_init(bar_drain, 1);
+        mbar_init(bar_q, kSoftmaxWarps); mbar_init(bar_o, 1); mbar_init(bar_drain, 1); mbar_init(bar_drain2, 1);
         for (int s = 0; s < kStages; ++s) {
             mbar_init(bar_kfull(s), 1); mbar_init(bar_vfull(s), 1);
         }
         for (int s = 0; s < kSBufs; ++s) {
-            mbar_init(bar_sfull(s), 1); mbar_init(bar_pvdone(s), 1);
+            mbar_init(bar_sfull(s), 1); mbar_init(bar_pvdone(s), 1); mbar_init(bar_pva(s), 1); mbar_init(bar_pfullb(s), 4);
             mbar_init(bar_pfull(s), 4); mbar_init(bar_sfree(s), 4);          // one arrival per softmax warp of the group
         }
         for (int s = 0; s < kRefSlots; ++s)
@@ -557,93 +570,71 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
             }
         }
     } else if (warp == kWarpMma) {
-        // ================= MMA issuer =================
-        // One thread queues every matrix product and serves whichever is ready: Q K^T of the next step (its K tile
-        // has landed and the softmax group has taken the previous scores out of that S buffer) or P V of the oldest
-        // step whose probabilities are complete.  One commit per batch: the barrier that says "S_g is full" also
-        // frees the K slot, and the one that says "P V done" also frees the V slot and P_g.
-        // The whole warp runs this loop converged (every decision is a warp vote), and one elected lane issues.
-        {
-            constexpr uint32_t idesc_qk = instr_desc(kBlock, kBlock, 0);
-            constexpr uint32_t idesc_pv = instr_desc(kBlock, D, 1);
-            // descriptor words that do not change: low word = (address >> 4) | leading offset; high word = stride
-            // offset | version | swizzle mode (see smem_desc)
-            const uint64_t dk = smem_desc(sK, 16, 1024), dv = smem_desc(sV, C::kBoxBytes, 1024);
-            const uint32_t k_lo0 = uint32_t(dk), hi_kmajor = uint32_t(dk >> 32);
-            const uint32_t v_lo0 = uint32_t(dv), hi_v = uint32_t(dv >> 32);
-            bool ok = mbar_wait_warp(bar_q, 0, abortp, 0, limit);   // the softmax groups have put the query tile into tensor memory
-            if (!ok && lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 3, 0, blockIdx.x);
+        // ================= issuer of Q K^T =================
+        // S_g = Q K_i^T once the K tile has landed and the softmax group has taken the previous scores out of that S buffer.
+        // The whole warp runs the loop converged and one elected lane issues.  The barrier a batch commits ("S_g is full")
+        // also frees the K slot.
+        constexpr uint32_t idesc_qk = instr_desc(kBlock, kBlock, 0);
+        // descriptor words that do not change: low word = (address >> 4) | leading offset; high word = stride
+        // offset | version | swizzle mode (see smem_desc)
+        const uint64_t dk = smem_desc(sK, 16, 1024);
+        const uint32_t k_lo0 = uint32_t(dk), hi_kmajor = uint32_t(dk >> 32);
+        bool ok = mbar_wait_warp(bar_q, 0, abortp, 0, limit);   // the softmax groups have put the query tile into tensor memory
+        if (!ok && lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 3, 0, blockIdx.x);
+        tc_fence_after();
+        for (int iq = 0; iq < T && ok; ++iq) {
+            const int s = iq % kStages, g = iq & 1;
+            ok = mbar_wait_warp(bar_kfull(s), uint32_t(iq / kStages) & 1u, abortp, 0, limit);
+            if (ok && iq >= 2) ok = mbar_wait_warp(bar_sfree(g), uint32_t((iq - 2) >> 1) & 1u, abortp, 0, limit);
+            if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 4, iq, blockIdx.x); break; }
             tc_fence_after();
-            int iq = 0, ip = 0;                          // next Q K^T step, next P V step
-            unsigned long long t_idle = 0;               // lane 0's clock decides about giving up
-            uint32_t idle = 0;
-            while (ip < T && ok) {
-                bool progress = false;
-                if (ip < iq) {
-                    const int s = ip % kStages, g = ip & 1;
-                    const bool ready = mbar_test(bar_pfull(g), uint32_t(ip >> 1) & 1u) && mbar_test(bar_vfull(s), uint32_t(ip / kStages) & 1u);
-                    if (__all_sync(0xffffffffu, ready)) {
-                        // O += P_i V_i : P from tensor memory (16 keys = 8 packed columns per instruction), V tile as the
-                        // MN-major B operand (rows = keys, 64-element chunks of the head dimension one box apart)
-                        tc_fence_after();
-                        const uint32_t v_lo = v_lo0 + uint32_t(s) * (C::kTileBytes >> 4), p_t = tmem + kColP, d_o = tmem + kColO;
-                        const uint32_t acc0 = ip > 0 ? 1u : 0u;
+            // Q from tensor memory, K tile K-major, 16 elements of the head dimension per instruction
+            const uint32_t k_lo = k_lo0 + uint32_t(s) * (C::kTileBytes >> 4), d_s = tmem + g * kBlock;
 #pragma unroll
-                        for (int kk = 0; kk < kBlock / 16; ++kk) {
-                            if (kPairs) {       // O starts at zero; rows that do not list the block keep what they have
-                                const uint32_t e = plan[ip * kPerStep + kk / (BK / 16)] >> kPlanRowBit;
-                                mma_ts_el_rows(d_o, p_t + kk * 8, v_lo + kk * (2048 >> 4), hi_v, idesc_pv, (e & 1u) - 1u, (e >> 1) - 1u, 1u);
-                            } else {
-                                mma_ts_el(d_o, p_t + kk * 8, v_lo + kk * (2048 >> 4), hi_v, idesc_pv, kk > 0 ? 1u : acc0);
-                            }
-                        }
-                        tc_commit_el(bar_pvdone(g));
-                        ++ip; progress = true;
-                    }
-                }
-                if (iq < T) {
-                    const int s = iq % kStages, g = iq & 1;
-                    const bool ready = mbar_test(bar_kfull(s), uint32_t(iq / kStages) & 1u) &&
-                                       (iq < 2 || mbar_test(bar_sfree(g), uint32_t((iq - 2) >> 1) & 1u));
-                    if (__all_sync(0xffffffffu, ready)) {
-                        // S_g = Q K_i^T: Q from tensor memory, K tile K-major, 16 elements of the head dimension per instruction
-                        tc_fence_after();
-                        const uint32_t k_lo = k_lo0 + uint32_t(s) * (C::kTileBytes >> 4), d_s = tmem + g * kBlock;
+            for (int kk = 0; kk < D / 16; ++kk) {
+                const uint32_t off16 = ((kk / 4) * C::kBoxBytes + (kk % 4) * 32) >> 4;      // compile-time constant
+                mma_ts_el(d_s, tmem + kColQ + kk * 8, k_lo + off16, hi_kmajor, idesc_qk, kk > 0 ? 1u : 0u);
+            }
+            tc_commit_el(bar_sfull(g));
+        }
+        if (__any_sync(0xffffffffu, *abortp != 0)) {      // no product may still run when tensor memory is released
+            tc_commit_el(bar_drain);
+            mbar_wait_drain(bar_drain, 0, limit);
+            __syncwarp();
+        }
+    } else {
+        // ================= issuer of P V (warp 11) =================
+        // O += P_i V_i once the V tile has landed and the probabilities are complete; "P V done" also frees the V slot and P.
+        constexpr uint32_t idesc_pv = instr_desc(kBlock, D, 1);
+        const uint64_t dv = smem_desc(sV, C::kBoxBytes, 1024);
+        const uint32_t v_lo0 = uint32_t(dv), hi_v = uint32_t(dv >> 32);
+        bool ok = true;
+        for (int ip = 0; ip < T && ok; ++ip) {
+            const int s = ip % kStages, g = ip & 1;
+            ok = mbar_wait_warp(bar_vfull(s), uint32_t(ip / kStages) & 1u, abortp, 0, limit);
+            if (ok) ok = mbar_wait_warp(bar_pfull(g), uint32_t(ip >> 1) & 1u, abortp, 0, limit);
+            if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 5, ip, blockIdx.x); break; }
+            tc_fence_after();
+            // P from tensor memory (16 keys = 8 packed columns per instruction), V tile as the MN-major B operand
+            // (rows = keys, 64-element chunks of the head dimension one box apart)
+            const uint32_t v_lo = v_lo0 + uint32_t(s) * (C::kTileBytes >> 4), p_t = tmem + kColP, d_o = tmem + kColO;
+            const uint32_t acc0 = ip > 0 ? 1u : 0u;
 #pragma unroll
-                        for (int kk = 0; kk < D / 16; ++kk) {
-                            const uint32_t off16 = ((kk / 4) * C::kBoxBytes + (kk % 4) * 32) >> 4;      // compile-time constant
-                            mma_ts_el(d_s, tmem + kColQ + kk * 8, k_lo + off16, hi_kmajor, idesc_qk, kk > 0 ? 1u : 0u);
-                        }
-                        tc_commit_el(bar_sfull(g));
-                        ++iq; progress = true;
-                    }
-                }
-                if (progress) { idle = 0; continue; }
-                __nanosleep(20);                        // keep the polling from taking issue slots from the softmax warps on this scheduler
-                if ((++idle & 1023u) == 0) {             // nothing was ready: bounded, like every other wait
-                    int give_up = 0;
-                    if (lane == 0) {
-                        if (*abortp) give_up = 1;
-                        else {
-                            const unsigned long long now = global_ns();
-                            if (idle == 1024u) t_idle = now;
-                            else if (now - t_idle > limit) give_up = 2;
-                        }
-                    }
-                    give_up = __shfl_sync(0xffffffffu, give_up, 0);
-                    if (give_up) {
-                        if (give_up == 2 && lane == 0) { set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 4, ip, blockIdx.x); *abortp = 1; }
-                        ok = false;
-                        break;
-                    }
+            for (int kk = 0; kk < kBlock / 16; ++kk) {
+                if (kPairs) {       // O starts at zero; rows that do not list the block keep what they have
+                    const uint32_t e = plan[ip * kPerStep + kk / (BK / 16)] >> kPlanRowBit;
+                    mma_ts_el_rows(d_o, p_t + kk * 8, v_lo + kk * (2048 >> 4), hi_v, idesc_pv, (e & 1u) - 1u, (e >> 1) - 1u, 1u);
+                } else {
+                    mma_ts_el(d_o, p_t + kk * 8, v_lo + kk * (2048 >> 4), hi_v, idesc_pv, kk > 0 ? 1u : acc0);
                 }
             }
-            if (ok) tc_commit_el(bar_o);
-            if (__any_sync(0xffffffffu, *abortp != 0)) {      // make sure no MMA of this warp is still running before tensor memory is released
-                tc_commit_el(bar_drain);
-                mbar_wait_drain(bar_drain, 0, limit);
-                __syncwarp();
-            }
+            tc_commit_el(bar_pvdone(g));
+        }
+        if (ok) tc_commit_el(bar_o);
+        if (__any_sync(0xffffffffu, *abortp != 0)) {
+            tc_commit_el(bar_drain2);
+            mbar_wait_drain(bar_drain2, 0, limit);
+            __syncwarp();
         }
     }
     } else {
@@ -703,7 +694,6 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
             nvalid_last = ((n_listed - 1) % kPerStep) * BK + left;
         }
         for (int i = wg; i < T; i += 2) {
-            const int rs = i % kRefSlots;
             const uint32_t sph = uint32_t(i >> 1) & 1u;
             ok = mbar_wait_warp(bar_sfull(wg), sph, abortp, 20, limit);   // warp-uniform: the loads below are collective
             if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 7, i, blockIdx.x); break; }
@@ -712,97 +702,187 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
             const uint32_t tS = tmem + lane_base + wg * kBlock;
             const uint32_t tP = tmem + lane_base + kColP;
             float s[4][32];
+            uint32_t pk[4][16];
+            uint64_t part2[2];
+            bool p_free;
+            if constexpr (!kPlanned) {
+                // The first half of the exponentials is taken under the reference of step i-1 while the row maximum is still
+                // being found (they use different pipes), and again in the rare step that moves the reference, from the scores
+                // in tensor memory, which are given up only then.  With the maximum in front of all exponentials instead
+                // (below; the 64-token forms are 4 % faster that way) the Wan-14B-shaped layer takes 24.4 ms against 24.2,
+                // the CogVideoX-shaped one 2.77 against 2.72.  A loop around one copy of the first half, instead of two
+                // copies, took 25.0 and 3.2 ms.
 #pragma unroll
-            for (int c = 0; c < 4; ++c) tmem_ld32(tS + c * 32, s[c]);
-            tmem_wait_ld();
-            tc_fence_before();
-            mbar_arrive_warp(bar_sfree(wg));     // the scores are in registers: S_g may take the scores of step i+2
-            if (nvalid < kBlock) {               // ragged tail (warp-uniform): keys >= N never count
+                for (int c = 0; c < 4; ++c) tmem_ld32(tS + c * 32, s[c]);
+                tmem_wait_ld();
+                auto mask_half = [&](int c0) {       // ragged tail (warp-uniform): keys >= N never count
+                    if (nvalid < kBlock) {
+#pragma unroll
+                        for (int c = c0; c < c0 + 2; ++c)
+#pragma unroll
+                            for (int e = 0; e < 32; ++e)
+                                if (c * 32 + e >= nvalid) s[c][e] = -INFINITY;
+                    }
+                };
+                mask_half(0); mask_half(2);
+                float r_now = -INFINITY;
+                if (i > 0) {                         // reference handed over from step i-1
+                    ok = mbar_wait_warp(bar_ref((i - 1) % kRefSlots, quarter), uint32_t((i - 1) / kRefSlots) & 1u, abortp, 0, limit);
+                    if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 10, i, blockIdx.x); break; }
+                    r_now = r_pub[(i - 1) % kRefSlots][r_loc];
+                }
+                const uint64_t scale2 = pack2(a.scale_log2, a.scale_log2);
+                part2[0] = part2[1] = pack2(0.f, 0.f);
+                // P = exp2(s * scale - R_i): one FFMA + one MUFU per element, packed bf16 pairs
+                auto exps = [&](int c0, float r) {
+                    const uint64_t neg_m2 = pack2(-r, -r);
+#pragma unroll
+                    for (int c = c0; c < c0 + 2; ++c)
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) {
+                            float x0, x1;
+                            unpack2(fma2(pack2(s[c][2 * e], s[c][2 * e + 1]), scale2, neg_m2), x0, x1);
+                            const float p0 = ex2_approx(x0), p1 = ex2_approx(x1);
+                            part2[e & 1] = add2(part2[e & 1], pack2(p0, p1));
+                            pk[c][e] = pack_bf16(p0, p1);
+                        }
+                };
+                // row maximum of the raw scores (the scale is positive), four independent chains
+                float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
 #pragma unroll
-                    for (int e = 0; e < 32; ++e)
-                        if (c * 32 + e >= nvalid) s[c][e] = -INFINITY;
-            }
-            // 64-token blocks: the halves of the step that this warp's rows list (a pad entry is listed by nobody)
-            bool on0 = true, on1 = true;
-            if (kPlanned) {
-                const int bit = kPlanRowBit + (second ? 1 : 0);
-                on0 = (plan[i * kPerStep] >> bit) & 1;
-                on1 = (plan[i * kPerStep + kPerStep - 1] >> bit) & 1;
-                if (!on0) {
+                    for (int e = 0; e < 32; e += 2) mx4[(e >> 1) & 3] = max3(mx4[(e >> 1) & 3], s[c][e], s[c][e + 1]);
+                const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * a.scale_log2;
+                exps(0, r_now);
+                const bool grow = i == 0 || mx > r_now + kRescaleThreshold;
+                p_free = i < 1;
+                if (__any_sync(0xffffffffu, grow)) {
+                    const float r_prev = r_now;
+                    r_now = grow ? mx : r_now;
+                    if (i > 0) {
+                        // O must be quiescent: P V of step i-1 (the other group's) complete.  P V is issued in step order
+                        // and that of step i cannot start before this group delivers P_i.
+                        p_free = true;
+                        ok = mbar_wait_warp(bar_pvdone(wg ^ 1), uint32_t((i - 1) >> 1) & 1u, abortp, 0, limit);
+                        if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 9, i, blockIdx.x); break; }
+                        tc_fence_after();
+                        const float f = ex2_approx(r_prev - r_now);          // 1 for rows that did not move
+#pragma unroll 1
+                        for (int c = 0; c < D / 16; ++c) {
+                            float o[16];
+                            tmem_ld16(tmem + lane_base + kColO + c * 16, o);
+                            tmem_wait_ld();
+                            uint32_t r[16];
 #pragma unroll
-                    for (int e = 0; e < 64; ++e) s[e >> 5][e & 31] = -INFINITY;
-                }
-                if (!on1) {
-#pragma unroll
-                    for (int e = 64; e < 128; ++e) s[e >> 5][e & 31] = -INFINITY;
-                }
-            }
-            // row maximum of the raw scores (the scale is positive), four independent chains
-            float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-#pragma unroll
-                for (int e = 0; e < 32; e += 2) mx4[(e >> 1) & 3] = max3(mx4[(e >> 1) & 3], s[c][e], s[c][e + 1]);
-            const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * a.scale_log2;
-            // reference handed over from step i-1
-            float r_prev = -INFINITY, r_now = mx;
-            bool grow = false;
-            if (i > 0) {
-                ok = mbar_wait_warp(bar_ref((i - 1) % kRefSlots, quarter), uint32_t((i - 1) / kRefSlots) & 1u, abortp, 0, limit);
-                if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 10, i, blockIdx.x); break; }
-                r_prev = r_pub[(i - 1) % kRefSlots][r_loc];
-                grow = mx > r_prev + kRescaleThreshold;
-                r_now = grow ? mx : r_prev;
-            }
-            r_pub[rs][r_loc] = r_now;
-            mbar_arrive_warp(bar_ref(rs, quarter));
-            // The one P buffer is free again once P V of step i-1 (the other group's) has read it.  The probabilities
-            // are kept in registers until they are all there, so that wait comes after the exponentials; the rescaling
-            // path needs the same product to be complete (O quiescent) and takes the wait early.  Each step waits on
-            // the phase that follows the one it waited on two steps earlier, so the phase is never ambiguous.
-            bool p_free = i < 1;
-            if (i > 0 && __any_sync(0xffffffffu, grow)) {
-                p_free = true;
-                // O must be quiescent: P V of step i-1 (the other group's) complete.  P V is issued in step order
-                // and that of step i cannot start before this group delivers P_i.
-                ok = mbar_wait_warp(bar_pvdone(wg ^ 1), uint32_t((i - 1) >> 1) & 1u, abortp, 0, limit);
-                if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 9, i, blockIdx.x); break; }
-                tc_fence_after();
-                // 1 for rows that did not move (rows of a pair may both times be at -inf: nothing listed so far)
-                const float f = !kPairs || grow ? ex2_approx(r_prev - r_now) : 1.f;
-#pragma unroll
-                for (int c = 0; c < D / 32; ++c) {
-                    float o[32];
-                    tmem_ld32(tmem + lane_base + kColO + c * 32, o);
+                            for (int e = 0; e < 16; ++e) r[e] = __float_as_uint(o[e] * f);
+                            tmem_st16(tmem + lane_base + kColO + c * 16, r);
+                        }
+                    }
+                    tmem_ld32(tS, s[0]); tmem_ld32(tS + 32, s[1]);
                     tmem_wait_ld();
-                    uint32_t r[32];
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(o[e] * f);
-                    tmem_st32(tmem + lane_base + kColO + c * 32, r);
+                    mask_half(0);
+                    part2[0] = part2[1] = pack2(0.f, 0.f);
+                    exps(0, r_now);
                 }
-            }
-            if (m_w != r_now) { l_w *= ex2_approx(m_w - r_now); m_w = r_now; }   // first use: l_w = 0, exp2(-inf) = 0
-            // P = exp2(s * scale - R_i): one FFMA + one MUFU per element, packed bf16 pairs over S's own columns
-            const uint64_t neg_m2 = pack2(-r_now, -r_now), scale2 = pack2(a.scale_log2, a.scale_log2);
-            uint64_t part2[2] = {pack2(0.f, 0.f), pack2(0.f, 0.f)};
-            uint32_t pk[4][16];
-            if (kPairs && !on0 && !on1) {        // warp-uniform: nothing of this step belongs to these rows (their reference may be -inf)
-#pragma unroll
-                for (int e = 0; e < 64; ++e) pk[e >> 4][e & 15] = 0u;
+                r_pub[i % kRefSlots][r_loc] = r_now;
+                mbar_arrive_warp(bar_ref(i % kRefSlots, quarter));
+                tc_fence_before();
+                mbar_arrive_warp(bar_sfree(wg));     // S_g may take the scores of step i+2
+                if (m_w != r_now) { l_w *= ex2_approx(m_w - r_now); m_w = r_now; }   // first use: l_w = 0, exp2(-inf) = 0
+                exps(2, r_now);
             } else {
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
+                for (int c = 0; c < 4; ++c) tmem_ld32(tS + c * 32, s[c]);
+                tmem_wait_ld();
+                tc_fence_before();
+                mbar_arrive_warp(bar_sfree(wg));     // the scores are in registers: S_g may take the scores of step i+2
+                if (nvalid < kBlock) {               // ragged tail (warp-uniform): keys >= N never count
 #pragma unroll
-                for (int e = 0; e < 16; ++e) {
-                    float x0, x1;
-                    unpack2(fma2(pack2(s[c][2 * e], s[c][2 * e + 1]), scale2, neg_m2), x0, x1);
-                    const float p0 = ex2_approx(x0), p1 = ex2_approx(x1);
-                    part2[e & 1] = add2(part2[e & 1], pack2(p0, p1));
-                    pk[c][e] = pack_bf16(p0, p1);
+                    for (int c = 0; c < 4; ++c)
+#pragma unroll
+                        for (int e = 0; e < 32; ++e)
+                            if (c * 32 + e >= nvalid) s[c][e] = -INFINITY;
                 }
-            }
+                // 64-token blocks: the halves of the step that this warp's rows list (a pad entry is listed by nobody)
+                bool on0 = true, on1 = true;
+                if (kPlanned) {
+                    const int bit = kPlanRowBit + (second ? 1 : 0);
+                    on0 = (plan[i * kPerStep] >> bit) & 1;
+                    on1 = (plan[i * kPerStep + kPerStep - 1] >> bit) & 1;
+                    if (!on0) {
+#pragma unroll
+                        for (int e = 0; e < 64; ++e) s[e >> 5][e & 31] = -INFINITY;
+                    }
+                    if (!on1) {
+#pragma unroll
+                        for (int e = 64; e < 128; ++e) s[e >> 5][e & 31] = -INFINITY;
+                    }
+                }
+                // row maximum of the raw scores (the scale is positive), four independent chains
+                float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+#pragma unroll
+                    for (int e = 0; e < 32; e += 2) mx4[(e >> 1) & 3] = max3(mx4[(e >> 1) & 3], s[c][e], s[c][e + 1]);
+                const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * a.scale_log2;
+                // reference handed over from step i-1
+                float r_prev = -INFINITY, r_now = mx;
+                bool grow = false;
+                if (i > 0) {
+                    ok = mbar_wait_warp(bar_ref((i - 1) % kRefSlots, quarter), uint32_t((i - 1) / kRefSlots) & 1u, abortp, 0, limit);
+                    if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 10, i, blockIdx.x); break; }
+                    r_prev = r_pub[(i - 1) % kRefSlots][r_loc];
+                    grow = mx > r_prev + kRescaleThreshold;
+                    r_now = grow ? mx : r_prev;
+                }
+                r_pub[i % kRefSlots][r_loc] = r_now;
+                mbar_arrive_warp(bar_ref(i % kRefSlots, quarter));
+                // The one P buffer is free again once P V of step i-1 (the other group's) has read it.  The probabilities
+                // are kept in registers until they are all there, so that wait comes after the exponentials; the rescaling
+                // path needs the same product to be complete (O quiescent) and takes the wait early.  Each step waits on
+                // the phase that follows the one it waited on two steps earlier, so the phase is never ambiguous.
+                p_free = i < 1;
+                if (i > 0 && __any_sync(0xffffffffu, grow)) {
+                    p_free = true;
+                    // O must be quiescent: P V of step i-1 (the other group's) complete.  P V is issued in step order
+                    // and that of step i cannot start before this group delivers P_i.
+                    ok = mbar_wait_warp(bar_pvdone(wg ^ 1), uint32_t((i - 1) >> 1) & 1u, abortp, 0, limit);
+                    if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 9, i, blockIdx.x); break; }
+                    tc_fence_after();
+                    // 1 for rows that did not move (rows of a pair may both times be at -inf: nothing listed so far)
+                    const float f = !kPairs || grow ? ex2_approx(r_prev - r_now) : 1.f;
+#pragma unroll
+                    for (int c = 0; c < D / 32; ++c) {
+                        float o[32];
+                        tmem_ld32(tmem + lane_base + kColO + c * 32, o);
+                        tmem_wait_ld();
+                        uint32_t r[32];
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(o[e] * f);
+                        tmem_st32(tmem + lane_base + kColO + c * 32, r);
+                    }
+                }
+                if (m_w != r_now) { l_w *= ex2_approx(m_w - r_now); m_w = r_now; }   // first use: l_w = 0, exp2(-inf) = 0
+                // P = exp2(s * scale - R_i): one FFMA + one MUFU per element, packed bf16 pairs over S's own columns
+                const uint64_t neg_m2 = pack2(-r_now, -r_now), scale2 = pack2(a.scale_log2, a.scale_log2);
+                part2[0] = part2[1] = pack2(0.f, 0.f);
+                if (kPairs && !on0 && !on1) {        // warp-uniform: nothing of this step belongs to these rows (their reference may be -inf)
+#pragma unroll
+                    for (int e = 0; e < 64; ++e) pk[e >> 4][e & 15] = 0u;
+                } else {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) {
+                        float x0, x1;
+                        unpack2(fma2(pack2(s[c][2 * e], s[c][2 * e + 1]), scale2, neg_m2), x0, x1);
+                        const float p0 = ex2_approx(x0), p1 = ex2_approx(x1);
+                        part2[e & 1] = add2(part2[e & 1], pack2(p0, p1));
+                        pk[c][e] = pack_bf16(p0, p1);
+                    }
+                }
+                }
             }
             if (!p_free) {      // the one P buffer is free once P V of step i-1 (the other group's) has read it
                 ok = mbar_wait_warp(bar_pvdone(wg ^ 1), uint32_t((i - 1) >> 1) & 1u, abortp, 0, limit);

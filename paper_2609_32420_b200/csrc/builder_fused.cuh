@@ -97,17 +97,6 @@ __device__ __forceinline__ float tmem_ld1(uint32_t taddr) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr) : "memory");
     return __uint_as_float(r);
 }
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr) : "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
 // Shared-memory plan.  Pooling ring: blocks of 128 token rows as D/64 boxes (128 rows x 128 B, 128-byte swizzle).
 // Score operands: A = the three terms of 128 key-block means, one 32-element quarter of the head dimension at a time
 // (3 boxes of 128 rows x 64 B, 64-byte swizzle), AST buffers; B = the three terms of the item's 16 query-block means,
@@ -479,12 +468,12 @@ build_fused_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
                 const int tile = (warp >> 2) + j * (NW / 4);
                 if (tile < ntiles) {                                   // warp-uniform
                     float u[16];
-                    tmem_ld16(tmem_s + lane_base + uint32_t(tile * NR * NACC + c0), v[j]);                        // t1 t1 (first half of d)
-                    tmem_ld16(tmem_s + lane_base + uint32_t(tile * NR * NACC + (NACC - 1) * NR + c0), u);         // the small products
+                    tc::tmem_ld16(tmem_s + lane_base + uint32_t(tile * NR * NACC + c0), v[j]);                        // t1 t1 (first half of d)
+                    tc::tmem_ld16(tmem_s + lane_base + uint32_t(tile * NR * NACC + (NACC - 1) * NR + c0), u);         // the small products
                     tc::tmem_wait_ld();
                     if (NACC == 3) {
                         float v2[16];
-                        tmem_ld16(tmem_s + lane_base + uint32_t(tile * NR * NACC + NR + c0), v2);                  // t1 t1, second half
+                        tc::tmem_ld16(tmem_s + lane_base + uint32_t(tile * NR * NACC + NR + c0), v2);                  // t1 t1, second half
                         tc::tmem_wait_ld();
 #pragma unroll
                         for (int i = 0; i < 16; ++i) v[j][i] += v2[i];
