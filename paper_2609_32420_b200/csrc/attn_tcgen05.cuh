@@ -1070,16 +1070,23 @@ inline carnator_status launch_tc(const AttnArgs& a, const CUtensorMap& mk, const
                                  cudaStream_t stream, char* err, size_t errlen) {
     const uint32_t smem = tc::Cfg<D>::kSmemBytes + (BQ == 64 || BK == 64 ? tc::plan_bytes(a.nkb) : 0u);
     auto kern = tc::attn_tcgen05_kernel<D, BQ, BK>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    if (e != cudaSuccess) { snprintf(err, errlen, "cudaFuncSetAttribute(tcgen05): %s", cudaGetErrorString(e)); return CARNATOR_ERR_CUDA; }
-    // The register hand-over inside the kernel only completes if the CTA owns enough registers: check what the
-    // compiler allocated instead of finding out on the device.
-    cudaFuncAttributes fa;
-    e = cudaFuncGetAttributes(&fa, kern);
-    if (e != cudaSuccess) { snprintf(err, errlen, "cudaFuncGetAttributes(tcgen05): %s", cudaGetErrorString(e)); return CARNATOR_ERR_CUDA; }
-    if (fa.numRegs * tc::kThreads < tc::kSoftmaxWarps * 32 * tc::kRegsSoftmax + 128 * tc::kRegsService) {
-        snprintf(err, errlen, "attn_tcgen05_kernel was built with %d registers per thread: too few for its setmaxnreg split", fa.numRegs);
-        return CARNATOR_ERR_UNSUPPORTED;
+    static SmemAllowed allowed;
+    cudaError_t e;
+    int dev;
+    if (!allowed.has(smem, &dev)) {      // once: with room for the longest plan
+        const uint32_t most = tc::Cfg<D>::kSmemBytes + (BQ == 64 || BK == 64 ? tc::plan_bytes(tc::kPlanMaxKeyBlocks) : 0u);
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(most));
+        if (e != cudaSuccess) { snprintf(err, errlen, "cudaFuncSetAttribute(tcgen05): %s", cudaGetErrorString(e)); return CARNATOR_ERR_CUDA; }
+        // The register hand-over inside the kernel only completes if the CTA owns enough registers: check what the
+        // compiler allocated instead of finding out on the device.
+        cudaFuncAttributes fa;
+        e = cudaFuncGetAttributes(&fa, kern);
+        if (e != cudaSuccess) { snprintf(err, errlen, "cudaFuncGetAttributes(tcgen05): %s", cudaGetErrorString(e)); return CARNATOR_ERR_CUDA; }
+        if (fa.numRegs * tc::kThreads < tc::kSoftmaxWarps * 32 * tc::kRegsSoftmax + 128 * tc::kRegsService) {
+            snprintf(err, errlen, "attn_tcgen05_kernel was built with %d registers per thread: too few for its setmaxnreg split", fa.numRegs);
+            return CARNATOR_ERR_UNSUPPORTED;
+        }
+        allowed.set(most, dev);
     }
     dim3 grid(BQ == 64 ? ceil_div(a.nqb, 2) : a.nqb, a.H, a.B);
     e = launch_dependent(kern, grid, dim3(tc::kThreads), smem, stream, mk, mv, a);

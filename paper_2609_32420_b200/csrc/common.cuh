@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
+#include <atomic>
 
 #include "carnator.h"
 
@@ -97,6 +98,22 @@ struct Geometry {
 // Programmatic dependent launch: the next kernel of a call starts while this one drains, and waits here for its results.
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// How much dynamic shared memory a kernel has been allowed on each device: asking the runtime costs about a microsecond a
+// call.  One static object per kernel, at the place that launches it.
+struct SmemAllowed {
+    static constexpr int kDevices = 64;
+    std::atomic<uint32_t> bytes[kDevices];
+    // true if `need` is already allowed on the current device
+    bool has(size_t need, int* dev) const {
+        *dev = -1;
+        if (cudaGetDevice(dev) != cudaSuccess || *dev < 0 || *dev >= kDevices) return false;
+        return bytes[*dev].load(std::memory_order_acquire) >= need;
+    }
+    void set(size_t now, int dev) {
+        if (dev >= 0 && dev < kDevices) bytes[dev].store(uint32_t(now), std::memory_order_release);
+    }
+};
 
 // Launch that may begin before the kernel ahead of it in the stream has ended (that kernel calls grid_launch_dependents,
 // this one grid_wait before it reads anything of it).
