@@ -465,12 +465,14 @@ static carnator_status compact_impl(const uint8_t* mask, const uint8_t* recomput
         st = allow_smem(kern, smem);
         if (st != CARNATOR_OK) return st;
     }
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // behind the region kernels, for instance
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = unsigned(ca.ctas); at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(unsigned(s->B) * s->H * ca.ctas); cfg.blockDim = dim3(kCompactThreads);
-    cfg.dynamicSmemBytes = smem; cfg.stream = stream; cfg.attrs = at; cfg.numAttrs = 1;
+    cfg.dynamicSmemBytes = smem; cfg.stream = stream; cfg.attrs = at; cfg.numAttrs = 2;
     CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, ca));
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return CARNATOR_OK;
@@ -811,11 +813,13 @@ extern "C" carnator_status carnator_build_regions(const uint8_t* evidence, const
     uint8_t* dist = static_cast<uint8_t*>(ws) + align256(sizeof(WsHeader));
     const int n = s->T * s->Hg * s->Wg;
     CUDA_TRY(cudaMemsetAsync(hdr, 0, sizeof(WsHeader), stream));
-    region_distance_kernel<<<ceil_div(n, 256), 256, 0, stream>>>(evidence, s->T, s->Hg, s->Wg, r_active, r_context, dist,
-                                                                 active, context, hdr);
+    static_assert(kRegionMaxR == 32, "the largest r_active + r_context accepted above");
+    const int tx = ceil_div(s->Wg, kRegionTileX), ty = ceil_div(s->Hg, kRegionTileY);
+    region_distance_kernel<<<unsigned(int64_t(s->T) * tx * ty), kRegionTileX * kRegionTileY, 0, stream>>>(
+        evidence, s->Hg, s->Wg, tx, ty, r_active, r_context, dist, active, context, hdr);
     LAUNCH_CHECK("region_distance_kernel");
-    region_weight_kernel<<<ceil_div(n, 256), 256, 0, stream>>>(dist, n, r_active, hdr, W);
-    LAUNCH_CHECK("region_weight_kernel");
+    CUDA_TRY(launch_dependent(region_weight_kernel, dim3(ceil_div(n, 256)), dim3(256), 0, stream, dist, n, r_active, hdr, W));
+    g_launches.fetch_add(1, std::memory_order_relaxed);
     return CARNATOR_OK;
 }
 
@@ -852,8 +856,9 @@ extern "C" carnator_status carnator_region_block_flags(const uint8_t* region, co
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     const int n_video = s->T * s->Hg * s->Wg;
     const int nblocks = ceil_div(s->n_text + n_video, block);
-    region_block_flags_kernel<<<ceil_div(nblocks, 8), 256, 0, stream>>>(region, s->n_text, n_video, block, text_value, nblocks, flags);
-    LAUNCH_CHECK("region_block_flags_kernel");
+    CUDA_TRY(launch_dependent(region_block_flags_kernel, dim3(ceil_div(nblocks, 8)), dim3(256), 0, stream, region, s->n_text, n_video,
+                              block, text_value, nblocks, flags));
+    g_launches.fetch_add(1, std::memory_order_relaxed);
     return CARNATOR_OK;
 }
 

@@ -34,6 +34,7 @@ __global__ void __launch_bounds__(kCompactThreads) compact_order_kernel(CompactA
     const int nqb = a.nqb, nkb = a.nkb, b = bh / a.H;
     const int share = (nqb + a.ctas - 1) / a.ctas, i_lo = min(nqb, rank_cta * share), i_hi = min(nqb, i_lo + share);
     grid_launch_dependents();
+    grid_wait();
     if (blockIdx.x == 0 && tid < int(sizeof(WsHeader) / 4)) reinterpret_cast<int32_t*>(a.hdr)[tid] = 0;
     const uint8_t* ctx = a.context_k ? a.context_k + int64_t(b) * nkb : nullptr;
     unsigned active = ~0u, recomp = 0u;          // flags of this warp's next 32 rows, fetched together

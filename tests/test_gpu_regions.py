@@ -108,3 +108,18 @@ def test_region_restricted_attention_end_to_end(impl, name, kw):
     assert (Oh[skipped] == 3.0).all() and (Lh[skipped] == -7.0).all()
     eff = (mask != 0) & (aq != 0)[:, None, :, None] & (ck != 0)[:, None, None, :]
     assert cn.compacted_tiles(shape, ws) == int(eff.sum())
+
+
+@pytest.mark.parametrize("T,H,W,ra,rc", [(1, 1, 1, 1, 0), (2, 9, 33, 2, 3), (3, 8, 32, 1, 31), (2, 70, 65, 16, 16), (1, 7, 200, 3, 2)])
+def test_regions_at_the_edges_of_a_tile(T, H, W, ra, rc):
+    """Frames smaller than, equal to and just past a tile of 8 x 32 tokens, the largest accepted radius, evidence in the corners."""
+    rng = np.random.default_rng(T * H * W + ra)
+    ev = (rng.random((T, H, W)) < 0.002).astype(np.uint8)
+    ev[0, 0, 0] = 1
+    ev[T - 1, H - 1, W - 1] = 1
+    shape = cn.make_shape(1, 1, T * H * W, 128, 0, T, H, W, 128, 128)
+    a, c, Wt = cn.build_regions(torch.from_numpy(ev).cuda(), shape, ra, rc)
+    a_ref, c_ref, W_ref = orc.build_regions(ev, ra, rc)
+    np.testing.assert_array_equal(a.cpu().numpy() != 0, a_ref)
+    np.testing.assert_array_equal(c.cpu().numpy() != 0, c_ref)
+    np.testing.assert_allclose(Wt.cpu().numpy(), W_ref, atol=1e-6)
