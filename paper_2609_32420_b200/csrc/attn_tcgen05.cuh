@@ -198,6 +198,16 @@ __device__ __forceinline__ void mma_ts_el_rows(uint32_t d_tmem, uint32_t a_tmem,
         "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, {%5, %5, %6, %6}, p;\n\t}"
         ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(off_lo), "r"(off_hi), "r"(accumulate) : "memory");
 }
+// D[tmem] (+)= A[smem] * B[smem], both descriptors given as (low word, shared high word); converged warp, one elected
+// lane issues (see mma_ts_el)
+__device__ __forceinline__ void mma_ss_el(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p, e;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %5, 0;\n\t"
+        "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate) : "memory");
+}
 __device__ __forceinline__ void tc_commit_el(uint32_t bar) {
     asm volatile(
         "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"

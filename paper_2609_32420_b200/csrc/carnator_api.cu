@@ -908,13 +908,12 @@ extern "C" carnator_status carnator_seed_expansion(const void* Q, const void* K,
     const int64_t n_bn = int64_t(s->B) * s->N;
     if (seed_tcgen05_supported(s, n_pos + n_neg)) {
         WsHeader* hdr = static_cast<WsHeader*>(ws);
-        CUDA_TRY(cudaMemsetAsync(hdr, 0, sizeof(WsHeader), stream));
         int sms = 0;
         st = sm_count(&sms);
         if (st != CARNATOR_OK) return st;
         tc::SeedGatherArgs ga;
         ga.K = a.K; for (int i = 0; i < 3; ++i) ga.ks[i] = a.ks[i];
-        ga.seeds = seeds; ga.n_seeds = n_pos + n_neg; ga.H = s->H; ga.N = s->N;
+        ga.seeds = seeds; ga.n_seeds = n_pos + n_neg; ga.H = s->H; ga.N = s->N; ga.hdr = hdr;
         ga.out = reinterpret_cast<__nv_bfloat16*>(static_cast<char*>(ws) + align256(sizeof(WsHeader)) +
                                                    align256(size_t(s->B) * s->H * s->N * 4));
         tc::SeedTcArgs ta;
@@ -932,8 +931,8 @@ extern "C" carnator_status carnator_seed_expansion(const void* Q, const void* K,
         st = s->D == 128 ? launch_seed_tc<128>(ga, ta, mq, ms, sms, stream, g_cuda_error, sizeof(g_cuda_error))
                          : launch_seed_tc<64>(ga, ta, mq, ms, sms, stream, g_cuda_error, sizeof(g_cuda_error));
         if (st != CARNATOR_OK) return st;
-        head_mean_kernel<<<unsigned((n_bn + 255) / 256), 256, 0, stream>>>(a.per_head, s->B, s->H, s->N, contrast);
-        LAUNCH_CHECK("head_mean_kernel");
+        CUDA_TRY(launch_dependent(head_mean_kernel, dim3(unsigned((n_bn + 255) / 256)), dim3(256), 0, stream, a.per_head, s->B, s->H, s->N, contrast));
+        g_launches.fetch_add(1, std::memory_order_relaxed);
         return CARNATOR_OK;
     }
     dim3 grid(ceil_div(s->N, 128), s->H, s->B);

@@ -124,6 +124,7 @@ __global__ void __launch_bounds__(256) seed_expand_kernel(SeedArgs a) {
 // mean over heads, in head order (deterministic)
 __global__ void __launch_bounds__(256) head_mean_kernel(const float* __restrict__ per_head, int B, int H, int N,
                                                         float* __restrict__ out) {
+    grid_wait();
     const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= int64_t(B) * N) return;
     const int b = int(i / N), n = int(i % N);

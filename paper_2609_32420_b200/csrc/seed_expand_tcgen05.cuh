@@ -37,14 +37,18 @@ struct SeedGatherArgs {
     int64_t ks[3];
     const int32_t* seeds;
     __nv_bfloat16* out;      // [B*H][kSeedCap][D]
+    WsHeader* hdr;
     int n_seeds, H, N;
 };
 
-// one 16-byte piece per thread; rows past the seed count and seeds outside [0, N) become zero rows
+// one 16-byte piece per thread; the first CTA clears the workspace header; rows past the seed count and seeds outside [0, N) become zero rows
 template <int D>
 __global__ void __launch_bounds__(256) seed_gather_kernel(SeedGatherArgs a) {
     constexpr int VEC = D / 8;
+    grid_launch_dependents();
     const int idx = blockIdx.x * 256 + threadIdx.x;
+    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x < sizeof(WsHeader) / 4)
+        reinterpret_cast<int32_t*>(a.hdr)[threadIdx.x] = 0;
     if (idx >= kSeedCap * VEC) return;
     const int r = idx / VEC, v = idx % VEC;
     const int h = blockIdx.y, b = blockIdx.z;
@@ -62,17 +66,6 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
         ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1) : "memory");
 }
-// D[tmem] (+)= A[smem] * B[smem], both descriptors given as (low word, shared high word); converged warp, one elected
-// lane issues (see mma_ts_el)
-__device__ __forceinline__ void mma_ss_el(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p, e;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %5, 0;\n\t"
-        "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
-        "elect.sync _|e, 0xffffffff;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate) : "memory");
-}
-
 template <int D>
 struct SeedCfg {
     static constexpr int kBoxes = D / 64;
@@ -102,7 +95,7 @@ seed_expand_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
     auto bar_sfull = [&](int g, int c) { return bars + 64 + 8 * (g * 2 + c); };   // chunk c of a tile of group g is in tensor memory
     auto bar_sfree = [&](int c) { return bars + 96 + 8 * c; };         // the tile's group has read chunk c
     volatile int* abortp = &abort_flag;
-    const unsigned long long limit = a.hdr->wait_limit_ns ? a.hdr->wait_limit_ns : kDefaultWaitNs;
+    grid_launch_dependents();
 
     // this CTA's tiles: a contiguous range of the (batch, head, query tile) order, so a head's seed rows are loaded
     // once per CTA that touches the head
@@ -122,6 +115,8 @@ seed_expand_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(512) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    grid_wait();                            // launched while the gather kernel drains
+    const unsigned long long limit = a.hdr->wait_limit_ns ? a.hdr->wait_limit_ns : kDefaultWaitNs;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -282,8 +277,7 @@ inline carnator_status launch_seed_tc(const tc::SeedGatherArgs& ga, const tc::Se
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::kSmemBytes));
     if (e != cudaSuccess) { snprintf(err, errlen, "cudaFuncSetAttribute(seed tcgen05): %s", cudaGetErrorString(e)); return CARNATOR_ERR_CUDA; }
     const int grid = a.tiles < sms ? a.tiles : sms;
-    kern<<<grid, tc::kSeedThreads, C::kSmemBytes, stream>>>(mq, ms, a);
-    e = cudaGetLastError();
+    e = launch_dependent(kern, dim3(grid), dim3(tc::kSeedThreads), C::kSmemBytes, stream, mq, ms, a);
     if (e != cudaSuccess) { snprintf(err, errlen, "seed_expand_tc_kernel: %s", cudaGetErrorString(e)); return CARNATOR_ERR_CUDA; }
     return CARNATOR_OK;
 }
