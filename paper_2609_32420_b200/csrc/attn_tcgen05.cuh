@@ -485,8 +485,6 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
     auto bar_ref = [&](int s, int q) { return bars + 224 + 8 * (s * 4 + q); };   // r_pub slot s, lane quarter q
     auto bar_fin = [&](int q) { return bars + 320 + 8 * q; };
     auto bar_pvdone = [&](int s) { return bars + 352 + 8 * s; };     // P V of the step that used score buffer s has completed
-    auto bar_pva = [&](int s) { return bars + 368 + 8 * s; };
-    auto bar_pfullb = [&](int s) { return bars + 384 + 8 * s; };
     volatile int* abortp = &abort_flag;
     // every bounded wait of this CTA gives up after `limit` (2 s unless the workspace header asks for less)
     const unsigned long long limit = a.hdr->wait_limit_ns ? a.hdr->wait_limit_ns : kDefaultWaitNs;
@@ -498,7 +496,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
             mbar_init(bar_kfull(s), 1); mbar_init(bar_vfull(s), 1);
         }
         for (int s = 0; s < kSBufs; ++s) {
-            mbar_init(bar_sfull(s), 1); mbar_init(bar_pvdone(s), 1); mbar_init(bar_pva(s), 1); mbar_init(bar_pfullb(s), 4);
+            mbar_init(bar_sfull(s), 1); mbar_init(bar_pvdone(s), 1);
             mbar_init(bar_pfull(s), 4); mbar_init(bar_sfree(s), 4);          // one arrival per softmax warp of the group
         }
         for (int s = 0; s < kRefSlots; ++s)
