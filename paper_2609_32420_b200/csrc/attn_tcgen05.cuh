@@ -31,6 +31,7 @@
 // the workspace header, raises a CTA-wide abort flag, and every role drains and returns.
 #pragma once
 #include <cuda.h>
+#include <algorithm>
 
 #include "common.cuh"
 #include "attn_portable.cuh"
@@ -410,12 +411,21 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
     __shared__ float fin[2][2][kBlock];         // per warpgroup: final reference maximum and partial row sum
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int b = blockIdx.z, h = blockIdx.y;
+    // Grid at D = 128: (heads of a group, position in the execution order, groups of heads), see head_group.  At D = 64:
+    // (position, head, batch entry); computed coordinates cost that loop 0.9 %.
+    constexpr bool kGroups = D == 128;
+    int b, h;
+    if constexpr (kGroups) {
+        const uint32_t head = blockIdx.z * gridDim.x + blockIdx.x;
+        if (head >= uint32_t(a.B) * uint32_t(a.H)) return;      // the last group may be short
+        b = int(head / uint32_t(a.H)); h = int(head - uint32_t(b) * uint32_t(a.H));
+    } else { b = blockIdx.z; h = blockIdx.y; }
     const int64_t bh = int64_t(b) * a.H + h;
     grid_wait();                            // launched while the compaction drains
     constexpr bool kPairs = BQ == 64, kPlanned = BQ == 64 || BK == 64;
     constexpr int kPerStep = kBlock / BK;             // listed key blocks in a step
-    const int x0 = kPairs ? 2 * blockIdx.x : blockIdx.x;
+    const int place = kGroups ? blockIdx.y : blockIdx.x;
+    const int x0 = kPairs ? 2 * place : place;
     const int I = a.order[bh * a.nqb + x0];
     int T = a.counts[bh * a.nqb + I];                 // steps = listed key blocks
     const int32_t* list = a.lists + (bh * a.nqb + I) * int64_t(a.nkb);
@@ -430,7 +440,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
     if (kPlanned) {
         __shared__ int plan_total;
         if (T > a.nkb || T2 > a.nkb) {                // counts that cannot come from compaction
-            if (tid == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_CHECK, 20, max(T, T2), blockIdx.x);
+            if (tid == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_CHECK, 20, max(T, T2), place);
             return;
         }
         if (T <= 0 && T2 <= 0) {                      // nothing to attend to: O = 0, LSE = -inf where a block is listed empty
@@ -450,7 +460,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
         n_listed = build_plan<kPairs>(a, list, max(T, 0), a.lists + (bh * a.nqb + max(I2, 0)) * int64_t(a.nkb), max(T2, 0),
                                       words, plan, &plan_total);
         if (n_listed < 0) {
-            if (tid == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_CHECK, 21, I, blockIdx.x);
+            if (tid == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_CHECK, 21, I, place);
             return;
         }
     }
@@ -459,7 +469,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
 
     if (T < 0) return;                      // skipped query block (region-restricted form): output untouched
     if (T > a.nkb) {                        // a count that cannot come from compaction: stop before reading a list that long
-        if (tid == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_CHECK, 20, T, blockIdx.x);
+        if (tid == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_CHECK, 20, T, place);
         return;
     }
     if (T == 0) {                           // nothing to attend to: O = 0, LSE = -inf
@@ -489,8 +499,11 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
     // every bounded wait of this CTA gives up after `limit` (2 s unless the workspace header asks for less)
     const unsigned long long limit = a.hdr->wait_limit_ns ? a.hdr->wait_limit_ns : kDefaultWaitNs;
 
+    // for the epilogue: kept in registers through the loop they slow it down by 1.3 % (grid coordinates are free, these are not)
+    __shared__ volatile int at_b, at_h;
     if (tid == 0) {
         abort_flag = 0;
+        if (kGroups) { at_b = b; at_h = h; }
         mbar_init(bar_q, kSoftmaxWarps); mbar_init(bar_o, 1); mbar_init(bar_drain, 1); mbar_init(bar_drain2, 1);
         for (int s = 0; s < kStages; ++s) {
             mbar_init(bar_kfull(s), 1); mbar_init(bar_vfull(s), 1);
@@ -527,15 +540,15 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
             for (int i = 0; i < T; ++i) {
                 const int s = i % kStages, u = i - kStages;     // the slot is free once Q K^T of step u has completed
                 if (u >= 0 && !mbar_wait(bar_sfull(u & 1), uint32_t(u >> 1) & 1u, abortp, 100, limit)) {
-                    set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 1, i, blockIdx.x); break;
+                    set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 1, i, place); break;
                 }
                 const int J = kPlanned ? 0 : list[i];
                 if (!kPlanned && (J < 0 || J >= a.nkb || (i > 0 && J <= list[i - 1]))) {   // malformed list: stop before touching memory
-                    set_status(a.hdr, CARNATOR_ERR_DEVICE_CHECK, 21, i, blockIdx.x); *abortp = 1; break;
+                    set_status(a.hdr, CARNATOR_ERR_DEVICE_CHECK, 21, i, place); *abortp = 1; break;
                 }
                 // Test of the time-out path only: the first K tile of the first query block in the order is never
                 // requested, so the wait for it runs out and the CTA takes the abort-and-drain path.
-                if (i == 0 && a.hdr->debug_withhold != 0 && blockIdx.x == 0 && bh == 0) continue;
+                if (i == 0 && a.hdr->debug_withhold != 0 && place == 0 && bh == 0) continue;
                 mbar_expect_tx(bar_kfull(s), C::kTileBytes);
 #pragma unroll
                 for (int kh = 0; kh < kPerStep; ++kh) {
@@ -558,7 +571,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
             for (int i = 0; i < T; ++i) {
                 const int s = i % kStages, u = i - kStages;     // the slot is free once P V of step u has completed
                 if (u >= 0 && !mbar_wait(bar_pvdone(u & 1), uint32_t(u >> 1) & 1u, abortp, 100, limit)) {
-                    set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 2, i, blockIdx.x); break;
+                    set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 2, i, place); break;
                 }
                 const int J = kPlanned ? 0 : list[i];
                 if (!kPlanned && (J < 0 || J >= a.nkb)) { *abortp = 1; break; }   // reported by the K producer
@@ -588,13 +601,13 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
         const uint64_t dk = smem_desc(sK, 16, 1024);
         const uint32_t k_lo0 = uint32_t(dk), hi_kmajor = uint32_t(dk >> 32);
         bool ok = mbar_wait_warp(bar_q, 0, abortp, 0, limit);   // the softmax groups have put the query tile into tensor memory
-        if (!ok && lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 3, 0, blockIdx.x);
+        if (!ok && lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 3, 0, place);
         tc_fence_after();
         for (int iq = 0; iq < T && ok; ++iq) {
             const int s = iq % kStages, g = iq & 1;
             ok = mbar_wait_warp(bar_kfull(s), uint32_t(iq / kStages) & 1u, abortp, 0, limit);
             if (ok && iq >= 2) ok = mbar_wait_warp(bar_sfree(g), uint32_t((iq - 2) >> 1) & 1u, abortp, 0, limit);
-            if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 4, iq, blockIdx.x); break; }
+            if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 4, iq, place); break; }
             tc_fence_after();
             // Q from tensor memory, K tile K-major, 16 elements of the head dimension per instruction
             const uint32_t k_lo = k_lo0 + uint32_t(s) * (C::kTileBytes >> 4), d_s = tmem + g * kBlock;
@@ -621,7 +634,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
             const int s = ip % kStages, g = ip & 1;
             ok = mbar_wait_warp(bar_vfull(s), uint32_t(ip / kStages) & 1u, abortp, 0, limit);
             if (ok) ok = mbar_wait_warp(bar_pfull(g), uint32_t(ip >> 1) & 1u, abortp, 0, limit);
-            if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 5, ip, blockIdx.x); break; }
+            if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 5, ip, place); break; }
             tc_fence_after();
             // P from tensor memory (16 keys = 8 packed columns per instruction), V tile as the MN-major B operand
             // (rows = keys, 64-element chunks of the head dimension one box apart)
@@ -704,7 +717,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
         for (int i = wg; i < T; i += 2) {
             const uint32_t sph = uint32_t(i >> 1) & 1u;
             ok = mbar_wait_warp(bar_sfull(wg), sph, abortp, 20, limit);   // warp-uniform: the loads below are collective
-            if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 7, i, blockIdx.x); break; }
+            if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 7, i, place); break; }
             tc_fence_after();
             const int nvalid = (i == T - 1) ? nvalid_last : kBlock;      // >= 1; < 128 only for a ragged last block
             const uint32_t tS = tmem + lane_base + wg * kBlock;
@@ -736,7 +749,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
                 float r_now = -INFINITY;
                 if (i > 0) {                         // reference handed over from step i-1
                     ok = mbar_wait_warp(bar_ref((i - 1) % kRefSlots, quarter), uint32_t((i - 1) / kRefSlots) & 1u, abortp, 0, limit);
-                    if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 10, i, blockIdx.x); break; }
+                    if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 10, i, place); break; }
                     r_now = r_pub[(i - 1) % kRefSlots][r_loc];
                 }
                 const uint64_t scale2 = pack2(a.scale_log2, a.scale_log2);
@@ -773,7 +786,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
                         // and that of step i cannot start before this group delivers P_i.
                         p_free = true;
                         ok = mbar_wait_warp(bar_pvdone(wg ^ 1), uint32_t((i - 1) >> 1) & 1u, abortp, 0, limit);
-                        if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 9, i, blockIdx.x); break; }
+                        if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 9, i, place); break; }
                         tc_fence_after();
                         const float f = ex2_approx(r_prev - r_now);          // 1 for rows that did not move
 #pragma unroll 1
@@ -839,7 +852,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
                 bool grow = false;
                 if (i > 0) {
                     ok = mbar_wait_warp(bar_ref((i - 1) % kRefSlots, quarter), uint32_t((i - 1) / kRefSlots) & 1u, abortp, 0, limit);
-                    if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 10, i, blockIdx.x); break; }
+                    if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 10, i, place); break; }
                     r_prev = r_pub[(i - 1) % kRefSlots][r_loc];
                     grow = mx > r_prev + kRescaleThreshold;
                     r_now = grow ? mx : r_prev;
@@ -856,7 +869,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
                     // O must be quiescent: P V of step i-1 (the other group's) complete.  P V is issued in step order
                     // and that of step i cannot start before this group delivers P_i.
                     ok = mbar_wait_warp(bar_pvdone(wg ^ 1), uint32_t((i - 1) >> 1) & 1u, abortp, 0, limit);
-                    if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 9, i, blockIdx.x); break; }
+                    if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 9, i, place); break; }
                     tc_fence_after();
                     // 1 for rows that did not move (rows of a pair may both times be at -inf: nothing listed so far)
                     const float f = !kPairs || grow ? ex2_approx(r_prev - r_now) : 1.f;
@@ -894,7 +907,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
             }
             if (!p_free) {      // the one P buffer is free once P V of step i-1 (the other group's) has read it
                 ok = mbar_wait_warp(bar_pvdone(wg ^ 1), uint32_t((i - 1) >> 1) & 1u, abortp, 0, limit);
-                if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 12, i, blockIdx.x); break; }
+                if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 12, i, place); break; }
             }
 #pragma unroll
             for (int c = 0; c < 4; ++c) tmem_st16(tP + c * 16, pk[c]);
@@ -913,11 +926,11 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
             fin[wg][1][r_loc] = l_w;
             mbar_arrive_warp(bar_fin(quarter));
             ok = mbar_wait_warp(bar_fin(quarter), 0, abortp, 0, limit);
-            if (!ok && lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 11, T, blockIdx.x);
+            if (!ok && lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 11, T, place);
         }
         if (ok) {
             ok = mbar_wait_warp(bar_o, 0, abortp, 20, limit);
-            if (!ok && lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 8, T, blockIdx.x);
+            if (!ok && lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 8, T, place);
         }
         if (ok) {
             tc_fence_after();
@@ -928,7 +941,8 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
             // rows of a pair that list nothing: O = 0, LSE = -inf
             const float inv = !kPairs || l_tot > 0.f ? 1.f / l_tot : 0.f;
             // each group writes half of the head dimension
-            __nv_bfloat16* op = a.O + b * a.os[0] + h * a.os[1] + int64_t(row) * a.os[2] + wg * (D / 2);
+            const int eb = kGroups ? at_b : b, eh = kGroups ? at_h : h;
+            __nv_bfloat16* op = a.O + eb * a.os[0] + eh * a.os[1] + int64_t(row) * a.os[2] + wg * (D / 2);
 #pragma unroll
             for (int c = 0; c < D / 64; ++c) {
                 float o[32];
@@ -946,7 +960,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
                     }
                 }
             }
-            if (wg == 0 && row_in) a.LSE[bh * a.N + row] = !kPairs || l_tot > 0.f ? (r_fin + log2f(l_tot)) * kLn2 : -INFINITY;
+            if (wg == 0 && row_in) a.LSE[(int64_t(eb) * a.H + eh) * a.N + row] = !kPairs || l_tot > 0.f ? (r_fin + log2f(l_tot)) * kLn2 : -INFINITY;
         }
     }
 
@@ -1073,6 +1087,18 @@ inline bool tcgen05_takes(const carnator_shape* s) {
            tma_strides_ok(s, s->k_stride) && tma_strides_ok(s, s->v_stride);
 }
 
+// Heads that run side by side, the longest rows of all of them first.  One head after the other, the full rows of the last
+// head start when nearly everything else is done, and most SMs wait for them: five-frame clip (24 heads, 10 tiles per SM)
+// 406 -> 390 us.  Only for layers of up to 16 tiles per SM: on longer ones that wait is no longer seen.  As many heads as keep K and V within 24 MB, so that they stay
+// in either half of L2 (64 MB took 399 us).
+constexpr int64_t kHeadGroupBytes = int64_t(24) << 20;
+constexpr int64_t kHeadGroupTiles = 16 * 148;
+inline int64_t head_group(const AttnArgs& a, int D, int tiles_per_head) {
+    const int64_t heads = int64_t(a.B) * a.H, per_head = int64_t(a.N) * D * 4;
+    if (heads * tiles_per_head > kHeadGroupTiles && heads <= 65535) return 1;
+    return std::max<int64_t>(1, std::min(heads, kHeadGroupBytes / per_head));
+}
+
 template <int D, int BQ, int BK>
 inline carnator_status launch_tc(const AttnArgs& a, const CUtensorMap& mk, const CUtensorMap& mv,
                                  cudaStream_t stream, char* err, size_t errlen) {
@@ -1096,7 +1122,12 @@ inline carnator_status launch_tc(const AttnArgs& a, const CUtensorMap& mk, const
         }
         allowed.set(most, dev);
     }
-    dim3 grid(BQ == 64 ? ceil_div(a.nqb, 2) : a.nqb, a.H, a.B);
+    const unsigned tiles = unsigned(BQ == 64 ? ceil_div(a.nqb, 2) : a.nqb);      // of a head
+    dim3 grid(tiles, a.H, a.B);
+    if (D == 128) {
+        const int64_t heads = int64_t(a.B) * a.H, group = head_group(a, D, int(tiles));
+        grid = dim3(unsigned(group), tiles, unsigned((heads + group - 1) / group));
+    }
     e = launch_dependent(kern, grid, dim3(tc::kThreads), smem, stream, mk, mv, a);
     if (e != cudaSuccess) { snprintf(err, errlen, "attn_tcgen05_kernel: %s", cudaGetErrorString(e)); return CARNATOR_ERR_CUDA; }
     return CARNATOR_OK;

@@ -427,3 +427,26 @@ def test_compacted_lists_and_order(bq, bk, N, H):
         assert {tuple(o[i:i + 2]) for i in range(0, nqb, 2)} == pairs
         longest = [c[o[i:i + 2]].max() for i in range(0, nqb - 1, 2)]
         assert longest == sorted(longest, reverse=True)
+
+
+@pytest.mark.parametrize("B,H,N,bq,D", [(2, 6, 8200, 128, 128), (3, 7, 8200, 64, 64), (1, 3, 66000, 128, 128), (5, 9, 8200, 128, 128)])
+def test_heads_that_run_in_groups(B, H, N, bq, D):
+    """The tcgen05 kernel runs several heads of a small layer side by side: short last groups (5 + 5 + 2 and 11 + 10 heads), a long
+    head and a large layer whose heads run alone, against the portable kernel (its own tests compare it with the oracle)."""
+    gen = torch.Generator(device="cuda").manual_seed(N + H)
+    Q, K, V = (torch.randn((B, H, N, D), dtype=torch.bfloat16, device="cuda", generator=gen) for _ in range(3))
+    nb = -(-N // bq)
+    mask = (torch.rand((B, H, nb, nb), device="cuda", generator=gen) < 0.04).to(torch.uint8)
+    rec = (torch.rand((B, nb), device="cuda", generator=gen) < 0.02).to(torch.uint8)
+    out = []
+    for impl in (cn.IMPL_PORTABLE, cn.IMPL_AUTO):
+        shape = cn.make_shape(B, H, N, D, 0, 1, 1, N, bq, bq, Q, K, V, attn_impl=impl)
+        O = torch.full((B, H, N, D), float("nan"), dtype=torch.bfloat16, device="cuda")
+        O, L, ws = cn.sparse_attn(Q, K, V, mask, rec, shape, O=O)
+        assert cn.query_status(ws) == cn.OK
+        out.append((O.float(), L))
+    (O0, L0), (O1, L1) = out
+    # two correct executors: P and O rounded to bf16 in each, |O| below 5 here
+    assert float((O0 - O1).abs().max()) <= 2e-2 and float((O0 - O1).abs().mean()) <= 2e-3
+    fin = torch.isfinite(L0)
+    assert torch.equal(fin, torch.isfinite(L1)) and float((L0[fin] - L1[fin]).abs().max()) <= 1e-3
