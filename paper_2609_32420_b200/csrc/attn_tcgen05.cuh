@@ -35,6 +35,7 @@
 
 #include "common.cuh"
 #include "attn_portable.cuh"
+#include "attn_ring.h"
 
 namespace carnator {
 namespace tc {
@@ -42,7 +43,6 @@ namespace tc {
 constexpr int kBlock = 128;            // query rows per CTA = keys per step
 constexpr int kSBufs = 2;              // score buffers in tensor memory, one per softmax group
 constexpr int kRefSlots = 3;           // hand-over slots of the shared reference maximum
-constexpr int kStages = 3;             // ring slots for K tiles and for V tiles
 constexpr int kSoftmaxWarps = 8;       // two warpgroups taking the steps in turn
 constexpr int kThreads = (kSoftmaxWarps + 4) * 32;   // third warpgroup: two TMA producers, two MMA issuers
 constexpr int kWarpTmaK = 8, kWarpMma = 9, kWarpTmaV = 10;
@@ -72,7 +72,7 @@ __device__ __forceinline__ uint32_t mbar_try(uint32_t bar, uint32_t parity) {
         : "=r"(done) : "r"(bar), "r"(parity) : "memory");
     return done;
 }
-// Non-blocking form for polling loops: try_wait may suspend the thread for a while when the phase is not complete.
+// Non-blocking form, for a role that watches two barriers: try_wait may suspend the thread on the one it was given.
 __device__ __forceinline__ uint32_t mbar_test(uint32_t bar, uint32_t parity) {
     uint32_t done;
     asm volatile(
@@ -95,6 +95,24 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     for (uint32_t it = 0; it < (1u << 30); ++it) {
         if (sleep_ns) __nanosleep(sleep_ns);
         if (mbar_try(bar, parity)) return true;
+        if ((it & 255u) == 255u) {
+            if (*abort_flag) return false;
+            if (global_ns() - t0 > limit_ns) break;
+        }
+    }
+    *abort_flag = 1;
+    return false;
+}
+
+// Bounded wait of a producer for its ring slot, the slot of step u (attn_ring.h): bar0 is the barrier of the even steps, that
+// of the odd ones lies behind it.
+__device__ __forceinline__ bool mbar_wait_slot(uint32_t bar0, int u, volatile int* abort_flag, unsigned long long limit_ns) {
+    auto done = [&](int b, uint32_t parity) { return mbar_test(bar0 + 8 * b, parity) != 0; };
+    if (slot_is_free(u, done)) return true;
+    const unsigned long long t0 = global_ns();
+    for (uint32_t it = 0; it < (1u << 30); ++it) {
+        __nanosleep(100);
+        if (slot_is_free(u, done)) return true;
         if ((it & 255u) == 255u) {
             if (*abort_flag) return false;
             if (global_ns() - t0 > limit_ns) break;
@@ -539,7 +557,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
             int armed = -1;
             for (int i = 0; i < T; ++i) {
                 const int s = i % kStages, u = i - kStages;     // the slot is free once Q K^T of step u has completed
-                if (u >= 0 && !mbar_wait(bar_sfull(u & 1), uint32_t(u >> 1) & 1u, abortp, 100, limit)) {
+                if (u >= 0 && !mbar_wait_slot(bar_sfull(0), u, abortp, limit)) {
                     set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 1, i, place); break;
                 }
                 const int J = kPlanned ? 0 : list[i];
@@ -570,7 +588,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
             int armed = -1;
             for (int i = 0; i < T; ++i) {
                 const int s = i % kStages, u = i - kStages;     // the slot is free once P V of step u has completed
-                if (u >= 0 && !mbar_wait(bar_pvdone(u & 1), uint32_t(u >> 1) & 1u, abortp, 100, limit)) {
+                if (u >= 0 && !mbar_wait_slot(bar_pvdone(0), u, abortp, limit)) {
                     set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 2, i, place); break;
                 }
                 const int J = kPlanned ? 0 : list[i];

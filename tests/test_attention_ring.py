@@ -1,0 +1,145 @@
+"""The barriers of the tcgen05 attention kernel, every interleaving of its roles: no wait is passed before its event, and none
+is missed.  The steps' barriers and parities and the producers' rule are the kernel's own (csrc/attn_ring.h, compiled here);
+the roles' order of waits and arrivals is restated from csrc/attn_tcgen05.cuh."""
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+from paper_2609_32420_b200 import build
+
+
+@pytest.fixture(scope="module")
+def ring(tmp_path_factory):
+    d = tmp_path_factory.mktemp("ring")
+    src, lib = os.path.join(d, "ring.cpp"), os.path.join(d, "ring.so")
+    with open(src, "w") as f:
+        f.write('#include "attn_ring.h"\nusing namespace carnator::tc;\nextern "C" int bar(int i) { return step_bar(i); }\n'
+                'extern "C" int parity(int i) { return int(step_parity(i)); }\nextern "C" int stages() { return kStages; }\n'
+                '// c0, c1: phases that the two barriers have completed\n'
+                'extern "C" int slot_free(int u, int c0, int c1) { return slot_is_free(u, [=](int b, uint32_t p) { return ((b ? c1 : c0) & 1) != int(p); }); }\n')
+    subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I", build.CSRC, "-o", lib, src], check=True)
+    return ctypes.CDLL(lib)
+
+
+class Stuck(Exception):
+    pass
+
+
+class Early(Exception):
+    pass
+
+
+def explore(T, stages, bar, parity, slot_free, form, warps=1):
+    """Walks all reachable states of one block of T steps.  `bar`, `parity`: barrier of a step for "scores there" and "P V
+    done"; `slot_free`: the producers' rule.  `form`: "early" gives the scores' buffer back on reading them (64-token blocks), "late" after the reference,
+    "rescaling" like "late" with P V of the step before awaited in front of the reference, in every step.
+
+    Counters of a state: K tiles asked for / landed, V tiles asked for / landed, Q K^T issued / completed, P V issued /
+    completed, then per softmax warp (group-major) its operations done.  Each role's next operation follows from its counter."""
+    kslot, kpar = lambda i: i % stages, lambda i: (i // stages) & 1          # tiles: one barrier per ring slot
+    half, hpar = lambda i: i & 1, lambda i: (i >> 1) & 1                     # one barrier per softmax group
+    n_ops = 3                                                                # operations of a softmax warp per step (below)
+
+    def passed(at, par, done, i, event):
+        """A wait for event i of a kind whose events 0 .. done - 1 have happened, event j on barrier at(j)."""
+        c = sum(1 for j in range(done) if at(j) == at(i))                  # phases this barrier has completed
+        ok = (c & 1) != par(i)
+        if ok and i >= done:
+            raise Early(f"{event} {i} taken for done at {done}")
+        return ok
+
+    def free(done, u):
+        """A producer's wait for step u of a kind whose steps 0 .. done - 1 have completed."""
+        ok = slot_free(u, (done + 1) // 2, done // 2)
+        if ok and u >= done:
+            raise Early(f"slot of step {u} taken for free at {done}")
+        return ok
+
+    def group_done(st, g, op):
+        """Steps of group g whose operation `op` all its warps have done, as a step number: first one not done."""
+        n = min((o - op + n_ops - 1) // n_ops if o > op else 0 for o in st[8 + g * warps: 8 + (g + 1) * warps])
+        return g + 2 * n
+
+    def count(st, op):
+        """How many of steps 0, 1, 2, .. have done operation `op`, per group as separate barriers: steps below are done."""
+        return [group_done(st, g, op) for g in (0, 1)]
+
+    def group_wait(st, op, i, event):                                        # barriers indexed by the group
+        g = i & 1
+        done = (count(st, op)[g] - g) // 2                                   # phases of the group's barrier
+        ok = (done & 1) != hpar(i)
+        if ok and i // 2 >= done:
+            raise Early(f"{event} {i} taken for done")
+        return ok
+
+    def moves(st):
+        ka, kl, va, vl, qi, qd, pi, pd = st[:8]
+
+        def step(k, v=1):
+            n = list(st)
+            n[k] += v
+            return tuple(n)
+        if ka < T and (ka < stages or free(qd, ka - stages)):
+            yield step(0)
+        if kl < ka:
+            yield step(1)
+        if va < T and (va < stages or free(pd, va - stages)):
+            yield step(2)
+        if vl < va:
+            yield step(3)
+        sfree_op = 0 if form == "early" else 1
+        if qi < T and passed(kslot, kpar, kl, qi, "K tile") and (qi < 2 or group_wait(st, sfree_op, qi - 2, "scores read")):
+            yield step(4)
+        if qd < qi:
+            yield step(5)
+        if pi < T and passed(kslot, kpar, vl, pi, "V tile") and group_wait(st, 2, pi, "P"):
+            yield step(6)
+        if pd < pi:
+            yield step(7)
+        for g in (0, 1):
+            for w in range(warps):
+                k = 8 + g * warps + w
+                i, op = g + 2 * (st[k] // n_ops), st[k] % n_ops
+                if i >= T:
+                    continue
+                if op == 0:          # scores of step i are there; "early": S given back
+                    ok = passed(bar, parity, qd, i, "Q K^T")
+                elif op == 1:        # reference of step i - 1 (from the same warp of the other group), own one published; "late": S given back
+                    o = st[8 + (g ^ 1) * warps + w]
+                    refs = (o + 1) // n_ops                                  # steps of the other group with the reference published
+                    ok = i == 0 or (refs > 0 and (g ^ 1) + 2 * (refs - 1) >= i - 1)
+                    ok = ok and (form != "rescaling" or i == 0 or passed(bar, parity, pd, i - 1, "P V"))
+                else:                # P V of step i - 1 has read P; P of step i handed over
+                    ok = i == 0 or passed(bar, parity, pd, i - 1, "P V")
+                if ok:
+                    yield step(k)
+
+    start = (0,) * (8 + 2 * warps)
+    end = (T,) * 8 + tuple(n_ops * len(range(g, T, 2)) for g in (0, 1) for _ in range(warps))
+    seen, todo = {start}, [start]
+    while todo:
+        st = todo.pop()
+        nxt = list(moves(st))
+        if not nxt and st != end:
+            raise Stuck(st)
+        for n in nxt:
+            if n not in seen:
+                seen.add(n)
+                todo.append(n)
+    assert end in seen
+    return len(seen)
+
+
+@pytest.mark.parametrize("form,T,warps", [("early", 9, 1), ("late", 9, 1), ("rescaling", 9, 1), ("early", 6, 2), ("late", 6, 2)])
+def test_every_interleaving_ends_and_no_wait_is_passed_early(ring, form, T, warps):
+    assert explore(T, ring.stages(), ring.bar, ring.parity, ring.slot_free, form, warps) > 1000
+
+
+@pytest.mark.parametrize("form", ["early", "late", "rescaling"])
+def test_a_producer_that_watches_one_barrier_can_miss_its_phase(ring, form):
+    """The search finds the fault it is there for: a step and the one two steps on share a barrier."""
+    one = lambda u, c0, c1: ((c1 if u & 1 else c0) & 1) != ((u >> 1) & 1)
+    with pytest.raises(Stuck):
+        explore(6, ring.stages(), ring.bar, ring.parity, one, form)
