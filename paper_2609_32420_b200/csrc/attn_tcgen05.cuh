@@ -46,10 +46,11 @@ constexpr int kRefSlots = 3;           // hand-over slots of the shared referenc
 constexpr int kSoftmaxWarps = 8;       // two warpgroups taking the steps in turn
 constexpr int kThreads = (kSoftmaxWarps + 4) * 32;   // third warpgroup: two TMA producers, two MMA issuers
 constexpr int kWarpTmaK = 8, kWarpMma = 9, kWarpTmaV = 10;
-constexpr int kTmemCols = 512;         // S0 | S1 | P | Q | O
+constexpr int kTmemCols = 512;         // S0 | S1 | P | Q | O (| low part of P at D = 64, 64-token block forms)
 constexpr uint32_t kColP = 2 * kBlock;        // packed bf16 probabilities: 64 columns, one buffer for both groups
 constexpr uint32_t kColQ = 2 * kBlock + 64;   // the query tile as packed bf16 pairs: D / 2 columns (A operand of Q K^T)
 constexpr uint32_t kColO = 2 * kBlock + 2 * 64;
+constexpr uint32_t kColPLow = kColO + 64;     // D = 64, 64-token block forms: what is left of the probabilities (64 columns)
 constexpr int kRegsService = 72, kRegsSoftmax = 216;   // setmaxnreg targets (the literals in the kernel must match)
 constexpr float kRescaleThreshold = 8.0f;   // log2 units: P stays below 2^8, well inside bf16/fp32 range
 
@@ -416,7 +417,7 @@ __device__ __forceinline__ int build_plan(const AttnArgs& a, const int32_t* list
 //            in V) reaches it.
 //   BK = 64: a step is two listed blocks, brought by a copy each.
 // Why a union and not 64-row products: those run at half the tensor rate.  Wan-1.3B-shaped layer with 64-token blocks
-// (12 heads, 32760 tokens, 36 % of the tiles): 10.13 ms on the mma.sync kernel, 2.51 ms here; the unions hold about 15 % more
+// (12 heads, 32760 tokens, 36 % of the tiles): 10.13 ms on the mma.sync kernel, 3.60 ms here; the unions hold about 15 % more
 // tiles than the lists.
 template <int D, int BQ, int BK>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -442,6 +443,9 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
     grid_wait();                            // launched while the compaction drains
     constexpr bool kPairs = BQ == 64, kPlanned = BQ == 64 || BK == 64;
     constexpr int kPerStep = kBlock / BK;             // listed key blocks in a step
+    // The forms with 64-token blocks keep P to 16 bits, as a sum of two bf16 (see the exponentials).  Tensor memory has no
+    // columns left for the second part at D = 128: there it takes the place of the scores it was made from.
+    constexpr bool kLowInS = kPlanned && D == 128;
     const int place = kGroups ? blockIdx.y : blockIdx.x;
     const int x0 = kPairs ? 2 * place : place;
     const int I = a.order[bh * a.nqb + x0];
@@ -624,7 +628,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
         for (int iq = 0; iq < T && ok; ++iq) {
             const int s = iq % kStages, g = iq & 1;
             ok = mbar_wait_warp(bar_kfull(s), uint32_t(iq / kStages) & 1u, abortp, 0, limit);
-            if (ok && iq >= 2) ok = mbar_wait_warp(bar_sfree(g), uint32_t((iq - 2) >> 1) & 1u, abortp, 0, limit);
+            if (ok && iq >= 2) ok = mbar_wait_warp(kLowInS ? bar_pvdone(g) : bar_sfree(g), uint32_t((iq - 2) >> 1) & 1u, abortp, 0, limit);
             if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 4, iq, place); break; }
             tc_fence_after();
             // Q from tensor memory, K tile K-major, 16 elements of the head dimension per instruction
@@ -650,6 +654,14 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
         bool ok = true;
         for (int ip = 0; ip < T && ok; ++ip) {
             const int s = ip % kStages, g = ip & 1;
+            // Which rows list the step's key blocks.  Taken before the waits, with one choice between two batches: looked up per
+            // product the Wan-1.3B-shaped layer took 3.70 ms instead of 3.60, chosen per key block 3.75.
+            uint32_t e_step = 0u;
+            if (kPairs) {
+#pragma unroll
+                for (int kh = 0; kh < kPerStep; ++kh) e_step |= uint32_t(plan[ip * kPerStep + kh] >> kPlanRowBit) << (2 * kh);
+                e_step = __reduce_or_sync(0xffffffffu, e_step);
+            }
             ok = mbar_wait_warp(bar_vfull(s), uint32_t(ip / kStages) & 1u, abortp, 0, limit);
             if (ok) ok = mbar_wait_warp(bar_pfull(g), uint32_t(ip >> 1) & 1u, abortp, 0, limit);
             if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 5, ip, place); break; }
@@ -658,13 +670,22 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
             // (rows = keys, 64-element chunks of the head dimension one box apart)
             const uint32_t v_lo = v_lo0 + uint32_t(s) * (C::kTileBytes >> 4), p_t = tmem + kColP, d_o = tmem + kColO;
             const uint32_t acc0 = ip > 0 ? 1u : 0u;
+            const uint32_t low_t = tmem + (kLowInS ? uint32_t(g) * kBlock : kColPLow);
+            if (kPairs && e_step != (kPerStep == 2 ? 15u : 3u)) {      // rows that do not list a block keep what they have
 #pragma unroll
-            for (int kk = 0; kk < kBlock / 16; ++kk) {
-                if (kPairs) {       // O starts at zero; rows that do not list the block keep what they have
-                    const uint32_t e = plan[ip * kPerStep + kk / (BK / 16)] >> kPlanRowBit;
-                    mma_ts_el_rows(d_o, p_t + kk * 8, v_lo + kk * (2048 >> 4), hi_v, idesc_pv, (e & 1u) - 1u, (e >> 1) - 1u, 1u);
-                } else {
-                    mma_ts_el(d_o, p_t + kk * 8, v_lo + kk * (2048 >> 4), hi_v, idesc_pv, kk > 0 ? 1u : acc0);
+                for (int kh = 0; kh < kPerStep; ++kh) {
+                    const uint32_t off_lo = ((e_step >> (2 * kh)) & 1u) - 1u, off_hi = ((e_step >> (2 * kh + 1)) & 1u) - 1u;
+#pragma unroll
+                    for (int kk = kh * (BK / 16); kk < (kh + 1) * (BK / 16); ++kk) {
+                        mma_ts_el_rows(d_o, p_t + kk * 8, v_lo + kk * (2048 >> 4), hi_v, idesc_pv, off_lo, off_hi, 1u);
+                        mma_ts_el_rows(d_o, low_t + kk * 8, v_lo + kk * (2048 >> 4), hi_v, idesc_pv, off_lo, off_hi, 1u);
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int kk = 0; kk < kBlock / 16; ++kk) {
+                    mma_ts_el(d_o, p_t + kk * 8, v_lo + kk * (2048 >> 4), hi_v, idesc_pv, kPairs || kk > 0 ? 1u : acc0);      // kPairs: O starts at zero
+                    if (kPlanned) mma_ts_el(d_o, low_t + kk * 8, v_lo + kk * (2048 >> 4), hi_v, idesc_pv, 1u);
                 }
             }
             tc_commit_el(bar_pvdone(g));
@@ -740,8 +761,9 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
             const int nvalid = (i == T - 1) ? nvalid_last : kBlock;      // >= 1; < 128 only for a ragged last block
             const uint32_t tS = tmem + lane_base + wg * kBlock;
             const uint32_t tP = tmem + lane_base + kColP;
+            const uint32_t tLow = kLowInS ? tS : tmem + lane_base + kColPLow;
             float s[4][32];
-            uint32_t pk[4][16];
+            uint32_t pk[4][16], low[4][16];
             uint64_t part2[2];
             bool p_free;
             if constexpr (!kPlanned) {
@@ -834,8 +856,10 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
 #pragma unroll
                 for (int c = 0; c < 4; ++c) tmem_ld32(tS + c * 32, s[c]);
                 tmem_wait_ld();
-                tc_fence_before();
-                mbar_arrive_warp(bar_sfree(wg));     // the scores are in registers: S_g may take the scores of step i+2
+                if (!kLowInS) {
+                    tc_fence_before();
+                    mbar_arrive_warp(bar_sfree(wg));     // the scores are in registers: S_g may take the scores of step i+2
+                }
                 if (nvalid < kBlock) {               // ragged tail (warp-uniform): keys >= N never count
 #pragma unroll
                     for (int c = 0; c < 4; ++c)
@@ -903,13 +927,29 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
                     }
                 }
                 if (m_w != r_now) { l_w *= ex2_approx(m_w - r_now); m_w = r_now; }   // first use: l_w = 0, exp2(-inf) = 0
-                // P = exp2(s * scale - R_i): one FFMA + one MUFU per element, packed bf16 pairs over S's own columns
+                // P = exp2(s * scale - R_i), as two bf16: the upper half of the word and what that leaves.  The portable kernel,
+                // which these shapes ran on, has one bf16, but its reference is the running maximum, so that the largest weight
+                // of a row is 1 and exact.  Under a reference that lags the largest weight is rounded as well, and O comes out
+                // further from the fp64 result: relative error 1.713e-3 against 1.698e-3 on a 1024-token layer of D = 64, where
+                // the rounding of O alone is 1.654e-3; with scores three times as large the error of P is 2.4 times as large.
+                // As two bf16 it is 1.654e-3.  The second product per step costs 2.32 -> 3.60 ms on the Wan-1.3B-shaped layer.
+                // A reference without lag (2.81 ms) still came out above the portable kernel in 11 layers of 12.
                 const uint64_t neg_m2 = pack2(-r_now, -r_now), scale2 = pack2(a.scale_log2, a.scale_log2);
                 part2[0] = part2[1] = pack2(0.f, 0.f);
                 if (kPairs && !on0 && !on1) {        // warp-uniform: nothing of this step belongs to these rows (their reference may be -inf)
+                    if (!p_free) {
+                        ok = mbar_wait_warp(bar_pvdone(wg ^ 1), uint32_t((i - 1) >> 1) & 1u, abortp, 0, limit);
+                        if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 12, i, place); break; }
+                    }
+                    tc_fence_after();
+                    const uint32_t zero[32] = {};
 #pragma unroll
-                    for (int e = 0; e < 64; ++e) pk[e >> 4][e & 15] = 0u;
-                } else {
+                    for (int c = 0; c < 2; ++c) { tmem_st32(tP + c * 32, zero); tmem_st32(tLow + c * 32, zero); }
+                    tmem_wait_st();
+                    tc_fence_before();
+                    mbar_arrive_warp(bar_pfull(wg));
+                    continue;
+                }
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
 #pragma unroll
@@ -918,9 +958,11 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
                         unpack2(fma2(pack2(s[c][2 * e], s[c][2 * e + 1]), scale2, neg_m2), x0, x1);
                         const float p0 = ex2_approx(x0), p1 = ex2_approx(x1);
                         part2[e & 1] = add2(part2[e & 1], pack2(p0, p1));
-                        pk[c][e] = pack_bf16(p0, p1);
+                        const uint32_t b0 = __float_as_uint(p0), b1 = __float_as_uint(p1);
+                        pk[c][e] = __byte_perm(b0, b1, 0x7632);
+                        low[c][e] = pack_bf16(p0 - __uint_as_float(b0 & 0xFFFF0000u), p1 - __uint_as_float(b1 & 0xFFFF0000u));
                     }
-                }
+                    if (kLowInS) tmem_st16(tLow + c * 16, low[c]);    // this warp has read these rows' scores, and nobody else does
                 }
             }
             if (!p_free) {      // the one P buffer is free once P V of step i-1 (the other group's) has read it
@@ -928,7 +970,10 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
                 if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 12, i, place); break; }
             }
 #pragma unroll
-            for (int c = 0; c < 4; ++c) tmem_st16(tP + c * 16, pk[c]);
+            for (int c = 0; c < 4; ++c) {
+                tmem_st16(tP + c * 16, pk[c]);
+                if (kPlanned && !kLowInS) tmem_st16(tLow + c * 16, low[c]);
+            }
             {
                 float s0, s1, s2, s3;
                 unpack2(part2[0], s0, s1); unpack2(part2[1], s2, s3);

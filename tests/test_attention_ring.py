@@ -34,7 +34,8 @@ class Early(Exception):
 def explore(T, stages, bar, parity, slot_free, form, warps=1):
     """Walks all reachable states of one block of T steps.  `bar`, `parity`: barrier of a step for "scores there" and "P V
     done"; `slot_free`: the producers' rule.  `form`: "early" gives the scores' buffer back on reading them (64-token blocks), "late" after the reference,
-    "rescaling" like "late" with P V of the step before awaited in front of the reference, in every step.
+    "rescaling" like "late" with P V of the step before awaited in front of the reference, in every step, "low" with P V of the
+    step itself (the scores' columns hold a part of P until then).
 
     Counters of a state: K tiles asked for / landed, V tiles asked for / landed, Q K^T issued / completed, P V issued /
     completed, then per softmax warp (group-major) its operations done.  Each role's next operation follows from its counter."""
@@ -90,7 +91,8 @@ def explore(T, stages, bar, parity, slot_free, form, warps=1):
         if vl < va:
             yield step(3)
         sfree_op = 0 if form == "early" else 1
-        if qi < T and passed(kslot, kpar, kl, qi, "K tile") and (qi < 2 or group_wait(st, sfree_op, qi - 2, "scores read")):
+        if qi < T and passed(kslot, kpar, kl, qi, "K tile") and \
+                (qi < 2 or (passed(bar, parity, pd, qi - 2, "P V") if form == "low" else group_wait(st, sfree_op, qi - 2, "scores read"))):
             yield step(4)
         if qd < qi:
             yield step(5)
@@ -132,12 +134,12 @@ def explore(T, stages, bar, parity, slot_free, form, warps=1):
     return len(seen)
 
 
-@pytest.mark.parametrize("form,T,warps", [("early", 9, 1), ("late", 9, 1), ("rescaling", 9, 1), ("early", 6, 2), ("late", 6, 2)])
+@pytest.mark.parametrize("form,T,warps", [("early", 9, 1), ("late", 9, 1), ("rescaling", 9, 1), ("low", 9, 1), ("early", 6, 2), ("late", 6, 2), ("low", 6, 2)])
 def test_every_interleaving_ends_and_no_wait_is_passed_early(ring, form, T, warps):
     assert explore(T, ring.stages(), ring.bar, ring.parity, ring.slot_free, form, warps) > 1000
 
 
-@pytest.mark.parametrize("form", ["early", "late", "rescaling"])
+@pytest.mark.parametrize("form", ["early", "late", "rescaling", "low"])
 def test_a_producer_that_watches_one_barrier_can_miss_its_phase(ring, form):
     """The search finds the fault it is there for: a step and the one two steps on share a barrier."""
     one = lambda u, c0, c1: ((c1 if u & 1 else c0) & 1) != ((u >> 1) & 1)

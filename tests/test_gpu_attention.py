@@ -351,6 +351,31 @@ def test_blocks_of_64_on_the_tensor_core_kernel(D, bq, bk, N, density):
     assert cn.compacted_tiles(shape, ws) == int(eff.sum())
 
 
+@pytest.mark.parametrize("H,N,D,bq,bk,density,peak", [(2, 1024, 64, 64, 64, 0.4, 1), (22, 302, 64, 64, 64, 0.6, 1), (3, 528, 128, 64, 64, 0.5, 3),
+                                                      (2, 4700, 128, 64, 128, 0.3, 1), (2, 3471, 64, 128, 64, 0.2, 3), (2, 2288, 128, 128, 64, 0.3, 1)])
+def test_blocks_of_64_are_no_further_from_the_exact_result(H, N, D, bq, bk, density, peak):
+    """Against the same in 64 bits the tensor-core kernel is no further off than the portable one, in O and in LSE, on flat and on
+    peaked scores.  What the portable kernel rounds most finely, the largest weight of a row, must not be rounded here either."""
+    gen = torch.Generator(device="cuda").manual_seed(N + D)
+    Q, K, V = (torch.randn((1, H, N, D), dtype=torch.bfloat16, device="cuda", generator=gen) for _ in range(3))
+    Q *= peak
+    nqb, nkb = -(-N // bq), -(-N // bk)
+    mask = torch.rand((1, H, nqb, nkb), device="cuda", generator=gen) < density
+    mask[..., 0] = True
+    on = mask.repeat_interleave(bq, 2).repeat_interleave(bk, 3)[:, :, :N, :N]
+    x = (Q.double() @ K.double().transpose(2, 3) / np.sqrt(D)).masked_fill_(~on, -np.inf)
+    L_ref, O_ref = x.logsumexp(3), x.softmax(3) @ V.double()
+    err = []
+    for impl in (cn.IMPL_PORTABLE, cn.IMPL_AUTO):
+        shape = cn.make_shape(1, H, N, D, 0, 1, 1, N, bq, bk, Q, K, V, attn_impl=impl)
+        O, L, ws = cn.sparse_attn(Q, K, V, mask.to(torch.uint8), None, shape)
+        assert cn.query_status(ws) == cn.OK
+        err.append((float((O.double() - O_ref).norm()), float((L.double() - L_ref).norm())))
+    assert err[1][0] <= err[0][0], err
+    # LSE, 32-bit arithmetic in both: a few units in the last place of the largest reference
+    assert err[1][1] <= max(err[0][1], 2.0 ** -22 * float(L_ref.norm())), err
+
+
 @pytest.mark.parametrize("bk", [64, 128])
 def test_query_blocks_that_share_a_tile_do_not_see_each_others_keys(bk):
     """Two 64-token query blocks share a tile.  Infinities and NaN in the K and V of a block must reach only the rows that
