@@ -969,6 +969,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
                 ok = mbar_wait_warp(bar_pvdone(wg ^ 1), uint32_t((i - 1) >> 1) & 1u, abortp, 0, limit);
                 if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 12, i, place); break; }
             }
+            tc_fence_after();          // its reads of P come before the stores below
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 tmem_st16(tP + c * 16, pk[c]);

@@ -3,6 +3,7 @@ is missed.  The steps' barriers and parities and the producers' rule are the ker
 the roles' order of waits and arrivals is restated from csrc/attn_tcgen05.cuh."""
 import ctypes
 import os
+import re
 import subprocess
 
 import pytest
@@ -145,3 +146,17 @@ def test_a_producer_that_watches_one_barrier_can_miss_its_phase(ring, form):
     one = lambda u, c0, c1: ((c1 if u & 1 else c0) & 1) != ((u >> 1) & 1)
     with pytest.raises(Stuck):
         explore(6, ring.stages(), ring.bar, ring.parity, one, form)
+
+
+def test_every_wait_that_orders_tensor_memory_is_followed_by_a_fence():
+    """What another role's products or loads did to tensor memory is ordered before this role's accesses by the barrier and by
+    tcgen05.fence::after_thread_sync behind the wait: in the source, a fence between each such wait and the next access."""
+    with open(os.path.join(build.CSRC, "attn_tcgen05.cuh")) as f:
+        text = re.sub(r"//[^\n]*", "", f.read())
+    text = text[text.index("attn_tcgen05_kernel("):text.index("wait_timeout_selftest_kernel")]
+    waits = [m.end() for m in re.finditer(r"mbar_wait_warp\((?:kLowInS \? )?bar_(?:sfull|sfree|pvdone|pfull|q\b|o\b)", text)]
+    assert len(waits) >= 8
+    for at in waits:
+        access = re.compile(r"\b(?:tmem_ld|tmem_st|mma_ts_el|mma_ss_el)").search(text, at)
+        fence = text.find("tc_fence_after()", at)
+        assert access is None or at < fence < access.start(), text[at - 60:access.end() + 20]
