@@ -1170,8 +1170,8 @@ inline carnator_status launch_tc(const AttnArgs& a, const CUtensorMap& mk, const
     auto kern = tc::attn_tcgen05_kernel<D, BQ, BK>;
     static SmemAllowed allowed;
     cudaError_t e;
-    int dev;
-    if (!allowed.has(smem, &dev)) {      // once: with room for the longest plan
+    const unsigned long long ctx = context_id();
+    if (!allowed.has(ctx)) {             // once: with room for the longest plan
         const uint32_t most = tc::Cfg<D>::kSmemBytes + (BQ == 64 || BK == 64 ? tc::plan_bytes(tc::kPlanMaxKeyBlocks) : 0u);
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(most));
         if (e != cudaSuccess) { snprintf(err, errlen, "cudaFuncSetAttribute(tcgen05): %s", cudaGetErrorString(e)); return CARNATOR_ERR_CUDA; }
@@ -1184,7 +1184,7 @@ inline carnator_status launch_tc(const AttnArgs& a, const CUtensorMap& mk, const
             snprintf(err, errlen, "attn_tcgen05_kernel was built with %d registers per thread: too few for its setmaxnreg split", fa.numRegs);
             return CARNATOR_ERR_UNSUPPORTED;
         }
-        allowed.set(most, dev);
+        allowed.add(ctx);
     }
     const unsigned tiles = unsigned(BQ == 64 ? ceil_div(a.nqb, 2) : a.nqb);      // of a head
     dim3 grid(tiles, a.H, a.B);

@@ -117,12 +117,11 @@ template <int D, int R, int NPL>
 carnator_status launch_score_select_r(const BuildWs& w, float* scores_opt, float scale, int B, const SelectArgs& sa, cudaStream_t stream) {
     const size_t smem = score_select_smem<D, R>(sa.nkb);
     static SmemAllowed allowed;
-    int dev;
-    if (!allowed.has(smem, &dev)) {      // once, for the longest row of this form
-        const size_t most = score_select_smem<D, R>(32 * NPL);
-        carnator_status st = allow_smem(score_select_kernel<D, R, NPL>, most);
+    const unsigned long long ctx = context_id();
+    if (!allowed.has(ctx)) {      // once, for the longest row of this form
+        carnator_status st = allow_smem(score_select_kernel<D, R, NPL>, score_select_smem<D, R>(32 * NPL));
         if (st != CARNATOR_OK) return st;
-        allowed.set(most, dev);
+        allowed.add(ctx);
     }
     const cudaError_t e = launch_dependent(score_select_kernel<D, R, NPL>, dim3(ceil_div(sa.nqb, R), sa.H, B), dim3(R * 32), smem, stream,
                                            w.qbar, w.kbar, scores_opt, scale, sa);

@@ -99,20 +99,30 @@ struct Geometry {
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// How much dynamic shared memory a kernel has been allowed on each device: asking the runtime costs about a microsecond a
-// call.  One static object per kernel, at the place that launches it.
+// Number of the current CUDA context, unique for the life of the process (a reset of the device makes a new one); 0 if there
+// is none yet.
+inline unsigned long long context_id() {
+    typedef int (*CtxGetIdFn)(void*, unsigned long long*);
+    static const CtxGetIdFn fn = [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPoint("cuCtxGetId", &p, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess)
+            return reinterpret_cast<CtxGetIdFn>(p);
+        cudaGetLastError();
+        return CtxGetIdFn(nullptr);
+    }();
+    unsigned long long id = 0;
+    return fn && fn(nullptr, &id) == 0 ? id : 0;
+}
+
+// Contexts in which a kernel has been allowed the dynamic shared memory of its largest launch (an attribute of the kernel in
+// each context): asking the runtime on every call costs about a microsecond.  One static object per kernel, at the place that
+// launches it.  A context that is not in its slot is asked for again.
 struct SmemAllowed {
-    static constexpr int kDevices = 64;
-    std::atomic<uint32_t> bytes[kDevices];
-    // true if `need` is already allowed on the current device
-    bool has(size_t need, int* dev) const {
-        *dev = -1;
-        if (cudaGetDevice(dev) != cudaSuccess || *dev < 0 || *dev >= kDevices) return false;
-        return bytes[*dev].load(std::memory_order_acquire) >= need;
-    }
-    void set(size_t now, int dev) {
-        if (dev >= 0 && dev < kDevices) bytes[dev].store(uint32_t(now), std::memory_order_release);
-    }
+    static constexpr int kSlots = 16;
+    std::atomic<unsigned long long> ctx[kSlots];
+    bool has(unsigned long long id) const { return id != 0 && ctx[id % kSlots].load(std::memory_order_acquire) == id; }
+    void add(unsigned long long id) { if (id != 0) ctx[id % kSlots].store(id, std::memory_order_release); }
 };
 
 // Launch that may begin before the kernel ahead of it in the stream has ended (that kernel calls grid_launch_dependents,
