@@ -107,6 +107,8 @@ int topk_count_host(float ratio, int n) {
     return k < 1 ? 1 : (k > n ? n : k);
 }
 
+// `bytes`: what the kernel's largest launch takes, whatever this one does.  A smaller figure would lower the limit under
+// another thread that is about to launch the same kernel on a larger layer.
 template <typename K>
 carnator_status allow_smem(K kernel, size_t bytes) {
     CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)));
@@ -173,7 +175,7 @@ constexpr size_t kMaxDynamicSmem = 226 * 1024;     // 227 KiB per CTA less the k
 template <int D, int NPL, int PST, int AST>
 carnator_status launch_fused_r(const FusedArgs& fa, const CUtensorMap (&maps)[4], int nkb, int sms, cudaStream_t stream) {
     const size_t smem = FusedSmem<D, PST, AST>::bytes(nkb, fa.nkb_pad);
-    carnator_status st = allow_smem(build_fused_kernel<D, NPL, PST, AST>, smem);
+    carnator_status st = allow_smem(build_fused_kernel<D, NPL, PST, AST>, kMaxDynamicSmem);
     if (st != CARNATOR_OK) return st;
     // the register hand-over inside the kernel (setmaxnreg) only completes if the CTA owns 256 x 40 + 512 x 96 registers
     cudaFuncAttributes attr;
@@ -461,7 +463,7 @@ static carnator_status compact_impl(const uint8_t* mask, const uint8_t* recomput
     const size_t smem = compact_smem(nqb, pairs);
     auto kern = pairs ? compact_order_kernel<true> : compact_order_kernel<false>;
     if (smem > 48 * 1024) {
-        st = allow_smem(kern, smem);
+        st = allow_smem(kern, compact_smem(kMaxQueryBlocks, pairs));
         if (st != CARNATOR_OK) return st;
     }
     cudaLaunchAttribute at[2];

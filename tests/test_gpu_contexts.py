@@ -75,3 +75,73 @@ def test_a_second_context_on_the_device():
     """What a kernel was allowed in one context (dynamic shared memory) it has not been allowed in another."""
     r = subprocess.run([sys.executable, "-c", TWO_CONTEXTS], cwd=ROOT, capture_output=True, text=True, timeout=300, env=dict(os.environ, PYTHONPATH=ROOT))
     assert r.returncode == 0 and "same outputs" in r.stdout, r.stdout + r.stderr
+
+
+# n calls in a row without coming back to Python, whose lock would keep the two threads apart
+LOOPS = r"""
+#include "carnator.h"
+extern "C" int compaction(decltype(&carnator_compact_mask) f, const uint8_t* mask, const carnator_shape* s, void* ws, size_t bytes, void* stream, int n) {
+    for (int i = 0; i < n; ++i) if (int st = f(mask, nullptr, s, ws, bytes, stream)) return st;
+    return 0;
+}
+extern "C" int builder(decltype(&carnator_build_connectivity) f, const void* Q, const void* K, const carnator_shape* s, const carnator_build_params* p,
+                       uint8_t* mask, void* ws, size_t bytes, void* stream, int n) {
+    for (int i = 0; i < n; ++i) if (int st = f(Q, K, s, p, mask, nullptr, ws, bytes, stream)) return st;
+    return 0;
+}
+"""
+
+
+@pytest.mark.parametrize("call", ["compaction", "builder"])
+def test_two_threads_with_layers_of_different_size(call, tmp_path):
+    """Kernels whose shared memory grows with the layer: one thread's smaller layer must not take back what another thread's
+    larger one is about to be launched with."""
+    import ctypes
+    import threading
+
+    import torch
+
+    from paper_2609_32420_b200 import build
+    from paper_2609_32420_b200 import carnator as cn
+    src, lib = tmp_path / "loops.cpp", tmp_path / "loops.so"
+    src.write_text(LOOPS)
+    subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-I", build.INCLUDE, "-o", str(lib), str(src)], check=True)
+    loops = ctypes.CDLL(str(lib))
+    vp, n = ctypes.c_void_p, 400
+    entry = lambda f: ctypes.cast(f, vp)
+
+    def compaction(nqb, stream):        # 64-token query blocks: 10 bytes of shared memory a row, above the 48 KB that need no leave
+        shape = cn.make_shape(1, 1, nqb * 64, 64, 0, 1, 1, nqb * 64, 64, 128)
+        mask = torch.ones((1, 1, shape.nqb, shape.nkb), dtype=torch.uint8, device="cuda")
+        ws = torch.empty(cn.attn_workspace_bytes(shape), dtype=torch.uint8, device="cuda")
+        held = (mask, ws, shape)
+        return held, lambda: loops.compaction(entry(cn.lib().carnator_compact_mask), vp(mask.data_ptr()), ctypes.byref(shape), vp(ws.data_ptr()),
+                                              ctypes.c_size_t(ws.numel()), vp(stream.cuda_stream), n)
+
+    def builder(nb, stream):            # the persistent builder: a row of scores per query block of an item
+        N = nb * 128
+        Q, K = (torch.randn((1, 16, N, 64), device="cuda").to(torch.bfloat16) for _ in range(2))
+        shape = cn.make_shape(1, 16, N, 64, 0, 1, 1, N, 128, 128, Q, K)
+        p = cn.BuildParams()
+        p.mode, p.keep_ratio, p.mass, p.window_frames, p.count_includes_forced = cn.MODE_TOPK, 0.2, 0.5, -1, 1
+        mask = torch.empty((1, 16, nb, nb), dtype=torch.uint8, device="cuda")
+        ws = torch.empty(cn.build_workspace_bytes(shape, p), dtype=torch.uint8, device="cuda")
+        held = (Q, K, mask, ws, shape, p)
+        return held, lambda: loops.builder(entry(cn.lib().carnator_build_connectivity), vp(Q.data_ptr()), vp(K.data_ptr()), ctypes.byref(shape),
+                                           ctypes.byref(p), vp(mask.data_ptr()), vp(ws.data_ptr()), ctypes.c_size_t(ws.numel()), vp(stream.cuda_stream), n)
+    make, sizes = (compaction, (5200, 4950)) if call == "compaction" else (builder, (320, 260))
+    streams = [torch.cuda.Stream() for _ in sizes]
+    jobs = [make(nb, s) for nb, s in zip(sizes, streams)]
+    torch.cuda.synchronize()
+    status = [None, None]
+
+    def work(i):
+        torch.cuda.set_device(0)
+        status[i] = jobs[i][1]()
+    threads = [threading.Thread(target=work, args=(i,)) for i in (0, 1)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert status == [0, 0], (status, cn.last_cuda_error())
