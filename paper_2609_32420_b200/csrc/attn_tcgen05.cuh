@@ -1174,12 +1174,12 @@ inline carnator_status launch_tc(const AttnArgs& a, const CUtensorMap& mk, const
     if (!allowed.has(ctx)) {             // once: with room for the longest plan
         const uint32_t most = tc::Cfg<D>::kSmemBytes + (BQ == 64 || BK == 64 ? tc::plan_bytes(tc::kPlanMaxKeyBlocks) : 0u);
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(most));
-        if (e != cudaSuccess) { snprintf(err, errlen, "cudaFuncSetAttribute(tcgen05): %s", cudaGetErrorString(e)); return CARNATOR_ERR_CUDA; }
+        if (e != cudaSuccess) return cuda_error(e, "cudaFuncSetAttribute(tcgen05)", err, errlen);
         // The register hand-over inside the kernel only completes if the CTA owns enough registers: check what the
         // compiler allocated instead of finding out on the device.
         cudaFuncAttributes fa;
         e = cudaFuncGetAttributes(&fa, kern);
-        if (e != cudaSuccess) { snprintf(err, errlen, "cudaFuncGetAttributes(tcgen05): %s", cudaGetErrorString(e)); return CARNATOR_ERR_CUDA; }
+        if (e != cudaSuccess) return cuda_error(e, "cudaFuncGetAttributes(tcgen05)", err, errlen);
         if (fa.numRegs * tc::kThreads < tc::kSoftmaxWarps * 32 * tc::kRegsSoftmax + 128 * tc::kRegsService) {
             snprintf(err, errlen, "attn_tcgen05_kernel was built with %d registers per thread: too few for its setmaxnreg split", fa.numRegs);
             return CARNATOR_ERR_UNSUPPORTED;
@@ -1193,7 +1193,7 @@ inline carnator_status launch_tc(const AttnArgs& a, const CUtensorMap& mk, const
         grid = dim3(unsigned(group), tiles, unsigned((heads + group - 1) / group));
     }
     e = launch_dependent(kern, grid, dim3(tc::kThreads), smem, stream, mk, mv, a);
-    if (e != cudaSuccess) { snprintf(err, errlen, "attn_tcgen05_kernel: %s", cudaGetErrorString(e)); return CARNATOR_ERR_CUDA; }
+    if (e != cudaSuccess) return cuda_error(e, "attn_tcgen05_kernel", err, errlen);
     return CARNATOR_OK;
 }
 

@@ -249,7 +249,7 @@ inline carnator_status launch_block_mass(const void* Q, const void* K, const int
     {   // the kernel's setmaxnreg split (40 / 232) needs 168 registers per thread at launch
         cudaFuncAttributes fa;
         e = (D == 128) ? cudaFuncGetAttributes(&fa, tc::block_mass_kernel<128>) : cudaFuncGetAttributes(&fa, tc::block_mass_kernel<64>);
-        if (e != cudaSuccess) { snprintf(err, errlen, "cudaFuncGetAttributes(block_mass): %s", cudaGetErrorString(e)); return CARNATOR_ERR_CUDA; }
+        if (e != cudaSuccess) return cuda_error(e, "cudaFuncGetAttributes(block_mass)", err, errlen);
         if (fa.numRegs * tc::kMassThreads < tc::kMassSoftmaxWarps * 32 * 232 + 128 * 40) {
             snprintf(err, errlen, "block_mass_kernel was built with %d registers per thread: too few for its setmaxnreg split", fa.numRegs);
             return CARNATOR_ERR_UNSUPPORTED;
@@ -263,7 +263,7 @@ inline carnator_status launch_block_mass(const void* Q, const void* K, const int
         if (e == cudaSuccess) tc::block_mass_kernel<64><<<grid, tc::kMassThreads, tc::MassCfg<64>::kSmemBytes, stream>>>(mq, mk, a);
     }
     if (e == cudaSuccess) e = cudaGetLastError();
-    if (e != cudaSuccess) { snprintf(err, errlen, "block_mass_kernel: %s", cudaGetErrorString(e)); return CARNATOR_ERR_CUDA; }
+    if (e != cudaSuccess) return cuda_error(e, "block_mass_kernel", err, errlen);
     return CARNATOR_OK;
 }
 

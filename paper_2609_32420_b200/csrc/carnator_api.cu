@@ -26,10 +26,7 @@ namespace {
 std::atomic<long long> g_launches{0};
 thread_local char g_cuda_error[256] = "";
 
-carnator_status cuda_fail(cudaError_t e, const char* where) {
-    snprintf(g_cuda_error, sizeof(g_cuda_error), "%s: %s", where, cudaGetErrorString(e));
-    return CARNATOR_ERR_CUDA;
-}
+carnator_status cuda_fail(cudaError_t e, const char* where) { return cuda_error(e, where, g_cuda_error, sizeof(g_cuda_error)); }
 
 #define CUDA_TRY(expr)                                              \
     do {                                                            \

@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
+#include <stdio.h>
 #include <atomic>
 
 #include "carnator.h"
@@ -98,6 +99,14 @@ struct Geometry {
 // Programmatic dependent launch: the next kernel of a call starts while this one drains, and waits here for its results.
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Notes a failed runtime call and takes it out of the runtime's record of the last error: it is reported here, and the next
+// call's launch check must not find it again.
+inline carnator_status cuda_error(cudaError_t e, const char* where, char* err, size_t errlen) {
+    snprintf(err, errlen, "%s: %s", where, cudaGetErrorString(e));
+    cudaGetLastError();
+    return CARNATOR_ERR_CUDA;
+}
 
 // Number of the current CUDA context, unique for the life of the process (a reset of the device makes a new one); 0 if there
 // is none yet.

@@ -272,13 +272,13 @@ inline carnator_status launch_seed_tc(const tc::SeedGatherArgs& ga, const tc::Se
     dim3 ggrid((tc::kSeedCap * (D / 8) + 255) / 256, a.H, a.B);
     tc::seed_gather_kernel<D><<<ggrid, 256, 0, stream>>>(ga);
     cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) { snprintf(err, errlen, "seed_gather_kernel: %s", cudaGetErrorString(e)); return CARNATOR_ERR_CUDA; }
+    if (e != cudaSuccess) return cuda_error(e, "seed_gather_kernel", err, errlen);
     auto kern = tc::seed_expand_tc_kernel<D>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::kSmemBytes));
-    if (e != cudaSuccess) { snprintf(err, errlen, "cudaFuncSetAttribute(seed tcgen05): %s", cudaGetErrorString(e)); return CARNATOR_ERR_CUDA; }
+    if (e != cudaSuccess) return cuda_error(e, "cudaFuncSetAttribute(seed tcgen05)", err, errlen);
     const int grid = a.tiles < sms ? a.tiles : sms;
     e = launch_dependent(kern, dim3(grid), dim3(tc::kSeedThreads), C::kSmemBytes, stream, mq, ms, a);
-    if (e != cudaSuccess) { snprintf(err, errlen, "seed_expand_tc_kernel: %s", cudaGetErrorString(e)); return CARNATOR_ERR_CUDA; }
+    if (e != cudaSuccess) return cuda_error(e, "seed_expand_tc_kernel", err, errlen);
     return CARNATOR_OK;
 }
 

@@ -145,3 +145,27 @@ def test_two_threads_with_layers_of_different_size(call, tmp_path):
         t.join()
     torch.cuda.synchronize()
     assert status == [0, 0], (status, cn.last_cuda_error())
+
+
+def test_a_refused_launch_does_not_fail_the_next_call():
+    """More heads than a grid has rows: the runtime refuses the launch and the call says so.  The next call, a good one, must
+    not report that error again."""
+    import torch
+
+    from paper_2609_32420_b200 import carnator as cn
+    H, N, D = 70000, 64, 64             # heads that share their tokens, one row of 64 apart
+    x = torch.randn((N + H, D), device="cuda").to(torch.bfloat16)
+    t = x.as_strided((1, H, N, D), (D * (N + H), D, D, 1))
+    shape = cn.make_shape(1, H, N, D, 0, 1, 1, N, 64, 64, t, t, t, t)
+    mask = torch.ones((1, H, 1, 1), dtype=torch.uint8, device="cuda")
+    L = torch.empty((1, H, N), device="cuda")
+    O = torch.empty_like(x).as_strided((1, H, N, D), t.stride())
+    with pytest.raises(cn.CarnatorError) as e:
+        cn.sparse_attn(t, t, t, mask, None, shape, O=O, LSE=L)
+    assert e.value.status == cn.ERR_CUDA
+    Q = torch.randn((1, 2, 512, D), device="cuda").to(torch.bfloat16)
+    shape = cn.make_shape(1, 2, 512, D, 0, 1, 1, 512, 128, 128, Q, Q)
+    p = cn.BuildParams()
+    p.mode, p.keep_ratio, p.mass, p.window_frames, p.count_includes_forced = cn.MODE_TOPK, 0.5, 0.5, -1, 1
+    m, _ = cn.build_connectivity(Q, Q, shape, p)
+    assert int(m.sum()) == 2 * 4 * 2
