@@ -1002,8 +1002,9 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
             const float r_fin = fmaxf(m0, m1);
             float l_tot = fin[0][1][r_loc] * ex2_approx(m0 - r_fin) + fin[1][1][r_loc] * ex2_approx(m1 - r_fin);
             if (kPairs && (second ? T2 : T1) <= 0) l_tot = 0.f;
-            // rows of a pair that list nothing: O = 0, LSE = -inf
-            const float inv = !kPairs || l_tot > 0.f ? 1.f / l_tot : 0.f;
+            // rows of a pair that list nothing: O = 0, LSE = -inf; a row whose sum is NaN: LSE = -inf in the forms with 64-token
+            // blocks, as the portable kernel has it, and NaN in that of 128
+            const float inv = !kPlanned || l_tot > 0.f ? 1.f / l_tot : 0.f;
             // each group writes half of the head dimension
             const int eb = kGroups ? at_b : b, eh = kGroups ? at_h : h;
             __nv_bfloat16* op = a.O + eb * a.os[0] + eh * a.os[1] + int64_t(row) * a.os[2] + wg * (D / 2);
@@ -1024,7 +1025,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
                     }
                 }
             }
-            if (wg == 0 && row_in) a.LSE[(int64_t(eb) * a.H + eh) * a.N + row] = !kPairs || l_tot > 0.f ? (r_fin + log2f(l_tot)) * kLn2 : -INFINITY;
+            if (wg == 0 && row_in) a.LSE[(int64_t(eb) * a.H + eh) * a.N + row] = !kPlanned || l_tot > 0.f ? (r_fin + log2f(l_tot)) * kLn2 : -INFINITY;
         }
     }
 

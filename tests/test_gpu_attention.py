@@ -475,3 +475,23 @@ def test_heads_that_run_in_groups(B, H, N, bq, D):
     assert float((O0 - O1).abs().max()) <= 2e-2 and float((O0 - O1).abs().mean()) <= 2e-3
     fin = torch.isfinite(L0)
     assert torch.equal(fin, torch.isfinite(L1)) and float((L0[fin] - L1[fin]).abs().max()) <= 1e-3
+
+
+@pytest.mark.parametrize("D,bq,bk", [(64, 64, 64), (128, 64, 128), (64, 128, 64), (128, 128, 64)])
+def test_rows_with_nan_come_out_alike_on_both_kernels(D, bq, bk):
+    """A NaN in a query reaches that query's output and nothing else; its LSE is -inf, as the portable kernel has it (a sum that
+    is not positive), for every form with 64-token blocks."""
+    rng = np.random.default_rng(D + bq)
+    N = 300
+    Q, K, V = (to_dev(rand_bits(rng, (1, 1, N, D))) for _ in range(3))
+    Q[0, 0, [0, 70, 299], 3] = float("nan")
+    mask = torch.ones((1, 1, -(-N // bq), -(-N // bk)), dtype=torch.uint8, device="cuda")
+    out = []
+    for impl in (cn.IMPL_PORTABLE, cn.IMPL_AUTO):
+        shape = cn.make_shape(1, 1, N, D, 0, 1, 1, N, bq, bk, Q, K, V, attn_impl=impl)
+        O, L, ws = cn.sparse_attn(Q, K, V, mask, None, shape)
+        assert cn.query_status(ws) == cn.OK
+        out.append((O.float(), L))
+    (O0, L0), (O1, L1) = out
+    assert torch.equal(O0.isnan(), O1.isnan()) and int(O1.isnan().any(-1).sum()) == 3
+    assert torch.equal(L0.isneginf(), L1.isneginf()) and torch.equal(L0.isnan(), L1.isnan())
