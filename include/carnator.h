@@ -195,7 +195,9 @@ carnator_status carnator_sparse_attn(const void* Q, const void* K, const void* V
                                      void* ws, size_t ws_bytes, void* stream);
 
 /* Number of evaluated (query block, key block) pairs after compaction, summed over
- * all heads.  Synchronises `stream`.  *tiles is a HOST pointer. */
+ * all heads.  Synchronises `stream`.  *tiles is a HOST pointer.  The sum is taken on
+ * the device and passes through a field of the header in `ws` that nothing else
+ * reads; lists, counts, order and status are left as they are. */
 carnator_status carnator_compacted_tiles(const carnator_shape* shape, const void* ws, size_t ws_bytes,
                                          void* stream, int64_t* tiles);
 

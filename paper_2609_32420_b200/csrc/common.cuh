@@ -19,7 +19,7 @@ constexpr unsigned long long kDefaultWaitNs = 2000000000ull;   // limit of a bou
 struct WsHeader {
     int32_t status;              // carnator_status set by kernels (0 = ok); first error wins
     int32_t info[3];             // where a bounded wait gave up / which check failed
-    unsigned long long tiles;    // evaluated (query block, key block) pairs after compaction
+    unsigned long long tiles;    // evaluated (query block, key block) pairs, written by carnator_compacted_tiles
     int32_t work[4];             // work-item counters of persistent kernels (zeroed with the header)
     unsigned long long wait_limit_ns;   // 0: the default limit of every bounded device-side wait; tests set a short one
     int32_t debug_withhold;      // 0 except in the test of the time-out path: the K producer withholds one copy
