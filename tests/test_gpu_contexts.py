@@ -169,3 +169,37 @@ def test_a_refused_launch_does_not_fail_the_next_call():
     p.mode, p.keep_ratio, p.mass, p.window_frames, p.count_includes_forced = cn.MODE_TOPK, 0.5, 0.5, -1, 1
     m, _ = cn.build_connectivity(Q, Q, shape, p)
     assert int(m.sum()) == 2 * 4 * 2
+
+
+FIRST_CALL = r"""
+import threading, torch
+from paper_2609_32420_b200 import carnator as cn
+n, N, D = 16, 512, 64
+x = torch.randn((1, 1, N, D), device="cuda").to(torch.bfloat16)
+shapes = [cn.make_shape(1, 1, N, D, 0, 1, 1, N, 128, 128, x, x, x) for _ in range(n)]
+spaces = [cn.compact_mask(torch.ones((1, 1, 4, 4), dtype=torch.uint8, device="cuda"), None, s) for s in shapes]
+out = [(torch.empty_like(x), torch.empty((1, 1, N), device="cuda")) for _ in range(n)]
+torch.cuda.synchronize()
+gate, failed = threading.Barrier(n), []
+def work(i):
+    torch.cuda.set_device(0)
+    gate.wait()
+    try:
+        cn.sparse_attn_compacted(x, x, x, shapes[i], spaces[i], O=out[i][0], LSE=out[i][1])
+    except Exception as e:
+        failed.append(str(e))
+threads = [threading.Thread(target=work, args=(i,)) for i in range(n)]
+[t.start() for t in threads]
+[t.join() for t in threads]
+torch.cuda.synchronize()
+assert not failed, failed
+assert all(torch.equal(o, out[0][0]) for o, _ in out)
+print("all alike")
+"""
+
+
+def test_first_calls_of_many_threads():
+    """The driver's tensor-map function is looked up by the first call that needs it; a call that comes during the look-up waits
+    for it.  A process of its own: the look-up happens once."""
+    r = subprocess.run([sys.executable, "-c", FIRST_CALL], cwd=ROOT, capture_output=True, text=True, timeout=300, env=dict(os.environ, PYTHONPATH=ROOT))
+    assert r.returncode == 0 and "all alike" in r.stdout, r.stdout + r.stderr
