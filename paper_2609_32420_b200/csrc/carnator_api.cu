@@ -128,9 +128,12 @@ carnator_status launch_score_select_r(const BuildWs& w, float* scores_opt, float
     return e == cudaSuccess ? CARNATOR_OK : cuda_fail(e, "score_select_kernel");
 }
 // Sixteen rows a CTA, unless that leaves SMs without one (twice over, so that a CTA's loads run under another's selection).
+// Rows of more than 640 blocks (32 keys a lane) fill an SM's registers with one CTA of eight rows, so there eight only as long
+// as no SM gets a second CTA: 2 heads of 900 blocks, D = 128, top-k, eight rows 74.3 us, sixteen 63.2; 1 head 41.4 and 57.7.
 template <int D, int NPL>
 carnator_status launch_score_select_d(const BuildWs& w, float* scores_opt, float scale, int B, const SelectArgs& sa, int sms, cudaStream_t stream) {
-    if (int64_t(B) * sa.H * ceil_div(sa.nqb, 16) < 2 * int64_t(sms)) return launch_score_select_r<D, 8, NPL>(w, scores_opt, scale, B, sa, stream);
+    const int64_t heads = int64_t(B) * sa.H;
+    if (NPL > 20 ? heads * ceil_div(sa.nqb, 8) <= sms : heads * ceil_div(sa.nqb, 16) < 2 * int64_t(sms)) return launch_score_select_r<D, 8, NPL>(w, scores_opt, scale, B, sa, stream);
     return launch_score_select_r<D, 16, NPL>(w, scores_opt, scale, B, sa, stream);
 }
 carnator_status launch_score_select(const BuildWs& w, float* scores_opt, float scale, int B, int D, const SelectArgs& sa, int sms, cudaStream_t stream) {
@@ -150,7 +153,7 @@ constexpr int kMaxKeyBlocksInRegisters = 32 * 32;     // a selecting warp holds 
 }  // namespace
 
 namespace {
-// Testing aid: 0 = choose by size, 1 = always the three kernels (pool, score, select), 2 = the persistent kernel
+// Testing aid: 0 = choose by size, 1 = always the separate kernels (pool, score and select), 2 = the persistent kernel
 // wherever it supports the shape; so that the two paths can be compared on any input.
 std::atomic<int> g_builder_path{0};
 
@@ -272,7 +275,7 @@ extern "C" carnator_status carnator_build_connectivity(const void* Q, const void
     sa.g.bq = s->block_q; sa.g.bk = s->block_k; sa.g.window = p->window_frames; sa.g.text_dense = p->text_dense;
 
     // The persistent kernel pays off once its scoring items fill the machine (its last items run after the pooling has
-    // ended); smaller layers take the three kernels.
+    // ended); smaller layers take the separate kernels: two up to 1024 key blocks, three beyond.
     int sms = 0;
     st = sm_count(&sms);
     if (st != CARNATOR_OK) return st;
