@@ -387,7 +387,7 @@ def attention_leg(D, w, n, inputs=None, keep=None):
            "frac_of_bf16_sustained": tflops / D.peaks["bf16_sustained"],
            "mufu_bound_ms": mufu, "frac_of_mufu_bound": (mufu / ms_attn) if mufu else None,
            "builder_gbs": qk_bytes / (ms_build * 1e-3) / 1e9, "builder_frac_of_hbm": qk_bytes / (ms_build * 1e-3) / 1e9 / D.peaks["hbm"],
-           "executor": "tcgen05" if D.impl != D.cn.IMPL_PORTABLE else "portable (mma.sync)",
+           "executor": "tcgen05" if D.impl != D.cn.IMPL_PORTABLE and (w.block == 128 or w.nkb <= 12288) else "portable (mma.sync)",
            "clocks": clocks}
     return out, inputs
 

@@ -175,7 +175,8 @@ carnator_status carnator_build_connectivity_exact(const void* Q, const void* K, 
  *
  * carnator_compact_mask writes, per (b,h,I), the ascending list of key blocks to
  * evaluate and its length, and per (b,h) an execution order of the query blocks
- * (longest list first).
+ * (longest list first; 64-token query blocks in pairs of like lists, longest pair
+ * first).
  * ------------------------------------------------------------------------ */
 size_t carnator_attn_workspace_bytes(const carnator_shape* shape);
 
@@ -405,7 +406,7 @@ carnator_status carnator_query_status(void* ws, void* stream);
 carnator_status carnator_selftest_wait_timeout(void* ws, uint64_t limit_ns, void* stream);
 
 /* Testing aid: which path carnator_build_connectivity takes in top-k mode.  0 = by size (the default), 1 = always
- * the three separate kernels (pool, score, select), 2 = the persistent fused kernel wherever it supports the shape.
+ * separate kernels (pool, then score and select in one up to 1024 key blocks and in two beyond), 2 = the persistent fused kernel wherever it supports the shape.
  * Both compute the same pooled scores up to the order of the fp32 sums.  Process-wide. */
 void            carnator_debug_set_builder_path(int32_t path);
 const char*     carnator_status_string(carnator_status s);

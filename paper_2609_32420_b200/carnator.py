@@ -343,7 +343,7 @@ BUILDER_AUTO, BUILDER_THREE_KERNELS, BUILDER_FUSED = 0, 1, 2
 
 
 def debug_set_builder_path(path: int) -> None:
-    """Testing aid: 0 = by size, 1 = three kernels, 2 = the fused persistent kernel where the shape allows it."""
+    """Testing aid: 0 = by size, 1 = the separate kernels, 2 = the fused persistent kernel where the shape allows it."""
     lib().carnator_debug_set_builder_path(int(path))
 
 

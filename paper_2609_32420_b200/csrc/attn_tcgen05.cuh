@@ -1,6 +1,7 @@
 // Block-sparse attention on the 5th-generation tensor cores: TMA loads of the listed K/V tiles,
 // tcgen05.mma with S = Q K^T and O += P V accumulated in tensor memory, online softmax in the
-// consumer warps.  One CTA per (batch, head, query block) of 128 queries; key blocks of 128.
+// consumer warps.  One CTA per 128 queries, a query block of 128 or a pair of 64; steps of 128 keys, one key block or two
+// (the forms with 64-token blocks are described at the kernel).
 // Paper: Section 3.3, "Historical Sparse-Connectivity Reuse" (only the block pairs the historical
 // structure lists are evaluated; Q, K, V are the target's own).
 //
@@ -25,7 +26,7 @@
 // softmax groups (straight from global memory) and serves as the A operand of every Q K^T, so those products
 // read only the K tile from shared memory, whose bandwidth the TMA writes and the operand reads share.  A group
 // signals when it no longer needs its scores in tensor memory, so Q K^T of its next step runs underneath its own
-// exponentials; it keeps its probabilities in registers until they are complete and stores them in one go, by
+// exponentials (not where the scores' columns hold a part of P, see kLowInS); it keeps its probabilities in registers until they are complete and stores them in one go, by
 // which time P V of the previous step has long read the one P buffer.  P V is issued in step order.
 // Every wait on an mbarrier is bounded; on expiry the role records CARNATOR_ERR_DEVICE_TIMEOUT in
 // the workspace header, raises a CTA-wide abort flag, and every role drains and returns.
@@ -172,31 +173,8 @@ __device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t adesc, uint64_t
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
         ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
 }
-// D[tmem] (+)= A[tmem] * B[smem]
-__device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
-}
-// Same with the descriptors given as (low word, shared high word): the issuing thread keeps the low words in
-// registers and only adds a constant per instruction, which keeps its dependent instruction chain short.
-__device__ __forceinline__ void mma_ss_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %5, 0;\n\t"
-        "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate) : "memory");
-}
-__device__ __forceinline__ void mma_ts_lo(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t.reg .b64 db;\n\tsetp.ne.b32 p, %5, 0;\n\t"
-        "mov.b64 db, {%2, %3};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate) : "memory");
-}
-// Forms for a converged warp: every lane executes the statement with the same operands and one elected lane issues
-// the instruction.  The compiler can then keep the descriptors in uniform registers, and queuing a batch costs the
+// Forms for a converged warp, the descriptors given as (low word, shared high word): D[tmem] (+)= A[tmem] * B[smem].  Every lane
+// executes the statement with the same operands and one elected lane issues the instruction.  The compiler can then keep the descriptors in uniform registers, and queuing a batch costs the
 // warp far fewer issue slots than it does from inside a one-lane branch: measured with two softmax groups running on
 // the same SM, 54 clk per instruction against 79.
 __device__ __forceinline__ void mma_ts_el(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc, uint32_t accumulate) {

@@ -10,7 +10,7 @@
 
 namespace carnator {
 
-constexpr int kMaxKeyBlocksBuilder = 4096;   // select kernel sorts one row in shared memory
+constexpr int kMaxKeyBlocksBuilder = 4096;   // rows above 1024 blocks are sorted in shared memory (mass) or held 128 keys a lane (top-k)
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr unsigned long long kDefaultWaitNs = 2000000000ull;   // limit of a bounded device-side wait unless the header says otherwise
@@ -34,7 +34,7 @@ __host__ __device__ inline int ceil_div(int a, int b) { return (a + b - 1) / b; 
 struct AttnWs {
     WsHeader* hdr;
     int32_t* counts;   // [B,H,nqb]   number of listed key blocks of each query block
-    int32_t* order;    // [B,H,nqb]   query blocks of a head, longest list first
+    int32_t* order;    // [B,H,nqb]   query blocks of a head, longest list first; of 64 tokens: pairs, longest pair first
     int32_t* lists;    // [B,H,nqb,nkb] ascending key-block indices, first counts[...] entries valid
     size_t bytes;
 };
