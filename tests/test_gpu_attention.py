@@ -254,6 +254,38 @@ def test_malformed_lists_are_reported_and_the_context_stays_usable(impl, fault):
     check_attention(o_to_host(O), L.cpu().numpy(), O_ref, L_ref, "after a reported list fault")
 
 
+@pytest.mark.parametrize("D,bq,bk", [(128, 64, 64), (64, 64, 128), (128, 128, 64)])
+@pytest.mark.parametrize("fault", ["index", "order", "count", "second_count"])
+def test_malformed_lists_of_64_token_blocks_are_reported(D, bq, bk, fault):
+    """The same for the forms with 64-token blocks, which read the lists into a plan first: the faulty list is the second one of
+    a pair where there are pairs."""
+    rng = np.random.default_rng(23)
+    B, H, N = 1, 1, 512
+    Qb, Kb, Vb = (rand_bits(rng, (B, H, N, D)) for _ in range(3))
+    Q, K, V = to_dev(Qb), to_dev(Kb), to_dev(Vb)
+    nq, nk = N // bq, N // bk
+    shape = cn.make_shape(B, H, N, D, 0, 1, 1, N, bq, bk, Q, K, V)
+    mask = torch.ones((B, H, nq, nk), dtype=torch.uint8, device="cuda")
+    ws = cn.compact_mask(mask, None, shape)
+    al = lambda x: (x + 255) // 256 * 256
+    counts = ws[256: 256 + 4 * nq].view(torch.int32)
+    lists = ws[256 + 2 * al(4 * nq):][: 4 * nq * nk].view(torch.int32).view(nq, nk)
+    assert counts.tolist() == [nk] * nq and lists[1].tolist() == list(range(nk))
+    if fault == "index":
+        lists[1, 1] = 1_000_000
+    elif fault == "order":
+        lists[1, 2] = 0
+    else:
+        counts[1 if fault == "second_count" else 0] = nk + 5
+    cn.sparse_attn_compacted(Q, K, V, shape, ws)
+    assert cn.query_status(ws) == cn.ERR_DEVICE_CHECK
+    ws = cn.compact_mask(mask, None, shape, ws=ws)
+    O, L = cn.sparse_attn_compacted(Q, K, V, shape, ws)
+    assert cn.query_status(ws) == cn.OK
+    O_ref, L_ref = orc.attention_full(Qb, Kb, Vb, N, bq, bk, 1.0 / np.sqrt(D), mask.cpu().numpy(), None)
+    check_attention(o_to_host(O), L.cpu().numpy(), O_ref, L_ref, "after a reported list fault")
+
+
 def test_bounded_wait_runs_out_and_reports_a_timeout():
     """The wait helper of the kernels on a barrier that nothing arms, limit 1 ms: the kernel must return by itself with
     CARNATOR_ERR_DEVICE_TIMEOUT in the header, and the device must work afterwards."""
@@ -295,6 +327,27 @@ def test_withheld_tile_makes_the_attention_kernel_time_out_drain_and_return():
     O, L = cn.sparse_attn_compacted(Q, K, V, shape, ws)
     assert cn.query_status(ws) == cn.OK
     O_ref, L_ref = orc.attention_full(Qb, Kb, Vb, N, 128, 128, 1.0 / np.sqrt(D), mask.cpu().numpy(), None)
+    check_attention(o_to_host(O), L.cpu().numpy(), O_ref, L_ref, "after a reported time-out")
+
+
+@pytest.mark.parametrize("D,bq,bk", [(128, 64, 64), (64, 64, 64), (128, 128, 64)])
+def test_withheld_tile_in_the_forms_with_64_token_blocks(D, bq, bk):
+    """The same for the forms with 64-token blocks, whose roles wait for one another in another order."""
+    rng = np.random.default_rng(24)
+    B, H, N = 1, 1, 700
+    Qb, Kb, Vb = (rand_bits(rng, (B, H, N, D)) for _ in range(3))
+    Q, K, V = to_dev(Qb), to_dev(Kb), to_dev(Vb)
+    shape = cn.make_shape(B, H, N, D, 0, 1, 1, N, bq, bk, Q, K, V)
+    mask = torch.ones((B, H, -(-N // bq), -(-N // bk)), dtype=torch.uint8, device="cuda")
+    ws = cn.compact_mask(mask, None, shape)
+    ws[:256].view(torch.int64)[cn.HDR_WAIT_LIMIT_NS // 8] = 2_000_000
+    ws[:256].view(torch.int32)[cn.HDR_DEBUG_WITHHOLD // 4] = 1
+    cn.sparse_attn_compacted(Q, K, V, shape, ws)
+    assert cn.query_status(ws) == cn.ERR_DEVICE_TIMEOUT
+    ws = cn.compact_mask(mask, None, shape, ws=ws)
+    O, L = cn.sparse_attn_compacted(Q, K, V, shape, ws)
+    assert cn.query_status(ws) == cn.OK
+    O_ref, L_ref = orc.attention_full(Qb, Kb, Vb, N, bq, bk, 1.0 / np.sqrt(D), mask.cpu().numpy(), None)
     check_attention(o_to_host(O), L.cpu().numpy(), O_ref, L_ref, "after a reported time-out")
 
 
@@ -454,18 +507,59 @@ def test_compacted_lists_and_order(bq, bk, N, H):
         assert longest == sorted(longest, reverse=True)
 
 
-@pytest.mark.parametrize("B,H,N,bq,D", [(2, 6, 8200, 128, 128), (3, 7, 8200, 64, 64), (1, 3, 66000, 128, 128), (5, 9, 8200, 128, 128)])
-def test_heads_that_run_in_groups(B, H, N, bq, D):
-    """The tcgen05 kernel runs several heads of a small layer side by side: short last groups (5 + 5 + 2 and 11 + 10 heads), a long
-    head and a large layer whose heads run alone, against the portable kernel (its own tests compare it with the oracle)."""
+@pytest.mark.parametrize("bq,bk,N,H", [(128, 128, 128 * 20, 2), (128, 128, 128 * 200, 2), (64, 64, 64 * 161, 1), (64, 128, 64 * 300 + 7, 1)])
+def test_compaction_with_inactive_rows_and_context_blocks(bq, bk, N, H):
+    """The region form's compaction from one CTA per head to a cluster of eight: rows that are not active count -1 and come last,
+    the others list their mask's context blocks."""
+    rng = np.random.default_rng(N)
+    B, D = 2, 64
+    nqb, nkb = -(-N // bq), -(-N // bk)
+    mask = (rng.random((B, H, nqb, nkb)) < 0.3).astype(np.uint8)
+    active, context = (rng.random((B, n)) < 0.6 for n in (nqb, nkb))
+    mask[:, :, 1] = 1
+    active[:, 1] = True
+    x = torch.zeros((B, H, N, D), dtype=torch.bfloat16, device="cuda")
+    shape = cn.make_shape(B, H, N, D, 0, 1, 1, N, bq, bk, x, x, x, x)
+    ws = torch.full((cn.attn_workspace_bytes(shape),), 0xAB, dtype=torch.uint8, device="cuda")
+    dev = lambda a: torch.from_numpy(a.astype(np.uint8)).cuda()
+    cn.sparse_attn_region(x, x, x, dev(mask), dev(active), dev(context), shape, torch.empty_like(x), torch.empty((B, H, N), device="cuda"), ws=ws)
+    eff = (mask != 0) & context[:, None, None, :] & active[:, None, :, None]
+    assert cn.query_status(ws) == cn.OK and cn.compacted_tiles(shape, ws) == int(eff.sum())
+    rows = B * H * nqb
+    al = lambda x: (x + 255) // 256 * 256
+    w = ws.cpu().numpy()
+    counts, order = (w[256 + k * al(rows * 4):][:rows * 4].view(np.int32).reshape(B * H, nqb) for k in range(2))
+    lists = w[256 + 2 * al(rows * 4):][:rows * nkb * 4].view(np.int32).reshape(B * H, nqb, nkb)
+    want = np.where(active[:, None], eff.sum(-1), -1).reshape(B * H, nqb)
+    np.testing.assert_array_equal(counts, want)
+    for bh in range(B * H):
+        for I in np.flatnonzero(want[bh] > 0):
+            np.testing.assert_array_equal(lists[bh, I, :want[bh, I]], np.flatnonzero(eff.reshape(B * H, nqb, nkb)[bh, I]))
+        c, o = want[bh], order[bh]
+        assert sorted(o.tolist()) == list(range(nqb))
+        if bq == 128:
+            np.testing.assert_array_equal(o, np.argsort(-c, kind="stable"))
+            continue
+        seq = np.lexsort((np.arange(nqb), np.where(c == nkb, 0, np.where(c > 0, 1, 2))))
+        assert {tuple(o[i:i + 2]) for i in range(0, nqb, 2)} == {tuple(seq[i:i + 2]) for i in range(0, nqb, 2)}
+        longest = [c[o[i:i + 2]].max() for i in range(0, nqb - 1, 2)]
+        assert longest == sorted(longest, reverse=True)
+
+
+@pytest.mark.parametrize("B,H,N,bq,bk,D", [(2, 6, 8200, 128, 128, 128), (3, 7, 8200, 64, 64, 64), (3, 7, 4100, 64, 64, 128), (3, 7, 4100, 128, 64, 128),
+                                           (1, 3, 66000, 128, 128, 128), (5, 9, 8200, 128, 128, 128)])
+def test_heads_that_run_in_groups(B, H, N, bq, bk, D):
+    """At D = 128 the tcgen05 kernel runs several heads of a small layer side by side: short last groups (5 + 5 + 2 heads of 8200
+    tokens, 11 + 10 of 4100), a long head and a large layer whose heads run alone; at D = 64 heads never share a group.  Against
+    the portable kernel (its own tests compare it with the oracle)."""
     gen = torch.Generator(device="cuda").manual_seed(N + H)
     Q, K, V = (torch.randn((B, H, N, D), dtype=torch.bfloat16, device="cuda", generator=gen) for _ in range(3))
-    nb = -(-N // bq)
-    mask = (torch.rand((B, H, nb, nb), device="cuda", generator=gen) < 0.04).to(torch.uint8)
+    nb, nk = -(-N // bq), -(-N // bk)
+    mask = (torch.rand((B, H, nb, nk), device="cuda", generator=gen) < 0.04).to(torch.uint8)
     rec = (torch.rand((B, nb), device="cuda", generator=gen) < 0.02).to(torch.uint8)
     out = []
     for impl in (cn.IMPL_PORTABLE, cn.IMPL_AUTO):
-        shape = cn.make_shape(B, H, N, D, 0, 1, 1, N, bq, bq, Q, K, V, attn_impl=impl)
+        shape = cn.make_shape(B, H, N, D, 0, 1, 1, N, bq, bk, Q, K, V, attn_impl=impl)
         O = torch.full((B, H, N, D), float("nan"), dtype=torch.bfloat16, device="cuda")
         O, L, ws = cn.sparse_attn(Q, K, V, mask, rec, shape, O=O)
         assert cn.query_status(ws) == cn.OK

@@ -201,3 +201,54 @@ def test_score_and_selection_at_the_edges_of_their_ranges(B, H, N, n_text, D, bq
     s = scores.cpu().numpy()
     assert np.abs(s - ref[1]).max() <= 2e-5
     check_mask(mask.cpu().numpy(), ref[0], ref[1], ref[2], ref[3], topk_mode=(mode == wl.MODE_TOPK), what=f"N={N}")
+
+
+def check_prefix(p, mask, forced, target, what):
+    """The rule on given masses p (64 bits, sum 1): always-kept blocks, and of the others the shortest prefix in descending order
+    (ties: lower index first) with which the kept mass reaches the target.  Sums of up to 1024 terms in 64 bits, in whatever
+    order, are good to 1024 * 2^-53, 1.2e-13."""
+    eps = 1.2e-13
+    free = np.flatnonzero(~forced)
+    ranked = free[np.lexsort((free, -p[free]))]
+    n = int(mask[ranked].sum())
+    assert mask[forced].all() and mask[ranked[:n]].all(), f"{what}: not a prefix"
+    kept = p[forced].sum() + p[ranked[:n]].sum()
+    assert kept >= target - eps or n == len(ranked), f"{what}: {kept} of {target}"
+    assert n == 0 or kept - p[ranked[n - 1]] < target + eps, f"{what}: longer than needed"
+    return n
+
+
+@pytest.mark.parametrize("mass", [1.0 - 2.0 ** -24, 1.0, 0.999], ids=["one_minus_2^-24", "one", "0.999"])
+@pytest.mark.parametrize("H,nb,D,spread", [(3, 61, 128, 9.0), (2, 200, 64, 9.0), (1, 500, 64, 12.0), (1, 1000, 128, 9.0), (2, 130, 64, 0.0), (1, 520, 64, -1.0),
+                                             (2, 1000, 128, -1.0)])
+def test_cumulative_mass_where_the_tail_decides(H, nb, D, spread, mass):
+    """Rows whose last admitted blocks weigh less than the 2^-31 that the search in units of 2^-30 can see (spread -1: one block
+    with nearly all of the mass, hundreds of 2^-32 each), targets that all blocks together may miss, and blocks with equal
+    scores at the threshold (every third is a copy of its neighbour; with a spread of 0 all are equal)."""
+    block, rng = 64, np.random.default_rng(nb)
+    u, v = (rng.standard_normal((1, H, nb, D)).astype(np.float32) for _ in range(2))
+    v[:, :, 2::3] = v[:, :, 1::3][:, :, :v[:, :, 2::3].shape[2]]
+    if spread < 0:
+        u[:] = u[:, :, :1]
+        v *= 0.3
+        v[:, :, 0] = u[:, :, 0] * 22.5 * np.sqrt(D) / (u[:, :, 0] ** 2).sum(-1, keepdims=True)
+    else:
+        u *= spread
+    tokens = lambda x: torch.from_numpy(np.repeat(x, block, axis=2)).cuda().to(torch.bfloat16)
+    Q, K = tokens(u), tokens(v)
+    N = nb * block
+    shape = cn.make_shape(1, H, N, D, 0, 1, 1, N, block, block, Q, K)
+    p = cn.BuildParams()
+    p.mode, p.mass, p.keep_ratio, p.window_frames, p.text_dense, p.count_includes_forced = cn.MODE_CUMMASS, mass, 0.5, -1, 0, 1
+    scores = torch.empty((1, H, nb, nb), dtype=torch.float32, device="cuda")
+    mask, ws = cn.build_connectivity(Q, K, shape, p, pooled_scores=scores)
+    assert cn.query_status(ws) == cn.OK
+    mask, scores = mask.cpu().numpy() != 0, scores.cpu().numpy().astype(np.float64)
+    target, beyond = float(np.float32(mass)), 0
+    for h in range(H):
+        for I in range(nb):
+            e = np.exp(scores[0, h, I] - scores[0, h, I].max())
+            e /= e.sum()
+            n = check_prefix(e, mask[0, h, I], np.zeros(nb, bool), target, f"head {h} row {I}")
+            beyond += n > 0 and np.sort(e)[::-1][n - 1] < 2.0 ** -31
+    assert beyond > 0 or spread == 0.0 or mass < 0.9999 or (mass < 1.0 and spread > 0)

@@ -89,3 +89,36 @@ def test_exact_builder_full_size_wan1p3b_sampled_head():
     w = wl.get("wan1p3b_480p")
     Qb, Kb, mask_g, bm_g = _run(w, 0.9)
     _check(w, 0.9, Qb, Kb, mask_g, bm_g, [(0, 5)], "wan1p3b_480p full exact mass=0.9")
+
+
+@pytest.mark.parametrize("mass", [1.0 - 2.0 ** -24, 1.0, 0.999], ids=["one_minus_2^-24", "one", "0.999"])
+@pytest.mark.parametrize("nb,D", [(37, 128), (290, 64)])
+def test_selection_where_the_tail_decides(nb, D, mass):
+    """Peaked attention: the last admitted blocks weigh less than 2^-31 or nothing at all, every third key block is a copy of its
+    neighbour; the selection against the rule on the masses that the call returns."""
+    from tests.test_gpu_builder import check_prefix
+    gen = torch.Generator(device="cuda").manual_seed(nb)
+    N = nb * 128
+    Q, K = (torch.randn((1, 1, N, D), device="cuda", generator=gen) for _ in range(2))
+    Q = (12.0 * Q.view(nb, 128, D)[:, :1].expand(nb, 128, D)).reshape(1, 1, N, D).to(torch.bfloat16)
+    K = K.view(nb, 128, D)
+    K[2::3] = K[1::3][:K[2::3].shape[0]]
+    K = K.reshape(1, 1, N, D).to(torch.bfloat16)
+    shape = cn.make_shape(1, 1, N, D, 0, 1, 1, N, 128, 128, Q, K)
+    L = _dense_lse_of(Q, K, shape, nb)
+    p = cn.BuildParams()
+    p.mode, p.mass, p.keep_ratio, p.window_frames = cn.MODE_CUMMASS, mass, 0.5, -1
+    bm = torch.empty((1, 1, nb, nb), dtype=torch.float32, device="cuda")
+    mask, ws = cn.build_connectivity_exact(Q, K, L, shape, p, block_mass=bm)
+    assert cn.query_status(ws) == cn.OK
+    mask, m = mask.cpu().numpy() != 0, bm.cpu().numpy().astype(np.float64)
+    assert (m < 2.0 ** -31).any()
+    for I in range(nb):
+        row = m[0, 0, I] / m[0, 0, I].sum()
+        check_prefix(row, mask[0, 0, I], np.zeros(nb, bool), float(np.float32(mass)), f"row {I}")
+
+
+def _dense_lse_of(Q, K, shape, nb):
+    ones = torch.ones((1, 1, nb, nb), dtype=torch.uint8, device="cuda")
+    shape.v_stride = shape.k_stride
+    return cn.sparse_attn(Q, K, K, ones, None, shape)[1]
