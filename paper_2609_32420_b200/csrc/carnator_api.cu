@@ -459,6 +459,15 @@ static carnator_status compact_impl(const uint8_t* mask, const uint8_t* recomput
     ca.H = s->H; ca.nqb = nqb; ca.nkb = nkb;
     ca.ctas = 1;
     while (ca.ctas < 8 && int64_t(nqb) * nkb > int64_t(kCompactPairsPerCta) * ca.ctas) ca.ctas *= 2;
+    // All heads at once, if that can be had by smaller clusters and then by smaller CTAs (an SM holds 2048 threads; a tenth
+    // more than fits is still one CTA for most).  384 heads of 100 rows: clusters of four 25.5 us, one CTA of 512 threads a
+    // head 15.7; 192 heads of 280 rows of 64 tokens 66.9 and 41.0; 800 heads of 40 rows 15.3 and 12.9 (256 threads).
+    int sms = 0, threads = kCompactThreads;
+    st = sm_count(&sms);
+    if (st != CARNATOR_OK) return st;
+    const int64_t heads = int64_t(s->B) * s->H, room = int64_t(sms) * 2048 * 11 / 10;
+    while (ca.ctas > 1 && heads * ca.ctas * threads > room) ca.ctas /= 2;
+    while (threads > 256 && heads * ca.ctas * threads > room) threads /= 2;
     const bool pairs = s->block_q == 64;
     const size_t smem = compact_smem(nqb, pairs);
     auto kern = pairs ? compact_order_kernel<true> : compact_order_kernel<false>;
@@ -472,7 +481,7 @@ static carnator_status compact_impl(const uint8_t* mask, const uint8_t* recomput
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = unsigned(ca.ctas); at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(unsigned(s->B) * s->H * ca.ctas); cfg.blockDim = dim3(kCompactThreads);
+    cfg.gridDim = dim3(unsigned(s->B) * s->H * ca.ctas); cfg.blockDim = dim3(unsigned(threads));
     cfg.dynamicSmemBytes = smem; cfg.stream = stream; cfg.attrs = at; cfg.numAttrs = 2;
     CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, ca));
     g_launches.fetch_add(1, std::memory_order_relaxed);

@@ -7,7 +7,7 @@
 
 namespace carnator {
 
-constexpr int kCompactThreads = 1024;
+constexpr int kCompactThreads = 1024;         // at most; 512 or 256 where there are many heads
 constexpr int kCompactPairsPerCta = 4096;
 constexpr int kMaxQueryBlocks = 12000;       // a head's sort keys in shared memory; also keeps key and index in one word
 
@@ -20,14 +20,16 @@ struct CompactArgs {
 
 // Lists, counts and order of one head by one cluster: a warp per row compacts with ballots, 128 bytes of the mask in flight,
 // then the cluster meets and every CTA ranks its share of the rows.  The cluster has 1 to 8 CTAs by the size of the head's
-// mask (4 K block pairs per CTA): one kernel where a clear and two kernels ran.  2 heads
-// of 16 rows: whole attention call 24.8 -> 21.5 us; 12 heads of 256 rows, region form: 12.1 us and a clear -> 10.2 us.
+// mask (4 K block pairs per CTA) and by the number of heads (see the launch): one kernel where a clear and two kernels ran.  2
+// heads of 16 rows: whole attention call 24.8 -> 21.5 us; 12 heads of 256 rows, region form: 12.1 us and a clear -> 10.2 us.
+// Two CTAs of 1024 threads have to fit an SM: with the next 128 bytes fetched ahead (38 registers and more) 40 heads of 592
+// rows took 46 to 61 us instead of 41.
 //   order: longest list first (stable), so that the longest CTAs of the attention kernel start first.
 //   kPairs (64-token query blocks): consecutive entries 2x, 2x+1 share a tile, so rows with like lists should meet: rows that
 //   list everything first, then the others, each by index (neighbours in the video), then the empty and skipped ones; the
 //   pairs are then put longest first.
 template <bool kPairs>
-__global__ void __launch_bounds__(kCompactThreads) compact_order_kernel(CompactArgs a) {
+__global__ void __launch_bounds__(kCompactThreads, 2) compact_order_kernel(CompactArgs a) {
     extern __shared__ __align__(16) int32_t csm[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int bh = blockIdx.x / a.ctas, rank_cta = blockIdx.x % a.ctas;
@@ -38,10 +40,11 @@ __global__ void __launch_bounds__(kCompactThreads) compact_order_kernel(CompactA
     if (blockIdx.x == 0 && tid < int(sizeof(WsHeader) / 4)) reinterpret_cast<int32_t*>(a.hdr)[tid] = 0;
     const uint8_t* ctx = a.context_k ? a.context_k + int64_t(b) * nkb : nullptr;
     unsigned active = ~0u, recomp = 0u;          // flags of this warp's next 32 rows, fetched together
-    for (int I = i_lo + warp, n_row = 0; I < i_hi; I += kCompactThreads / 32, ++n_row) {
+    const int nt = blockDim.x, nw = nt >> 5;
+    for (int I = i_lo + warp, n_row = 0; I < i_hi; I += nw, ++n_row) {
         const int64_t row = int64_t(bh) * nqb + I;
         if ((n_row & 31) == 0) {
-            const int mine = I + lane * (kCompactThreads / 32);
+            const int mine = I + lane * nw;
             const int64_t at = int64_t(b) * nqb + mine;
             const bool f_act = !a.active_q || (mine < i_hi && a.active_q[at] != 0);
             const bool f_rec = a.recompute && mine < i_hi && a.recompute[at] != 0;
@@ -92,29 +95,54 @@ __global__ void __launch_bounds__(kCompactThreads) compact_order_kernel(CompactA
         }
         return r;
     };
-    for (int i = tid; i < nq4; i += kCompactThreads) {
+    for (int i = tid; i < nq4; i += nt) {
         const int c = i < nqb ? __ldcg(a.counts + int64_t(bh) * nqb + i) : 0;
         cnt[i] = c;
-        const int v = kPairs ? (c == nkb ? 2 : (c > 0 ? 1 : 0)) : c;
-        key[i] = i < nqb ? v * 16384 + 16383 - i : INT32_MIN;
+        if (!kPairs) key[i] = i < nqb ? c * 16384 + 16383 - i : INT32_MIN;
     }
     __syncthreads();
     int32_t* order = a.order + int64_t(bh) * nqb;
     if (!kPairs) {
-        for (int i = i_lo + tid; i < i_hi; i += kCompactThreads) order[rank_of(key[i], nq4)] = i;
+        for (int i = i_lo + tid; i < i_hi; i += nt) order[rank_of(key[i], nq4)] = i;
         return;
     }
     uint16_t* const at = reinterpret_cast<uint16_t*>(csm + 2 * nq4);   // rows in pairing order
-    for (int i = tid; i < nqb; i += kCompactThreads) at[rank_of(key[i], nq4)] = uint16_t(i);
+    {   // Three classes, each by index: a thread counts those of its run of rows, a scan over the threads places them.  Ranked
+        // against all rows instead, in every CTA, 1 head of 12000 rows took 6.44 ms against 4.51, 12 heads of 512 rows 27.4 us against 19.3.
+        __shared__ uint32_t warp_sum[kCompactThreads / 32];
+        const int run = (nqb + nt - 1) / nt, r0 = min(nqb, tid * run), r1 = min(nqb, r0 + run);
+        auto bump = [&](int c) -> uint32_t { return c == nkb ? 1u << 16 : (c > 0 ? 1u : 0u); };      // full rows | other listed rows
+        uint32_t mine = 0u;
+        for (int i = r0; i < r1; ++i) mine += bump(cnt[i]);
+        uint32_t incl = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t up = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += up;
+        }
+        if (lane == 31) warp_sum[warp] = incl;
+        __syncthreads();
+        uint32_t before = incl - mine, total = 0u;
+        for (int w = 0; w < nw; ++w) {
+            if (w < warp) before += warp_sum[w];
+            total += warp_sum[w];
+        }
+        const int full = int(total >> 16), listed = int(total & 0xFFFFu);
+        int f = int(before >> 16), l = full + int(before & 0xFFFFu), e = full + listed + r0 - f - int(before & 0xFFFFu);
+        for (int i = r0; i < r1; ++i) {
+            const uint32_t b = bump(cnt[i]);
+            at[b >> 16 ? f++ : (b ? l++ : e++)] = uint16_t(i);
+        }
+    }
     __syncthreads();
     const int np = (nqb + 1) / 2, np4 = (np + 3) & ~3;
-    for (int p = tid; p < np4; p += kCompactThreads) {
+    for (int p = tid; p < np4; p += nt) {
         // a row left without a partner stays last: entries 2x, 2x + 1 have to remain pairs
         const int w = p >= np ? 0 : (2 * p + 1 < nqb ? max(cnt[at[2 * p]], cnt[at[2 * p + 1]]) : -2);
         key[p] = p < np ? w * 16384 + 16383 - p : INT32_MIN;
     }
     __syncthreads();
-    for (int p = rank_cta * kCompactThreads + tid; p < np; p += a.ctas * kCompactThreads) {
+    for (int p = rank_cta * nt + tid; p < np; p += a.ctas * nt) {
         const int r = rank_of(key[p], np4);
         order[2 * r] = at[2 * p];
         if (2 * p + 1 < nqb) order[2 * r + 1] = at[2 * p + 1];
