@@ -404,6 +404,25 @@ def test_blocks_of_64_on_the_tensor_core_kernel(D, bq, bk, N, density):
     assert cn.compacted_tiles(shape, ws) == int(eff.sum())
 
 
+@pytest.mark.parametrize("D,bq,bk", [(128, 64, 64), (64, 64, 64), (128, 128, 64), (64, 64, 128)])
+def test_every_number_of_steps_with_a_reference_that_keeps_moving(D, bq, bk):
+    """Rows of 1 to 11 listed key blocks (the three softmax groups and the tile rings come round at other steps), keys that grow from
+    block to block, so that most steps move the reference and rescale O, and halves of a pair that are several steps apart."""
+    rng = np.random.default_rng(D + bq + bk)
+    B, H, nk = 1, 1, 11
+    N = bk * (nk - 1) + 37
+    Qb, Kb, Vb = (rand_bits(rng, (B, H, N, D)) for _ in range(3))
+    grow = to_dev(Kb) * (1 + 0.5 * (torch.arange(N, device="cuda") // bk))[None, None, :, None].to(torch.bfloat16)
+    Kb = grow.view(torch.int16).cpu().numpy().view(np.uint16)
+    nq = -(-N // bq)
+    mask = np.zeros((B, H, nq, nk), dtype=np.uint8)
+    for I in range(nq):
+        mask[0, 0, I, nk - 1 - (I % nk):] = 1
+    O, L, _, _ = _run(Qb, Kb, Vb, N, 0, 1, 1, N, bq, bk, mask, None, cn.IMPL_AUTO)
+    O_ref, L_ref = orc.attention_full(Qb, Kb, Vb, N, bq, bk, 1.0 / np.sqrt(D), mask, None)
+    check_attention(o_to_host(O), L.cpu().numpy(), O_ref, L_ref, f"D{D} bq{bq} bk{bk}")
+
+
 @pytest.mark.parametrize("H,N,D,bq,bk,density,peak", [(2, 1024, 64, 64, 64, 0.4, 1), (22, 302, 64, 64, 64, 0.6, 1), (3, 528, 128, 64, 64, 0.5, 3),
                                                       (2, 4700, 128, 64, 128, 0.3, 1), (2, 3471, 64, 128, 64, 0.2, 3), (2, 2288, 128, 128, 64, 0.3, 1)])
 def test_blocks_of_64_are_no_further_from_the_exact_result(H, N, D, bq, bk, density, peak):
