@@ -420,28 +420,52 @@ __device__ __forceinline__ void select_row(const SelectArgs& a, const float* s, 
         };
         any = nfree > 0 && kept < target;
         if (any) {
-            // First on masses in units of 2^-30, whose warp sum is one instruction; the outcome is then checked in fp64.
+            // First on masses in units of 2^-20, with the count of the keys above them in the same word, so that one warp sum gives
+            // both: as soon as one key is left between the bounds, it is the threshold (about 13 steps for 139 random scores, 32
+            // down to the last bit).  The outcome is then checked in fp64.
             const uint32_t T0 = T;
-            const uint32_t goal = uint32_t(fmax(1.0, ceil((target - kept) * 1073741824.0)));
+            const uint32_t goal = uint32_t(fmax(1.0, ceil((target - kept) * 1048576.0)));
             uint32_t fine[NPL];
 #pragma unroll
-            for (int q = 0; q < NPL; ++q) fine[q] = uint32_t(e[q] * 1073741824.0 + 0.5);
+            for (int q = 0; q < NPL; ++q) fine[q] = key[q] != 0u ? (1u << 21) + uint32_t(e[q] * 1048576.0 + 0.5) : 0u;
+            int n_lo = nfree, n_hi = 0;                    // keys >= T, keys above the interval that is left
 #pragma unroll 1
             for (int bit = top; bit >= 0; --bit) {
                 const uint32_t cand = T | (1u << bit);
                 uint32_t m = 0u;
 #pragma unroll
                 for (int q = 0; q < NPL; ++q) m += key[q] >= cand ? fine[q] : 0u;
-                if (__reduce_add_sync(0xffffffffu, m) >= goal) T = cand;
+                m = __reduce_add_sync(0xffffffffu, m);
+                if ((m & 0x1FFFFFu) >= goal) { T = cand; n_lo = int(m >> 21); } else n_hi = int(m >> 21);
+                if (n_lo - n_hi <= 1) {
+                    const uint32_t last = T + ((1u << bit) - 1u);
+                    uint32_t k = 0u;
+#pragma unroll
+                    for (int q = 0; q < NPL; ++q) k = max(k, key[q] <= last ? key[q] : 0u);
+                    T = max(T, __reduce_max_sync(0xffffffffu, k));
+                    break;
+                }
             }
-            double over = mass_from(T + 1u);
-            if (!(over < target) || mass_from(T) < target) {       // not so in fp64: the same search on the masses themselves
+            double over, with;                             // mass kept with the keys > T, with the keys >= T
+            auto both_masses = [&] {
+                double gt = 0.0, eq = 0.0;
+#pragma unroll
+                for (int q = 0; q < NPL; ++q) {
+                    if (key[q] > T) gt += e[q];
+                    if (key[q] == T && key[q] != 0u) eq += e[q];
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) { gt += __shfl_xor_sync(0xffffffffu, gt, o); eq += __shfl_xor_sync(0xffffffffu, eq, o); }
+                over = kept + gt; with = kept + (gt + eq);
+            };
+            both_masses();
+            if (!(over < target) || with < target) {       // not so in fp64: the same search on the masses themselves
                 T = T0;
                 for (int bit = top; bit >= 0; --bit)
                     if (!(mass_from(T | (1u << bit)) < target)) T |= 1u << bit;
-                over = mass_from(T + 1u);
+                both_masses();
             }
-            if (mass_from(T) < target) need_eq = nkb;              // even all of them fall short: all are admitted (T is below every key)
+            if (with < target) need_eq = nkb;                      // even all of them fall short: all are admitted (T is at most the lowest key)
             else {
                 // the blocks with the threshold's key are admitted one by one, as long as the mass before them is short
                 int ties = 0;
@@ -480,15 +504,22 @@ __global__ void __launch_bounds__(256) select_rows_kernel(SelectArgs a, int rows
 
 // M2 + M3 for layers of up to 1024 key blocks: a CTA takes R query blocks of a head, computes their scores in fp32 (the
 // same sequence of FFMAs over the head dimension as score_kernel) into shared memory, and each of its R warps selects one
-// row there.  The key-block means come 128 at a time, 64 elements of the head dimension per step, through two cp.async
-// buffers; rows of 68 floats keep the 16-byte reads free of bank conflicts.  What this saves against score_kernel and a
-// selection kernel is a launch and the scores' way through memory.  Whole calls, before and after: 12 heads, 61 blocks, top-k
-// 34.1 -> 20.6 us; 48 heads, 139 blocks, cumulative mass 209 -> 61 us (the sort of every row took 153).
-constexpr int kScoreKeys = 128, kScoreLd = 68;
-template <int D, int R>
-constexpr size_t score_select_smem(int nkb) {
-    return size_t(2 * kScoreKeys * kScoreLd + R * D) * 4 + size_t(R) * ((nkb + 3) & ~3) * 4;
-}
+// row there.  A thread takes RG rows of one key block, so that a key-block mean read from shared memory serves RG products and a
+// query-block mean (one address for the warp) 32: the product is bound by those reads.  The key-block means come a tile of
+// key blocks at a time, 32 or 64 elements of the head dimension per step, through two cp.async buffers; rows of 36 or 68 floats
+// keep the 16-byte reads free of bank conflicts.  The tile is what a row of this form has, up to 256.  What this saves against score_kernel and
+// a selection kernel is a launch and the scores' way through memory.  Whole calls, against those: 12 heads, 61 blocks,
+// top-k 34.1 -> 18.5 us; 48 heads, 139 blocks, cumulative mass 209 -> 53.3 us (the sort of every row took 153; tiles of 128 key
+// blocks with four rows a thread and a search down to the last bit 59.7: this kernel alone 31.2 -> 24.6 us).
+template <int D, int R, int NPL>
+struct ScoreSelect {
+    // key blocks per tile; eight rows of 160 key blocks: two tiles of 128, whose threads take four rows, are done sooner than one of 160
+    static constexpr int kKeys = R == 8 && NPL == 5 ? 128 : (32 * NPL < 256 ? 32 * NPL : 256);
+    static constexpr int RG = kKeys <= 128 ? 4 : 8;                    // rows per thread
+    static constexpr int kSlab = kKeys <= 128 ? 64 : 32, kLd = kSlab + 4;    // elements of the head dimension per step
+    static_assert(kKeys * (R / RG) <= 32 * R && R % RG == 0, "a thread per key block and row group");
+    static constexpr size_t smem(int nkb) { return size_t(2 * kKeys * kLd + R * D) * 4 + size_t(R) * ((nkb + 3) & ~3) * 4; }
+};
 __device__ __forceinline__ void cp16(float* dst, const float* src, bool valid) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
                  ::"r"(uint32_t(__cvta_generic_to_shared(dst))), "l"(src), "r"(valid ? 16 : 0) : "memory");
@@ -496,23 +527,23 @@ __device__ __forceinline__ void cp16(float* dst, const float* src, bool valid) {
 template <int D, int R, int NPL>
 __global__ void __launch_bounds__(R * 32) score_select_kernel(const float* __restrict__ qbar, const float* __restrict__ kbar,
                                                               float* __restrict__ scores_out, float scale, SelectArgs a) {
+    using S = ScoreSelect<D, R, NPL>;
     extern __shared__ __align__(16) float ssm[];
-    constexpr int NT = R * 32, NG = NT / kScoreKeys, RG = R / NG;      // threads, row groups, rows per thread (4)
-    float* const sK = ssm;                                             // [2][128][68]
-    float* const sQ = sK + 2 * kScoreKeys * kScoreLd;                  // [R][D]
+    constexpr int NT = R * 32, RG = S::RG, kKeys = S::kKeys, kLd = S::kLd, kSlab = S::kSlab, kSlabs = D / kSlab;
+    float* const sK = ssm;                                             // [2][kKeys][kLd]
+    float* const sQ = sK + 2 * kKeys * kLd;                            // [R][D]
     float* const sS = sQ + R * D;                                      // [R][nkb_pad]
     const int nkb = a.nkb, nkb_pad = (nkb + 3) & ~3;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int I0 = blockIdx.x * R;
     const int64_t bh = int64_t(blockIdx.z) * a.H + blockIdx.y;
     const float* K = kbar + bh * nkb * D;
-    const int steps = ((nkb + kScoreKeys - 1) / kScoreKeys) * (D / 64);
+    const int steps = ((nkb + kKeys - 1) / kKeys) * kSlabs;
     auto load = [&](int st) {
-        const int j0 = (st / (D / 64)) * kScoreKeys, d0 = (st % (D / 64)) * 64;
-        for (int i = tid; i < kScoreKeys * 16; i += NT) {
-            const int j = i >> 4, c = (i & 15) * 4;
-            const bool in = j0 + j < nkb;
-            cp16(sK + (st & 1) * kScoreKeys * kScoreLd + j * kScoreLd + c, K + int64_t(in ? j0 + j : 0) * D + d0 + c, in);
+        const int j0 = (st / kSlabs) * kKeys, d0 = (st % kSlabs) * kSlab, n = min(kKeys, nkb - j0);
+        for (int i = tid; i < n * (kSlab / 4); i += NT) {
+            const int j = i / (kSlab / 4), c = (i % (kSlab / 4)) * 4;
+            cp16(sK + ((st & 1) * kKeys + j) * kLd + c, K + int64_t(j0 + j) * D + d0 + c, true);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
@@ -523,32 +554,33 @@ __global__ void __launch_bounds__(R * 32) score_select_kernel(const float* __res
     }
     load(0);
     float acc[RG];
-    const int key = tid & (kScoreKeys - 1), r0 = (tid / kScoreKeys) * RG;
+    const int key = tid % kKeys, r0 = (tid / kKeys) * RG;              // threads past the last row group only load and select
     for (int st = 0; st < steps; ++st) {
         if (st + 1 < steps) { load(st + 1); asm volatile("cp.async.wait_group 1;" ::: "memory"); }
         else asm volatile("cp.async.wait_group 0;" ::: "memory");
         __syncthreads();
-        const int d0 = (st % (D / 64)) * 64;
-        if (d0 == 0) {
+        const int d0 = (st % kSlabs) * kSlab, J = (st / kSlabs) * kKeys + key;
+        if (r0 < R && J < nkb) {
+            if (d0 == 0) {
 #pragma unroll
-            for (int r = 0; r < RG; ++r) acc[r] = 0.f;
-        }
-        const float* kr = sK + (st & 1) * kScoreKeys * kScoreLd + key * kScoreLd;
-        const float* qr = sQ + r0 * D + d0;
-#pragma unroll 4
-        for (int d = 0; d < 64; d += 4) {
-            const float4 k4 = *reinterpret_cast<const float4*>(kr + d);
-#pragma unroll
-            for (int r = 0; r < RG; ++r) {
-                const float4 q4 = *reinterpret_cast<const float4*>(qr + r * D + d);
-                acc[r] = fmaf(q4.x, k4.x, acc[r]); acc[r] = fmaf(q4.y, k4.y, acc[r]);
-                acc[r] = fmaf(q4.z, k4.z, acc[r]); acc[r] = fmaf(q4.w, k4.w, acc[r]);
+                for (int r = 0; r < RG; ++r) acc[r] = 0.f;
             }
-        }
-        const int J = (st / (D / 64)) * kScoreKeys + key;
-        if (d0 + 64 == D && J < nkb) {
+            const float* kr = sK + ((st & 1) * kKeys + key) * kLd;
+            const float* qr = sQ + r0 * D + d0;
+#pragma unroll 4
+            for (int d = 0; d < kSlab; d += 4) {
+                const float4 k4 = *reinterpret_cast<const float4*>(kr + d);
 #pragma unroll
-            for (int r = 0; r < RG; ++r) sS[(r0 + r) * nkb_pad + J] = scale * acc[r];
+                for (int r = 0; r < RG; ++r) {
+                    const float4 q4 = *reinterpret_cast<const float4*>(qr + r * D + d);
+                    acc[r] = fmaf(q4.x, k4.x, acc[r]); acc[r] = fmaf(q4.y, k4.y, acc[r]);
+                    acc[r] = fmaf(q4.z, k4.z, acc[r]); acc[r] = fmaf(q4.w, k4.w, acc[r]);
+                }
+            }
+            if (d0 + kSlab == D) {
+#pragma unroll
+                for (int r = 0; r < RG; ++r) sS[(r0 + r) * nkb_pad + J] = scale * acc[r];
+            }
         }
         __syncthreads();
     }

@@ -114,11 +114,11 @@ carnator_status allow_smem(K kernel, size_t bytes) {
 
 template <int D, int R, int NPL>
 carnator_status launch_score_select_r(const BuildWs& w, float* scores_opt, float scale, int B, const SelectArgs& sa, cudaStream_t stream) {
-    const size_t smem = score_select_smem<D, R>(sa.nkb);
+    const size_t smem = ScoreSelect<D, R, NPL>::smem(sa.nkb);
     static SmemAllowed allowed;
     const unsigned long long ctx = context_id();
     if (!allowed.has(ctx)) {      // once, for the longest row of this form
-        carnator_status st = allow_smem(score_select_kernel<D, R, NPL>, score_select_smem<D, R>(32 * NPL));
+        carnator_status st = allow_smem(score_select_kernel<D, R, NPL>, (ScoreSelect<D, R, NPL>::smem(32 * NPL)));
         if (st != CARNATOR_OK) return st;
         allowed.add(ctx);
     }
@@ -130,10 +130,13 @@ carnator_status launch_score_select_r(const BuildWs& w, float* scores_opt, float
 // Sixteen rows a CTA, unless that leaves SMs without one (twice over, so that a CTA's loads run under another's selection).
 // Rows of more than 640 blocks (32 keys a lane) fill an SM's registers with one CTA of eight rows, so there eight only as long
 // as no SM gets a second CTA: 2 heads of 900 blocks, D = 128, top-k, eight rows 74.3 us, sixteen 63.2; 1 head 41.4 and 57.7.
+// Rows of 257 to 640 blocks leave room for one CTA of sixteen or two of eight, which spread better: 31 heads of 266 blocks, D = 64,
+// cumulative mass, eight rows 112.9 us, sixteen 122.4 (48 heads of 139 blocks: 55.6 and 53.3).
 template <int D, int NPL>
 carnator_status launch_score_select_d(const BuildWs& w, float* scores_opt, float scale, int B, const SelectArgs& sa, int sms, cudaStream_t stream) {
     const int64_t heads = int64_t(B) * sa.H;
-    if (NPL > 20 ? heads * ceil_div(sa.nqb, 8) <= sms : heads * ceil_div(sa.nqb, 16) < 2 * int64_t(sms)) return launch_score_select_r<D, 8, NPL>(w, scores_opt, scale, B, sa, stream);
+    if (NPL > 20 ? heads * ceil_div(sa.nqb, 8) <= sms : heads * ceil_div(sa.nqb, 16) < (NPL == 20 ? 4 : 2) * int64_t(sms))
+        return launch_score_select_r<D, 8, NPL>(w, scores_opt, scale, B, sa, stream);
     return launch_score_select_r<D, 16, NPL>(w, scores_opt, scale, B, sa, stream);
 }
 carnator_status launch_score_select(const BuildWs& w, float* scores_opt, float scale, int B, int D, const SelectArgs& sa, int sms, cudaStream_t stream) {
@@ -141,6 +144,8 @@ carnator_status launch_score_select(const BuildWs& w, float* scores_opt, float s
 #define CARNATOR_SCORE_SELECT(NPL) \
     if (sa.nkb <= 32 * NPL) return D == 128 ? launch_score_select_d<128, NPL>(w, scores_opt, scale, B, sa, sms, stream) \
                                             : launch_score_select_d<64, NPL>(w, scores_opt, scale, B, sa, sms, stream);
+    CARNATOR_SCORE_SELECT(2)
+    CARNATOR_SCORE_SELECT(4)
     CARNATOR_SCORE_SELECT(5)
     CARNATOR_SCORE_SELECT(8)
     CARNATOR_SCORE_SELECT(20)
