@@ -319,6 +319,34 @@ __host__ __device__ constexpr uint32_t instr_desc(int M, int N, int b_mn_major) 
     return (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(b_mn_major) << 16) | (uint32_t(N >> 3) << 17) | (uint32_t(M >> 4) << 24);
 }
 
+// Output of a warp's 32 rows, half of the head dimension: O / l from tensor memory (row = lane) through shared memory (32 D bytes of
+// the K ring, which the last product has left behind) to global memory, so that a store covers whole lines.  With 16 bytes of its own
+// row per lane, a store touched 32 half sectors, and the output of a block took 1.9 us.
+template <int D>
+__device__ __forceinline__ void write_rows(uint32_t t_o, float inv, uint32_t stage, int lane, __nv_bfloat16* out, int64_t row_stride, int n_rows) {
+    constexpr int kPieces = D / 16;          // 16-byte pieces of a half row
+    auto spot = [&](int r, int p) { return stage + uint32_t(r * D + ((p ^ (D == 128 ? r & 7 : (r >> 1) & 3)) * 16)); };
+#pragma unroll
+    for (int c = 0; c < D / 64; ++c) {
+        float o[32];
+        tmem_ld32(t_o + c * 32, o);          // warp-collective: every lane takes part
+        tmem_wait_ld();
+#pragma unroll
+        for (int v = 0; v < 4; ++v)
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
+                ::"r"(spot(lane, c * 4 + v)), "r"(pack_bf16(o[8 * v] * inv, o[8 * v + 1] * inv)), "r"(pack_bf16(o[8 * v + 2] * inv, o[8 * v + 3] * inv)),
+                  "r"(pack_bf16(o[8 * v + 4] * inv, o[8 * v + 5] * inv)), "r"(pack_bf16(o[8 * v + 6] * inv, o[8 * v + 7] * inv)) : "memory");
+    }
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < kPieces; ++k) {
+        const int r = k * (32 / kPieces) + lane / kPieces, p = lane % kPieces;
+        uint4 u;
+        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(u.x), "=r"(u.y), "=r"(u.z), "=r"(u.w) : "r"(spot(r, p)) : "memory");
+        if (r < n_rows) *reinterpret_cast<uint4*>(out + r * row_stride + p * 8) = u;
+    }
+}
+
 // Shared-memory plan.  Every K / V tile is 128 rows x D held as D/64 boxes of 128 rows x 128 B
 // (128-byte swizzle).  K and V tiles travel through kStages-slot rings (separate rings, separate producers).
 template <int D>
@@ -354,11 +382,56 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
         b = int(head / uint32_t(a.H)); h = int(head - uint32_t(b) * uint32_t(a.H));
     } else { b = blockIdx.z; h = blockIdx.y; }
     const int64_t bh = int64_t(b) * a.H + h;
-    grid_wait();                            // launched while the compaction drains
     const int place = kGroups ? blockIdx.y : blockIdx.x;
+    // What the first step needs is on its way as early as it can be: the producers request the first ring of tiles as soon as the
+    // list is known, and the query rows are asked into L2, while the block sets itself up.  Waiting for the list, the header and
+    // the query rows one after the other behind the set-up, a block had its first scores 3.9 us later.  With the output in whole
+    // lines (write_rows): five-frame clip (10 blocks an SM) 384 -> 373 us, a region-restricted layer 564 -> 550, Wan-1.3B-shaped layer
+    // 2.19 -> 2.16 ms.
+    const uint32_t smem_base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
+    const uint32_t sK = smem_base + C::kOffK;
+    const uint32_t sV = smem_base + C::kOffV;
+    const uint32_t bars = smem_base + C::kOffBar;
+    const uint32_t bar_q = bars, bar_o = bars + 8, bar_drain = bars + 16, bar_drain2 = bars + 24;
+    auto bar_kfull = [&](int s) { return bars + 32 + 8 * s; };       // up to 4 stages each
+    auto bar_vfull = [&](int s) { return bars + 96 + 8 * s; };
+    auto bar_sfull = [&](int s) { return bars + 160 + 8 * s; };      // S_g holds fresh scores
+    auto bar_sfree = [&](int s) { return bars + 176 + 8 * s; };      // group g has read S_g into registers
+    auto bar_pfull = [&](int s) { return bars + 192 + 8 * s; };      // P_g is complete
+    auto bar_ref = [&](int s, int q) { return bars + 224 + 8 * (s * 4 + q); };   // r_pub slot s, lane quarter q
+    auto bar_fin = [&](int q) { return bars + 320 + 8 * q; };
+    auto bar_pvdone = [&](int s) { return bars + 352 + 8 * s; };     // P V of the step that used score buffer s has completed
+    volatile int* abortp = &abort_flag;
+    const bool producer = (warp == kWarpTmaK || warp == kWarpTmaV) && lane == 0;
+    if (producer) prefetch_tmap(warp == kWarpTmaK ? &mapK : &mapV);
+    grid_wait();                            // launched while the compaction drains
     const int I = a.order[bh * a.nqb + place];
+    // every bounded wait of this CTA gives up after `limit` (2 s unless the workspace header asks for less)
+    const unsigned long long limit = a.hdr->wait_limit_ns ? a.hdr->wait_limit_ns : kDefaultWaitNs;
+    int withhold = 0;
+    if (producer) {                         // each initialises the barriers of its own tiles, the K producer the others as well
+        if (warp == kWarpTmaK) {
+            withhold = a.hdr->debug_withhold;
+            abort_flag = 0;
+            mbar_init(bar_q, kSoftmaxWarps); mbar_init(bar_o, 1); mbar_init(bar_drain, 1); mbar_init(bar_drain2, 1);
+            for (int s = 0; s < kSBufs; ++s) {
+                mbar_init(bar_sfull(s), 1); mbar_init(bar_pvdone(s), 1);
+                mbar_init(bar_pfull(s), 4); mbar_init(bar_sfree(s), 4);          // one arrival per softmax warp of the group
+            }
+            for (int s = 0; s < kRefSlots; ++s)
+                for (int q = 0; q < 4; ++q) mbar_init(bar_ref(s, q), 1);
+            for (int q = 0; q < 4; ++q) mbar_init(bar_fin(q), 2);
+        }
+        for (int s = 0; s < kStages; ++s) mbar_init(warp == kWarpTmaK ? bar_kfull(s) : bar_vfull(s), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
     const int T = a.counts[bh * a.nqb + I];                 // steps = listed key blocks
     const int32_t* list = a.lists + (bh * a.nqb + I) * int64_t(a.nkb);
+    int first[kStages] = {};                // the first entries of the list, wherever there are so many
+    if (producer) {
+#pragma unroll
+        for (int i = 0; i < kStages; ++i) if (i < a.nkb) first[i] = list[i];
+    }
     const int q0 = I * kBlock;
     if (T < 0) return;                      // skipped query block (region-restricted form): output untouched
     if (T > a.nkb) {                        // a count that cannot come from compaction: stop before reading a list that long
@@ -375,43 +448,36 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
         return;
     }
 
-    const uint32_t smem_base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
-    const uint32_t sK = smem_base + C::kOffK;
-    const uint32_t sV = smem_base + C::kOffV;
-    const uint32_t bars = smem_base + C::kOffBar;
-    const uint32_t bar_q = bars, bar_o = bars + 8, bar_drain = bars + 16, bar_drain2 = bars + 24;
-    auto bar_kfull = [&](int s) { return bars + 32 + 8 * s; };       // up to 4 stages each
-    auto bar_vfull = [&](int s) { return bars + 96 + 8 * s; };
-    auto bar_sfull = [&](int s) { return bars + 160 + 8 * s; };      // S_g holds fresh scores
-    auto bar_sfree = [&](int s) { return bars + 176 + 8 * s; };      // group g has read S_g into registers
-    auto bar_pfull = [&](int s) { return bars + 192 + 8 * s; };      // P_g is complete
-    auto bar_ref = [&](int s, int q) { return bars + 224 + 8 * (s * 4 + q); };   // r_pub slot s, lane quarter q
-    auto bar_fin = [&](int q) { return bars + 320 + 8 * q; };
-    auto bar_pvdone = [&](int s) { return bars + 352 + 8 * s; };     // P V of the step that used score buffer s has completed
-    volatile int* abortp = &abort_flag;
-    // every bounded wait of this CTA gives up after `limit` (2 s unless the workspace header asks for less)
-    const unsigned long long limit = a.hdr->wait_limit_ns ? a.hdr->wait_limit_ns : kDefaultWaitNs;
-
+    // copies of the K (V) tile of key block J into ring slot s
+    auto load_tile = [&](bool is_k, int s, int J) {
+        const uint32_t full = is_k ? bar_kfull(s) : bar_vfull(s), dst = (is_k ? sK : sV) + s * C::kTileBytes;
+        mbar_expect_tx(full, C::kTileBytes);
+#pragma unroll
+        for (int x = 0; x < C::kBoxes; ++x) tma_load_4d(dst + x * C::kBoxBytes, is_k ? &mapK : &mapV, full, x * 64, J * kBlock, h, b);
+    };
+    int armed = -1;                         // last tile requested
+    bool malformed = false;                 // a list entry outside [0, nkb) or out of order: stop before touching memory
+    if (producer) {
+#pragma unroll
+        for (int i = 0; i < kStages; ++i) {
+            if (i >= T || malformed) break;
+            const int J = first[i];
+            malformed = J < 0 || J >= a.nkb || (i > 0 && J <= first[i > 0 ? i - 1 : 0]);
+            // Test of the time-out path only: the first K tile of the first query block in the order is never
+            // requested, so the wait for it runs out and the CTA takes the abort-and-drain path.
+            if (malformed || (i == 0 && withhold != 0 && place == 0 && bh == 0)) continue;
+            load_tile(warp == kWarpTmaK, i, J);
+            armed = i;
+        }
+    }
+    if (warp < kSoftmaxWarps) {             // the query rows, a line each: held in registers from here on they slow the loop down by 1.5 %
+        const int r = q0 + (tid & (kBlock - 1));
+        const __nv_bfloat16* qp = a.Q + b * a.qs[0] + h * a.qs[1] + int64_t(r) * a.qs[2] + (warp >> 2) * (D / 2);
+        if (r < a.N) asm volatile("prefetch.global.L2 [%0];" ::"l"(qp));
+    }
     // for the epilogue: kept in registers through the loop they slow it down by 1.3 % (grid coordinates are free, these are not)
     __shared__ volatile int at_b, at_h;
-    if (tid == 0) {
-        abort_flag = 0;
-        if (kGroups) { at_b = b; at_h = h; }
-        mbar_init(bar_q, kSoftmaxWarps); mbar_init(bar_o, 1); mbar_init(bar_drain, 1); mbar_init(bar_drain2, 1);
-        for (int s = 0; s < kStages; ++s) {
-            mbar_init(bar_kfull(s), 1); mbar_init(bar_vfull(s), 1);
-        }
-        for (int s = 0; s < kSBufs; ++s) {
-            mbar_init(bar_sfull(s), 1); mbar_init(bar_pvdone(s), 1);
-            mbar_init(bar_pfull(s), 4); mbar_init(bar_sfree(s), 4);          // one arrival per softmax warp of the group
-        }
-        for (int s = 0; s < kRefSlots; ++s)
-            for (int q = 0; q < 4; ++q) mbar_init(bar_ref(s, q), 1);
-        for (int q = 0; q < 4; ++q) mbar_init(bar_fin(q), 2);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (warp == kWarpTmaK && lane == 0) prefetch_tmap(&mapK);
-    if (warp == kWarpTmaV && lane == 0) prefetch_tmap(&mapV);
+    if (kGroups && tid == 0) { at_b = b; at_h = h; }
     if (warp == kWarpMma) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(kTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -428,24 +494,19 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
     asm volatile("setmaxnreg.dec.sync.aligned.u32 72;" ::: "memory");
     if (warp == kWarpTmaK) {
         // ================= TMA producer: the K tiles =================
+        // (the first ring is on its way)
         if (lane == 0) {
-            int armed = -1;
-            for (int i = 0; i < T; ++i) {
+            if (malformed) { set_status(a.hdr, CARNATOR_ERR_DEVICE_CHECK, 21, armed + 1, place); *abortp = 1; }
+            for (int i = kStages; i < T && !malformed; ++i) {
                 const int s = i % kStages, u = i - kStages;     // the slot is free once Q K^T of step u has completed
-                if (u >= 0 && !mbar_wait_slot(bar_sfull(0), u, abortp, limit)) {
+                if (!mbar_wait_slot(bar_sfull(0), u, abortp, limit)) {
                     set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 1, i, place); break;
                 }
                 const int J = list[i];
-                if (J < 0 || J >= a.nkb || (i > 0 && J <= list[i - 1])) {   // malformed list: stop before touching memory
+                if (J < 0 || J >= a.nkb || J <= list[i - 1]) {
                     set_status(a.hdr, CARNATOR_ERR_DEVICE_CHECK, 21, i, place); *abortp = 1; break;
                 }
-                // Test of the time-out path only: the first K tile of the first query block in the order is never
-                // requested, so the wait for it runs out and the CTA takes the abort-and-drain path.
-                if (i == 0 && a.hdr->debug_withhold != 0 && place == 0 && bh == 0) continue;
-                mbar_expect_tx(bar_kfull(s), C::kTileBytes);
-#pragma unroll
-                for (int x = 0; x < C::kBoxes; ++x)
-                    tma_load_4d(sK + s * C::kTileBytes + x * C::kBoxBytes, &mapK, bar_kfull(s), x * 64, J * kBlock, h, b);
+                load_tile(true, s, J);
                 armed = i;
             }
             if (*abortp) {      // copies in flight must land before the CTA gives its shared memory back
@@ -456,18 +517,15 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
     } else if (warp == kWarpTmaV) {
         // ================= TMA producer: the V tiles =================
         if (lane == 0) {
-            int armed = -1;
-            for (int i = 0; i < T; ++i) {
+            if (malformed) *abortp = 1;                         // reported by the K producer
+            for (int i = kStages; i < T && !malformed; ++i) {
                 const int s = i % kStages, u = i - kStages;     // the slot is free once P V of step u has completed
-                if (u >= 0 && !mbar_wait_slot(bar_pvdone(0), u, abortp, limit)) {
+                if (!mbar_wait_slot(bar_pvdone(0), u, abortp, limit)) {
                     set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 2, i, place); break;
                 }
                 const int J = list[i];
-                if (J < 0 || J >= a.nkb) { *abortp = 1; break; }   // reported by the K producer
-                mbar_expect_tx(bar_vfull(s), C::kTileBytes);
-#pragma unroll
-                for (int x = 0; x < C::kBoxes; ++x)
-                    tma_load_4d(sV + s * C::kTileBytes + x * C::kBoxBytes, &mapV, bar_vfull(s), x * 64, J * kBlock, h, b);
+                if (J < 0 || J >= a.nkb) { *abortp = 1; break; }
+                load_tile(false, s, J);
                 armed = i;
             }
             if (*abortp) {
@@ -717,24 +775,8 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
             const float inv = 1.f / l_tot;
             // each group writes half of the head dimension
             const int eb = kGroups ? at_b : b, eh = kGroups ? at_h : h;
-            __nv_bfloat16* op = a.O + eb * a.os[0] + eh * a.os[1] + int64_t(row) * a.os[2] + wg * (D / 2);
-#pragma unroll
-            for (int c = 0; c < D / 64; ++c) {
-                float o[32];
-                tmem_ld32(tmem + lane_base + kColO + wg * (D / 2) + c * 32, o);      // warp-collective: every lane takes part
-                tmem_wait_ld();
-                if (row_in) {
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) {
-                        uint4 u;
-                        u.x = pack_bf16(o[8 * v + 0] * inv, o[8 * v + 1] * inv);
-                        u.y = pack_bf16(o[8 * v + 2] * inv, o[8 * v + 3] * inv);
-                        u.z = pack_bf16(o[8 * v + 4] * inv, o[8 * v + 5] * inv);
-                        u.w = pack_bf16(o[8 * v + 6] * inv, o[8 * v + 7] * inv);
-                        *reinterpret_cast<uint4*>(op + c * 32 + v * 8) = u;
-                    }
-                }
-            }
+            __nv_bfloat16* op = a.O + eb * a.os[0] + eh * a.os[1] + int64_t(q0 + quarter * 32) * a.os[2] + wg * (D / 2);
+            write_rows<D>(tmem + lane_base + kColO + wg * (D / 2), inv, smem_base + C::kOffK + warp * (32 * D), lane, op, a.os[2], a.N - q0 - quarter * 32);
             if (wg == 0 && row_in) a.LSE[(int64_t(eb) * a.H + eh) * a.N + row] = (r_fin + log2f(l_tot)) * kLn2;
         }
     }
@@ -914,6 +956,15 @@ attn_tcgen05_b64_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_c
             a.LSE[bh * a.N + row] = -INFINITY;
         }
         return;
+    }
+    uint4 q_rows[D / 16];                             // half of a query row, by the first two softmax groups, fetched under the plan
+    if (warp < 8) {
+        const int r = tid & (kBlock - 1);
+        const bool second = kPairs && r >= BQ, in = (second ? T2 : T1) >= 0;
+        const int row = second ? q0_2 + r - BQ : q0 + r;
+        const __nv_bfloat16* qp = a.Q + b * a.qs[0] + h * a.qs[1] + int64_t(row) * a.qs[2] + (warp >> 2) * (D / 2);
+#pragma unroll
+        for (int v = 0; v < D / 16; ++v) q_rows[v] = in && row < a.N ? *reinterpret_cast<const uint4*>(qp + v * 8) : make_uint4(0, 0, 0, 0);
     }
     __shared__ int plan_total;
     unsigned char* area = smem_dyn + (((smem_u32(smem_dyn) + 1023u) & ~1023u) - smem_u32(smem_dyn)) + C::kOffPlan;
@@ -1105,11 +1156,10 @@ attn_tcgen05_b64_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_c
         if (wg < 2) {
             // The query tile goes into shared memory as the K tiles lie there (rows of 128 bytes, 16-byte pieces exchanged by
             // row); each of the first two groups brings half of the head dimension.
-            const __nv_bfloat16* qp = a.Q + b * a.qs[0] + h * a.qs[1] + int64_t(row) * a.qs[2] + wg * (D / 2);
             const uint32_t dst = sQ + (D == 128 ? wg * C::kBoxBytes : 0u) + r_loc * 128;
 #pragma unroll
             for (int v = 0; v < D / 16; ++v) {
-                const uint4 u = row_in ? *reinterpret_cast<const uint4*>(qp + v * 8) : make_uint4(0, 0, 0, 0);
+                const uint4 u = q_rows[v];
                 const int piece = D == 128 ? v : wg * 4 + v;
                 asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + uint32_t((piece ^ (r_loc & 7)) * 16)), "r"(u.x), "r"(u.y), "r"(u.z), "r"(u.w) : "memory");
             }
@@ -1276,24 +1326,10 @@ attn_tcgen05_b64_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_c
             if (kPairs && (second ? T2 : T1) <= 0) l_tot = 0.f;
             // rows of a pair that list nothing, and rows whose sum is NaN: LSE = -inf, as the portable kernel has it
             const float inv = l_tot > 0.f ? 1.f / l_tot : 0.f;
-            __nv_bfloat16* op = a.O + b * a.os[0] + h * a.os[1] + int64_t(row) * a.os[2] + wg * (D / 2);
-#pragma unroll
-            for (int c = 0; c < D / 64; ++c) {
-                float o[32];
-                tmem_ld32(tmem + lane_base + kO + wg * (D / 2) + c * 32, o);      // warp-collective: every lane takes part
-                tmem_wait_ld();
-                if (row_in) {
-#pragma unroll
-                    for (int v4 = 0; v4 < 4; ++v4) {
-                        uint4 u;
-                        u.x = pack_bf16(o[8 * v4 + 0] * inv, o[8 * v4 + 1] * inv);
-                        u.y = pack_bf16(o[8 * v4 + 2] * inv, o[8 * v4 + 3] * inv);
-                        u.z = pack_bf16(o[8 * v4 + 4] * inv, o[8 * v4 + 5] * inv);
-                        u.w = pack_bf16(o[8 * v4 + 6] * inv, o[8 * v4 + 7] * inv);
-                        *reinterpret_cast<uint4*>(op + c * 32 + v4 * 8) = u;
-                    }
-                }
-            }
+            // this warp's rows are consecutive tokens of one query block
+            const int row0 = row - lane;
+            __nv_bfloat16* op = a.O + b * a.os[0] + h * a.os[1] + int64_t(row0) * a.os[2] + wg * (D / 2);
+            write_rows<D>(tmem + lane_base + kO + wg * (D / 2), inv, sK + warp * (32 * D), lane, op, a.os[2], (kPairs && (second ? T2 : T1) < 0) ? 0 : a.N - row0);
             if (wg == 0 && row_in) a.LSE[bh * a.N + row] = l_tot > 0.f ? (r_fin + log2f(l_tot)) * kLn2 : -INFINITY;
         }
     }

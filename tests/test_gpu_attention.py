@@ -142,6 +142,27 @@ def test_strided_inputs_and_rows_past_n_untouched(impl):
     check_attention(o_to_host(O[:, :, :N]), L.cpu().numpy(), O_ref, L_ref, "strided")
 
 
+@pytest.mark.parametrize("D,block", [(128, 128), (64, 128), (128, 64), (64, 64)])
+@pytest.mark.parametrize("N", [1, 33, 95, 300])
+def test_output_in_a_token_major_buffer(D, block, N):
+    """O as a slice of a [B, rows, H, 2 D] buffer: a block's rows lie far apart, their tails end inside a warp's 32 rows, and nothing
+    beside them or behind the last token is written."""
+    rng = np.random.default_rng(N + D)
+    B, H, rows = 2, 3, N + 5
+    Qb, Kb, Vb = (rand_bits(rng, (B, H, N, D)) for _ in range(3))
+    Q, K, V = to_dev(Qb), to_dev(Kb), to_dev(Vb)
+    buf = torch.full((B, rows, H, 2 * D), 7.0, dtype=torch.bfloat16, device="cuda")
+    O = buf[..., D:].permute(0, 2, 1, 3)
+    shape = cn.make_shape(B, H, N, D, 0, 1, 1, N, block, block, Q, K, V, O)
+    nb = -(-N // block)
+    mask = (rng.random((B, H, nb, nb)) < 0.6).astype(np.uint8)
+    O, L, ws = cn.sparse_attn(Q, K, V, torch.from_numpy(mask).cuda(), None, shape, O=O)
+    assert cn.query_status(ws) == cn.OK
+    assert (buf[:, N:].float() == 7.0).all() and (buf[..., :D].float() == 7.0).all()
+    O_ref, L_ref = orc.attention_full(Qb, Kb, Vb, N, block, block, 1.0 / np.sqrt(D), mask, None)
+    check_attention(o_to_host(O[:, :, :N]), L.cpu().numpy(), O_ref, L_ref, f"D{D} block{block} N{N}")
+
+
 def test_keys_and_values_shared_over_heads():
     """A head stride of 0 broadcasts one K / V over all heads (accepted input).  A tensor map cannot express it, so the
     call must take the portable kernel and still match the oracle; asking for the tcgen05 kernel is refused."""
