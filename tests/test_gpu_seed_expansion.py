@@ -20,6 +20,10 @@ pytestmark = pytest.mark.gpu
     ("wan1p3b_480p", dict(H=3, T=8), 192, 320),      # 512 seeds: both tensor-memory chunks full; CTAs whose tile range spans two heads
     ("wan1p3b_480p", dict(H=2, T=3), 300, 100),      # the set boundary falls inside a chunk and inside a group of 32 columns
     ("cogvideox5b", dict(H=5, T=6), 257, 255),       # D = 64, a boundary one past the first chunk
+    ("wan1p3b_480p", dict(H=2, T=12), 16, 15),       # fewer columns than a group of 32; tiles of a CTA take two buffers in turn
+    ("cogvideox5b", dict(H=7, T=6), 32, 1),          # one past a group, D = 64
+    ("wan1p3b_480p", dict(H=2, T=12), 100, 156),     # the widest single chunk
+    ("wan1p3b_480p", dict(H=2, T=6), 130, 127),      # the narrowest two chunks: the second one column longer than a group
     ("wan1p3b_480p", dict(H=2, T=2), 400, 200),      # more seeds than the tensor-core form takes: the mma.sync kernel
 ])
 def test_seed_expansion_matches_oracle(name, kw, n_pos, n_neg):
