@@ -939,7 +939,7 @@ extern "C" carnator_status carnator_seed_expansion(const void* Q, const void* K,
         ta.scale_log2 = a.scale_log2;
         CUtensorMap mq, ms;      // the gathered rows as one [B*H*512, D] array: a box = 256 seed rows x 64 elements
         if (!tc::make_map(&mq, Q, s->B, s->H, s->N, s->D, s->q_stride, tc::kBlock) ||
-            !tc::make_map_2d(&ms, ga.out, int64_t(s->B) * s->H * tc::kSeedCap, s->D, tc::kSeedRows)) {
+            !tc::make_map_2d(&ms, ga.out, int64_t(s->B) * s->H * tc::kSeedCap, s->D, tc::kSeedChunk)) {
             snprintf(g_cuda_error, sizeof(g_cuda_error), "cuTensorMapEncodeTiled failed or is unavailable");
             return CARNATOR_ERR_CUDA;
         }

@@ -6,15 +6,15 @@
 // A first small kernel gathers the seed tokens' key rows of every head into one contiguous array (positives first,
 // 512 rows per head, unused rows zero).  The main kernel is persistent: a CTA takes a contiguous range of (head,
 // query tile) pairs, keeps the head's seed rows in shared memory (TMA, reloaded when the head changes), streams the
-// query tiles through a two-slot ring (TMA) and multiplies each by the seed rows (tcgen05.mma, M = 128 queries, N = the seeds
-// in whole groups of 32, up to 256: with N = 256 the query tile is read from shared memory half as often per flop as with N = 128,
-// which keeps the products off the shared-memory bandwidth limit).  More than 256 seeds are two chunks of equal width, each with a
-// buffer of tensor memory; up to 256 are one, and the tiles take two buffers in turn, so that the product of a tile runs under the
-// reading of the one before (one buffer and always 256 columns: 28 heads of 16421 tokens, 107 seeds 47.2 -> 36.9 us, 6 heads of 42323 tokens at
-// D = 64, 71 seeds 24.6 -> 18.9 us).  Two epilogue warpgroups take the tiles in turn, read the scores with tcgen05.ld and reduce
-// them to the two maxima of their row.
-// 512 seeds run at the 1000 W board limit: three or four chunks instead of two make no difference (376 and 390 against 381 us for
-// 40 heads of 75600 tokens), four column groups in flight per read instead of one take 388 us.
+// query tiles through a two-slot ring (TMA) and multiplies each by the seed rows in chunks of 256 seeds (tcgen05.mma, M = 128
+// queries, N = 256, or the seeds of the one chunk in whole groups of 32: with N = 256 the query tile is read from shared memory half as often
+// per flop as with N = 128, which keeps the products off the shared-memory bandwidth limit).  Two chunks have a buffer of tensor
+// memory each (2 x 256 fp32 columns, all 512); where one chunk is enough, the tiles take the two buffers in turn, so that the product of
+// a tile runs under the reading of the one before (one buffer and always 256 columns: 28 heads of 16421 tokens, 107 seeds 47.2 -> 36.9
+// us, 6 heads of 42323 tokens at D = 64, 71 seeds 24.6 -> 18.5 us).  Two epilogue warpgroups take the tiles in turn, read the
+// scores with tcgen05.ld and reduce them to the two maxima of their row.
+// 512 seeds run at the 1000 W board limit: three or four chunks instead of two (376 and 390 against 376 us for 40 heads of 75600
+// tokens) or four column groups in flight per read instead of one (388 us) bring nothing.
 // Every wait is bounded, as in the attention kernel.
 #pragma once
 #include "attn_tcgen05.cuh"
@@ -22,9 +22,8 @@
 namespace carnator {
 namespace tc {
 
-constexpr int kSeedCap = 512;            // seeds per call that this kernel takes: their scores fill tensor memory
-constexpr int kSeedRows = 256;           // seed rows per copy
-constexpr int kSeedChunks = 2;           // products per query tile, and buffers of tensor memory, for more than 256 seeds
+constexpr int kSeedCap = 512;            // seeds per call that this kernel takes (two chunks of tensor memory)
+constexpr int kSeedChunk = 256;          // seeds per product (N of the MMA) and per tensor-memory buffer
 constexpr int kSeedThreads = 320;        // warps 0-7: two epilogue groups; warp 8: TMA producer; warp 9: MMA issuer
 
 struct SeedTcArgs {
@@ -76,14 +75,16 @@ struct SeedCfg {
     static constexpr int kBoxes = D / 64;
     static constexpr uint32_t kQBox = 128 * 128;                    // 128 query rows x 128 B
     static constexpr uint32_t kQTile = kBoxes * kQBox;
-    static constexpr uint32_t kSBox = kSeedCap * 128;               // 512 seed rows x 128 B
+    static constexpr uint32_t kSBox = kSeedChunk * 128;             // 256 seed rows x 128 B
+    static constexpr uint32_t kSTile = kBoxes * kSBox;              // one chunk of seeds
     static constexpr uint32_t kOffSeed = 0;
-    static constexpr uint32_t kOffQ = kBoxes * kSBox;
+    static constexpr uint32_t kOffQ = (kSeedCap / kSeedChunk) * kSTile;
     static constexpr uint32_t kOffBar = kOffQ + 2 * kQTile;
     static constexpr uint32_t kSmemBytes = kOffBar + 256 + 1024;    // barriers + slack to align the base to 1 KiB
 };
 
-template <int D>
+// two: more than 256 seeds.  A template parameter: with both forms in one kernel the layer of 512 seeds took 1.5 % longer.
+template <int D, bool two>
 __global__ void __launch_bounds__(kSeedThreads, 1)
 seed_expand_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapSeed, const SeedTcArgs a) {
     using C = SeedCfg<D>;
@@ -96,8 +97,8 @@ seed_expand_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
     auto bar_qfull = [&](int s) { return bars + 8 * s; };              // query tile in ring slot s has landed
     auto bar_qfree = [&](int s) { return bars + 16 + 8 * s; };         // every product of the tile in slot s has completed
     const uint32_t bar_seed = bars + 32, bar_drain = bars + 40;        // the head's seed rows have landed
-    auto bar_sfull = [&](int g, int c) { return bars + 64 + 8 * (g * kSeedChunks + c); };   // chunk c of a tile of group g is in tensor memory
-    auto bar_sfree = [&](int u) { return bars + 128 + 8 * u; };        // the tile's group has read buffer u
+    auto bar_sfull = [&](int g, int c) { return bars + 64 + 8 * (g * 2 + c); };   // chunk c of a tile of group g is in tensor memory
+    auto bar_sfree = [&](int u) { return bars + 96 + 8 * u; };         // the tile's group has read buffer u
     volatile int* abortp = &abort_flag;
     grid_launch_dependents();
 
@@ -106,17 +107,12 @@ seed_expand_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
     const int t_begin = int(int64_t(blockIdx.x) * a.tiles / gridDim.x);
     const int t_end = int(int64_t(blockIdx.x + 1) * a.tiles / gridDim.x);
     const int ntiles = t_end - t_begin;
-    // More than 256 seeds: a buffer of tensor memory per chunk, used by every tile.  Otherwise one chunk, and the tiles take two
-    // buffers in turn.
-    const bool many = a.n_seeds > 256;
-    const int nchunks = many ? kSeedChunks : 1;
-    const int width = many ? ((a.n_seeds + kSeedChunks - 1) / kSeedChunks + 31) & ~31 : 256;      // seeds per chunk, columns per buffer
-    const int nloads = many ? kSeedCap / kSeedRows : 1;
+    const int nchunks = (a.n_seeds + kSeedChunk - 1) / kSeedChunk;     // two: a buffer of tensor memory each; one: the tiles take the buffers in turn
 
     if (tid == 0) {
         abort_flag = 0;
-        for (int s = 0; s < 2; ++s) { mbar_init(bar_qfull(s), 1); mbar_init(bar_qfree(s), 1); }
-        for (int c = 0; c < kSeedChunks; ++c) { mbar_init(bar_sfree(c), 4); mbar_init(bar_sfull(0, c), 1); mbar_init(bar_sfull(1, c), 1); }
+        for (int s = 0; s < 2; ++s) { mbar_init(bar_qfull(s), 1); mbar_init(bar_qfree(s), 1); mbar_init(bar_sfree(s), 4); }
+        for (int g = 0; g < 2; ++g) for (int c = 0; c < 2; ++c) mbar_init(bar_sfull(g, c), 1);
         mbar_init(bar_seed, 1); mbar_init(bar_drain, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -146,11 +142,11 @@ seed_expand_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
                     if (n > 0 && !mbar_wait(bar_qfree((n - 1) & 1), uint32_t((n - 1) >> 1) & 1u, abortp, 64, limit)) {
                         set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 60, n, blockIdx.x); break;
                     }
-                    mbar_expect_tx(bar_seed, uint32_t(nloads * C::kBoxes) * kSeedRows * 128u);
-                    for (int c = 0; c < nloads; ++c)
+                    mbar_expect_tx(bar_seed, uint32_t(nchunks) * C::kSTile);
+                    for (int c = 0; c < nchunks; ++c)
 #pragma unroll
                         for (int x = 0; x < C::kBoxes; ++x)
-                            tma_load_2d(sSeed + x * C::kSBox + c * (kSeedRows * 128), &mapSeed, bar_seed, x * 64, bh * kSeedCap + c * kSeedRows);
+                            tma_load_2d(sSeed + c * C::kSTile + x * C::kSBox, &mapSeed, bar_seed, x * 64, bh * kSeedCap + c * kSeedChunk);
                     seed_armed = true;
                 }
                 if (n >= 2 && !mbar_wait(bar_qfree(s), uint32_t((n - 2) >> 1) & 1u, abortp, 64, limit)) {
@@ -173,6 +169,8 @@ seed_expand_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
         // ================= MMA issuer (converged warp, one elected lane issues) =================
         const uint64_t dq = smem_desc(sQ, 16, 1024), ds = smem_desc(sSeed, 16, 1024);
         const uint32_t q_lo0 = uint32_t(dq), s_lo0 = uint32_t(ds), hi = uint32_t(dq >> 32);
+        // one chunk: as many columns as there are seeds
+        const uint32_t idesc = instr_desc(kBlock, two ? kSeedChunk : (a.n_seeds + 31) & ~31, 0);
         bool ok = true;
         int heads_seen = 0;
         for (int n = 0; n < ntiles && ok; ++n) {
@@ -187,15 +185,13 @@ seed_expand_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
             if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 63, n, blockIdx.x); break; }
             const uint32_t q_lo = q_lo0 + uint32_t(s) * (C::kQTile >> 4);
             for (int c = 0; c < nchunks && ok; ++c) {
-                const int u = many ? c : g;
-                if (n >= (many ? 1 : 2)) {       // the group of the tile before has read this buffer's scores out of tensor memory
-                    ok = mbar_wait_warp(bar_sfree(u), uint32_t(many ? n - 1 : (n - 2) >> 1) & 1u, abortp, 0, limit);
+                const int u = two ? c : g;
+                if (n >= (two ? 1 : 2)) {       // the group of the tile before has read this buffer's scores out of tensor memory
+                    ok = mbar_wait_warp(bar_sfree(u), uint32_t(two ? n - 1 : (n - 2) >> 1) & 1u, abortp, 0, limit);
                     if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 64, n, blockIdx.x); break; }
                 }
                 tc_fence_after();
-                // as many columns as the chunk has seeds (whole groups of 32)
-                const uint32_t idesc = instr_desc(kBlock, (min(width, a.n_seeds - c * width) + 31) & ~31, 0);
-                const uint32_t s_lo = s_lo0 + uint32_t(c * width) * (128 >> 4), d_s = tmem + uint32_t(u * width);
+                const uint32_t s_lo = s_lo0 + uint32_t(c) * (C::kSTile >> 4), d_s = tmem + uint32_t(u * kSeedChunk);
 #pragma unroll
                 for (int kk = 0; kk < D / 16; ++kk) {
                     const uint32_t offq = ((kk / 4) * C::kQBox + (kk % 4) * 32) >> 4, offs = ((kk / 4) * C::kSBox + (kk % 4) * 32) >> 4;
@@ -217,21 +213,21 @@ seed_expand_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
             const int t = t_begin + n;
             const int bh = t / a.nqb, I = t - bh * a.nqb;
             const int row = I * kBlock + quarter * 32 + lane;
-            const int64_t o = int64_t(bh) * a.N + row;
-            const float lse = row < a.N ? a.LSE[o] : 0.f;            // on its way while the products run
+            float lse = 0.f;                     // one chunk: on its way while the product runs
+            if (!two && row < a.N) lse = a.LSE[int64_t(bh) * a.N + row];
             float mpos = -INFINITY, mneg = -INFINITY;
             for (int c = 0; c < nchunks && ok; ++c) {
                 ok = mbar_wait_warp(bar_sfull(g, c), uint32_t(n >> 1) & 1u, abortp, 20, limit);
                 if (!ok) { if (lane == 0) set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 65, n, blockIdx.x); break; }
                 tc_fence_after();
-                const int u = many ? c : g;
-                const uint32_t t_s = tmem + lane_base + uint32_t(u * width);
+                const int u = two ? c : g;
+                const uint32_t t_s = tmem + lane_base + uint32_t(u * kSeedChunk);
 #pragma unroll 1
-                for (int at = 0; at < width; at += 32) {
-                    const int col0 = c * width + at;                       // seed index of the group's first column
+                for (int grp = 0; grp < kSeedChunk / 32; ++grp) {
+                    const int col0 = c * kSeedChunk + grp * 32;            // seed index of the group's first column
                     if (col0 >= a.n_seeds) break;                          // warp-uniform
                     float v[32];
-                    tmem_ld32(t_s + uint32_t(at), v);
+                    tmem_ld32(t_s + uint32_t(grp * 32), v);
                     tmem_wait_ld();
                     if (col0 + 32 <= a.n_pos || (col0 >= a.n_pos && col0 + 32 <= a.n_seeds)) {
                         float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};      // the whole group belongs to one set
@@ -252,7 +248,8 @@ seed_expand_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
                 mbar_arrive_warp(bar_sfree(u));
             }
             if (ok && row < a.N) {
-                const float l2 = lse * kLog2e;
+                const int64_t o = int64_t(bh) * a.N + row;
+                const float l2 = (two ? a.LSE[o] : lse) * kLog2e;
                 // an empty seed set contributes 0 (max over nothing)
                 const float pp = a.n_pos > 0 ? exp2f(mpos * a.scale_log2 - l2) : 0.f;
                 const float pn = a.n_seeds > a.n_pos ? exp2f(mneg * a.scale_log2 - l2) : 0.f;
@@ -287,7 +284,7 @@ inline carnator_status launch_seed_tc(const tc::SeedGatherArgs& ga, const tc::Se
     tc::seed_gather_kernel<D><<<ggrid, 256, 0, stream>>>(ga);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_error(e, "seed_gather_kernel", err, errlen);
-    auto kern = tc::seed_expand_tc_kernel<D>;
+    auto kern = a.n_seeds > tc::kSeedChunk ? tc::seed_expand_tc_kernel<D, true> : tc::seed_expand_tc_kernel<D, false>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::kSmemBytes));
     if (e != cudaSuccess) return cuda_error(e, "cudaFuncSetAttribute(seed tcgen05)", err, errlen);
     const int grid = a.tiles < sms ? a.tiles : sms;
