@@ -264,15 +264,22 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-// The same for a load whose registers are used across a loop: the wait hands them on, so no use of them can move above it.
-__device__ __forceinline__ void tmem_wait_ld(float (&v)[32]) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-        : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]),
-          "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), "+f"(v[14]), "+f"(v[15]),
-          "+f"(v[16]), "+f"(v[17]), "+f"(v[18]), "+f"(v[19]), "+f"(v[20]), "+f"(v[21]), "+f"(v[22]), "+f"(v[23]),
-          "+f"(v[24]), "+f"(v[25]), "+f"(v[26]), "+f"(v[27]), "+f"(v[28]), "+f"(v[29]), "+f"(v[30]), "+f"(v[31]) :: "memory");
+// Wait for this warp's loads from tensor memory.  It is given the registers that they fill and hands them on: arithmetic on them,
+// which is not volatile, depends on nothing else that would keep it behind the wait.
+template <int N>
+__device__ __forceinline__ void hand_on(float (&v)[N]) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) asm volatile("" : "+f"(v[i]));
 }
+__device__ __forceinline__ void hand_on(float& v) { asm volatile("" : "+f"(v)); }
+template <typename... V>
+__device__ __forceinline__ void tmem_wait_ld(V&... loaded) {
+    static_assert(sizeof...(V) > 0, "name what was loaded");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    (hand_on(loaded), ...);
+}
+// On the way out: a step that was given up may have left a load behind.
+__device__ __forceinline__ void tmem_drain_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
     asm volatile(
@@ -330,7 +337,7 @@ __device__ __forceinline__ void write_rows(uint32_t t_o, float inv, uint32_t sta
     for (int c = 0; c < D / 64; ++c) {
         float o[32];
         tmem_ld32(t_o + c * 32, o);          // warp-collective: every lane takes part
-        tmem_wait_ld();
+        tmem_wait_ld(o);
 #pragma unroll
         for (int v = 0; v < 4; ++v)
             asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
@@ -660,7 +667,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
             // copies, took 25.0 and 3.2 ms.
 #pragma unroll
             for (int c = 0; c < 4; ++c) tmem_ld32(tS + c * 32, s[c]);
-            tmem_wait_ld();
+            tmem_wait_ld(s[0], s[1], s[2], s[3]);
             auto mask_half = [&](int c0) {       // ragged tail (warp-uniform): keys >= N never count
                 if (nvalid < kBlock) {
 #pragma unroll
@@ -718,7 +725,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
                     for (int c = 0; c < D / 16; ++c) {
                         float o[16];
                         tmem_ld16(tmem + lane_base + kColO + c * 16, o);
-                        tmem_wait_ld();
+                        tmem_wait_ld(o);
                         uint32_t r[16];
 #pragma unroll
                         for (int e = 0; e < 16; ++e) r[e] = __float_as_uint(o[e] * f);
@@ -726,7 +733,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
                     }
                 }
                 tmem_ld32(tS, s[0]); tmem_ld32(tS + 32, s[1]);
-                tmem_wait_ld();
+                tmem_wait_ld(s[0], s[1]);
                 mask_half(0);
                 part2[0] = part2[1] = pack2(0.f, 0.f);
                 exps(0, r_now);
@@ -1196,10 +1203,10 @@ attn_tcgen05_b64_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_c
             if (on0 && on1 && nvalid == kBlock) {
                 float s0[32], s1[32], s2[32], s3[32];
                 tmem_ld32(tS, s0); tmem_ld32(tS + 32, s1);
-                tmem_wait_ld();
+                tmem_wait_ld(s0, s1);
                 tmem_ld32(tS + 64, s2); tmem_ld32(tS + 96, s3);
                 max_of(s0); max_of(s1);
-                tmem_wait_ld();
+                tmem_wait_ld(s2, s3);
                 max_of(s2); max_of(s3);
             } else {
 #pragma unroll 1
@@ -1243,7 +1250,7 @@ attn_tcgen05_b64_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_c
                 for (int c = 0; c < D / 16; ++c) {
                     float o[16];
                     tmem_ld16(tmem + lane_base + kO + c * 16, o);
-                    tmem_wait_ld();
+                    tmem_wait_ld(o);
                     uint32_t r[16];
 #pragma unroll
                     for (int e = 0; e < 16; ++e) r[e] = __float_as_uint(o[e] * f);
@@ -1302,7 +1309,7 @@ attn_tcgen05_b64_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_c
             tc_fence_before();
             mbar_arrive_warp(bar_pfull(wg));
         }
-        tmem_wait_ld();                     // a step that was given up may have left a load behind
+        tmem_drain_ld();
         // combine the groups' sums under the final reference (the later step holds the larger one)
         if (ok) {
             fin[wg][0][r_loc] = m_w;

@@ -163,7 +163,7 @@ block_mass_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
             float s[4][32];
 #pragma unroll
             for (int c = 0; c < 4; ++c) tmem_ld32(tS + c * 32, s[c]);
-            tmem_wait_ld();
+            tmem_wait_ld(s[0], s[1], s[2], s[3]);
             tc_fence_before();
             mbar_arrive_warp(bar_sfree(sb));     // the scores are in registers: the buffer may be refilled
             // exp2(s * scale - lse2), two scores per FMA-pipe instruction; -inf offset for rows past N gives 0

@@ -203,8 +203,8 @@ build_fused_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
             __nv_bfloat16* const dst = a.split[which] + (int64_t(it.bh) * nb + I) * D;
             const int64_t term_stride = int64_t(heads) * nb * D;
             tc::tc_fence_after();
-            const float sum = tmem_ld1(tmem + lane_base + uint32_t(buf * 16));
-            tc::tmem_wait_ld();
+            float sum = tmem_ld1(tmem + lane_base + uint32_t(buf * 16));
+            tc::tmem_wait_ld(sum);
             tc::tc_fence_before();
             tc::mbar_arrive_warp(bar_accfree(buf));
             if (I < nb) {
@@ -470,11 +470,11 @@ build_fused_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
                     float u[16];
                     tc::tmem_ld16(tmem_s + lane_base + uint32_t(tile * NR * NACC + c0), v[j]);                        // t1 t1 (first half of d)
                     tc::tmem_ld16(tmem_s + lane_base + uint32_t(tile * NR * NACC + (NACC - 1) * NR + c0), u);         // the small products
-                    tc::tmem_wait_ld();
+                    tc::tmem_wait_ld(v[j], u);
                     if (NACC == 3) {
                         float v2[16];
                         tc::tmem_ld16(tmem_s + lane_base + uint32_t(tile * NR * NACC + NR + c0), v2);                  // t1 t1, second half
-                        tc::tmem_wait_ld();
+                        tc::tmem_wait_ld(v2);
 #pragma unroll
                         for (int i = 0; i < 16; ++i) v[j][i] += v2[i];
                     }

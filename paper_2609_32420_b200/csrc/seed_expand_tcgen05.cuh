@@ -228,7 +228,7 @@ seed_expand_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
                     if (col0 >= a.n_seeds) break;                          // warp-uniform
                     float v[32];
                     tmem_ld32(t_s + uint32_t(grp * 32), v);
-                    tmem_wait_ld();
+                    tmem_wait_ld(v);
                     if (col0 + 32 <= a.n_pos || (col0 >= a.n_pos && col0 + 32 <= a.n_seeds)) {
                         float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};      // the whole group belongs to one set
 #pragma unroll

@@ -160,3 +160,17 @@ def test_every_wait_that_orders_tensor_memory_is_followed_by_a_fence():
         access = re.compile(r"\b(?:tmem_ld|tmem_st|mma_ts_el|mma_ss_el)").search(text, at)
         fence = text.find("tc_fence_after()", at)
         assert access is None or at < fence < access.start(), text[at - 60:access.end() + 20]
+
+
+def test_every_load_from_tensor_memory_is_handed_on_by_its_wait():
+    """Arithmetic on loaded registers is ordered behind the wait only if the wait names them; one without names leaves that to the
+    compiler's schedule (a row maximum of registers that are still being filled, without an error)."""
+    for name in sorted(os.listdir(build.CSRC)):
+        with open(os.path.join(build.CSRC, name)) as f:
+            text = re.sub(r"//[^\n]*", "", f.read())
+        loads = re.findall(r"(?:tmem_ld(?:16|32)\([^;]*, |float )(\w+(?:\[\w+\])?)(?:\)| = tmem_ld1\([^;]*\));", text)
+        calls = [m.group(1) for m in re.finditer(r"(?<!void )tmem_wait_ld\(([^;]*)\);", text)]
+        named = {v.strip() for c in calls for v in c.split(",")}
+        named |= {"s[c]"} if {"s[0]", "s[1]", "s[2]", "s[3]"} <= named else set()
+        assert "" not in named and set(loads) <= named, (name, loads, calls)
+        assert text.count("tcgen05.wait::ld") == (2 if name == "attn_tcgen05.cuh" else 0), name
