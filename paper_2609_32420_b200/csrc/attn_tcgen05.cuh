@@ -524,18 +524,19 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
     } else if (warp == kWarpTmaV) {
         // ================= TMA producer: the V tiles =================
         if (lane == 0) {
-            if (malformed) *abortp = 1;                         // reported by the K producer
+            // A malformed list is reported by the K producer, which raises the abort flag behind its report: raised here it could
+            // make a role that waits record a time-out first.
             for (int i = kStages; i < T && !malformed; ++i) {
                 const int s = i % kStages, u = i - kStages;     // the slot is free once P V of step u has completed
                 if (!mbar_wait_slot(bar_pvdone(0), u, abortp, limit)) {
                     set_status(a.hdr, CARNATOR_ERR_DEVICE_TIMEOUT, 2, i, place); break;
                 }
                 const int J = list[i];
-                if (J < 0 || J >= a.nkb) { *abortp = 1; break; }
+                if (J < 0 || J >= a.nkb) { malformed = true; break; }
                 load_tile(false, s, J);
                 armed = i;
             }
-            if (*abortp) {
+            if (malformed || *abortp) {
                 for (int k = 0; k < kStages && armed - k >= 0; ++k)
                     mbar_wait_drain(bar_vfull((armed - k) % kStages), uint32_t((armed - k) / kStages) & 1u, limit);
             }

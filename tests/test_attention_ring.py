@@ -174,3 +174,15 @@ def test_every_load_from_tensor_memory_is_handed_on_by_its_wait():
         named |= {"s[c]"} if {"s[0]", "s[1]", "s[2]", "s[3]"} <= named else set()
         assert "" not in named and set(loads) <= named, (name, loads, calls)
         assert text.count("tcgen05.wait::ld") == (2 if name == "attn_tcgen05.cuh" else 0), name
+
+
+def test_the_abort_flag_is_raised_behind_its_report():
+    """The first report stands, and a role that sees the flag while it waits reports a time-out: whoever raises the flag for another
+    reason has to have reported it."""
+    with open(os.path.join(build.CSRC, "attn_tcgen05.cuh")) as f:
+        text = re.sub(r"//[^\n]*", "", f.read())
+    text = text[text.index("attn_tcgen05_kernel("):text.index("wait_timeout_selftest_kernel")]
+    raised = [m.start() for m in re.finditer(r"\*abortp = 1", text)]
+    assert raised
+    for at in raised:
+        assert re.search(r"set_status\([^;]*\);\s*$", text[:at]), text[at - 80:at + 20]
