@@ -544,6 +544,9 @@ struct ScoreSelect {
     static constexpr int kKeys = R == 8 && NPL == 5 ? 128 : (32 * NPL < 256 ? 32 * NPL : 256);
     static constexpr int RG = kKeys <= 128 ? 4 : 8;                    // rows per thread
     static constexpr int kSlab = kKeys <= 128 ? 64 : 32, kLd = kSlab + 4;    // elements of the head dimension per step
+    // CTAs that an SM is to hold, where that has to be said (0: the compiler's choice).  It has given sixteen rows of 161 to 256 blocks 64
+    // registers or 76, and with 76 an SM holds one CTA instead of two: 48 heads of 256 blocks, D = 64, mass 0.9, 88.5 and 101.2 us.
+    static constexpr int kCtas = R == 16 && NPL == 8 ? 2 : 0;
     static_assert(kKeys * (R / RG) <= 32 * R && R % RG == 0, "a thread per key block and row group");
     static constexpr size_t smem(int nkb) { return size_t(2 * kKeys * kLd + R * D) * 4 + size_t(R) * ((nkb + 3) & ~3) * 4; }
 };
@@ -552,7 +555,7 @@ __device__ __forceinline__ void cp16(float* dst, const float* src, bool valid) {
                  ::"r"(uint32_t(__cvta_generic_to_shared(dst))), "l"(src), "r"(valid ? 16 : 0) : "memory");
 }
 template <int D, int R, int NPL>
-__global__ void __launch_bounds__(R * 32) score_select_kernel(const float* __restrict__ qbar, const float* __restrict__ kbar,
+__global__ void __launch_bounds__(R * 32, ScoreSelect<D, R, NPL>::kCtas) score_select_kernel(const float* __restrict__ qbar, const float* __restrict__ kbar,
                                                               float* __restrict__ scores_out, float scale, SelectArgs a) {
     using S = ScoreSelect<D, R, NPL>;
     extern __shared__ __align__(16) float ssm[];
