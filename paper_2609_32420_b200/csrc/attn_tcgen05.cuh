@@ -836,6 +836,8 @@ struct Cfg64 {
     static constexpr uint32_t kBoxBytes = kBlock * 128;
     static constexpr uint32_t kTileBytes = kBoxes * kBoxBytes;
     static constexpr int kKStages = 3, kVStages = D == 128 ? 2 : 3;
+    static_assert(kKStages == kSoftGroups, "a step's K slot and its score buffer are counted as one");
+    static_assert(kVStages <= kSoftGroups, "a V producer that waits for step i - kVStages must not find its barrier a step on");
     static constexpr uint32_t kOffK = 0;
     static constexpr uint32_t kOffV = kOffK + kKStages * kTileBytes;
     static constexpr uint32_t kOffQ = kOffV + kVStages * kTileBytes;
@@ -905,14 +907,6 @@ __device__ __forceinline__ int build_plan(const AttnArgs& a, const int32_t* list
     __syncthreads();
     return *total;
 }
-
-// Counts the steps of a ring of N slots: slot and phase of step i without a division.
-template <int N>
-struct Ring {
-    int slot = 0;
-    uint32_t phase = 0;
-    __device__ __forceinline__ void next() { if (++slot == N) { slot = 0; phase ^= 1u; } }
-};
 
 template <int D, int BQ, int BK>
 __global__ void __launch_bounds__(kThreads64, 1)

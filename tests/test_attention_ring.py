@@ -1,6 +1,7 @@
-"""The barriers of the tcgen05 attention kernel, every interleaving of its roles: no wait is passed before its event, and none
-is missed.  The steps' barriers and parities and the producers' rule are the kernel's own (csrc/attn_ring.h, compiled here);
-the roles' order of waits and arrivals is restated from csrc/attn_tcgen05.cuh."""
+"""The barriers of the tcgen05 attention kernels, every interleaving of their roles: no wait is passed before its event, and none
+is missed.  The steps' barriers and parities, the rings and the producers' rule are the kernels' own (csrc/attn_ring.h, compiled
+here); the roles' order of waits and arrivals is restated from csrc/attn_tcgen05.cuh: `explore` for attn_tcgen05_kernel (128-token
+blocks), `explore_b64` for attn_tcgen05_b64_kernel (64-token blocks)."""
 import ctypes
 import os
 import re
@@ -19,7 +20,10 @@ def ring(tmp_path_factory):
         f.write('#include "attn_ring.h"\nusing namespace carnator::tc;\nextern "C" int bar(int i) { return step_bar(i); }\n'
                 'extern "C" int parity(int i) { return int(step_parity(i)); }\nextern "C" int stages() { return kStages; }\n'
                 '// c0, c1: phases that the two barriers have completed\n'
-                'extern "C" int slot_free(int u, int c0, int c1) { return slot_is_free(u, [=](int b, uint32_t p) { return ((b ? c1 : c0) & 1) != int(p); }); }\n')
+                'extern "C" int slot_free(int u, int c0, int c1) { return slot_is_free(u, [=](int b, uint32_t p) { return ((b ? c1 : c0) & 1) != int(p); }); }\n'
+                'template <int N> static int at(int i) { Ring<N> r; while (i--) r.next(); return 2 * r.slot + int(r.phase); }\n'
+                '// slot and phase of step i in a ring of n slots\n'
+                'extern "C" int ring_at(int n, int i) { return n == 2 ? at<2>(i) : n == 3 ? at<3>(i) : at<4>(i); }\n')
     subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I", build.CSRC, "-o", lib, src], check=True)
     return ctypes.CDLL(lib)
 
@@ -34,9 +38,8 @@ class Early(Exception):
 
 def explore(T, stages, bar, parity, slot_free, form, warps=1):
     """Walks all reachable states of one block of T steps.  `bar`, `parity`: barrier of a step for "scores there" and "P V
-    done"; `slot_free`: the producers' rule.  `form`: "early" gives the scores' buffer back on reading them (64-token blocks), "late" after the reference,
-    "rescaling" like "late" with P V of the step before awaited in front of the reference, in every step, "low" with P V of the
-    step itself (the scores' columns hold a part of P until then).
+    done"; `slot_free`: the producers' rule.  `form`: "plain" gives the scores' buffer back once the reference is published,
+    "rescaling" awaits P V of the step before in front of that, in every step.
 
     Counters of a state: K tiles asked for / landed, V tiles asked for / landed, Q K^T issued / completed, P V issued /
     completed, then per softmax warp (group-major) its operations done.  Each role's next operation follows from its counter."""
@@ -91,9 +94,7 @@ def explore(T, stages, bar, parity, slot_free, form, warps=1):
             yield step(2)
         if vl < va:
             yield step(3)
-        sfree_op = 0 if form == "early" else 1
-        if qi < T and passed(kslot, kpar, kl, qi, "K tile") and \
-                (qi < 2 or (passed(bar, parity, pd, qi - 2, "P V") if form == "low" else group_wait(st, sfree_op, qi - 2, "scores read"))):
+        if qi < T and passed(kslot, kpar, kl, qi, "K tile") and (qi < 2 or group_wait(st, 1, qi - 2, "scores read")):
             yield step(4)
         if qd < qi:
             yield step(5)
@@ -107,9 +108,9 @@ def explore(T, stages, bar, parity, slot_free, form, warps=1):
                 i, op = g + 2 * (st[k] // n_ops), st[k] % n_ops
                 if i >= T:
                     continue
-                if op == 0:          # scores of step i are there; "early": S given back
+                if op == 0:          # scores of step i are there
                     ok = passed(bar, parity, qd, i, "Q K^T")
-                elif op == 1:        # reference of step i - 1 (from the same warp of the other group), own one published; "late": S given back
+                elif op == 1:        # reference of step i - 1 (from the same warp of the other group), own one published, S given back
                     o = st[8 + (g ^ 1) * warps + w]
                     refs = (o + 1) // n_ops                                  # steps of the other group with the reference published
                     ok = i == 0 or (refs > 0 and (g ^ 1) + 2 * (refs - 1) >= i - 1)
@@ -135,17 +136,114 @@ def explore(T, stages, bar, parity, slot_free, form, warps=1):
     return len(seen)
 
 
-@pytest.mark.parametrize("form,T,warps", [("early", 9, 1), ("late", 9, 1), ("rescaling", 9, 1), ("low", 9, 1), ("early", 6, 2), ("late", 6, 2), ("low", 6, 2)])
+def explore_b64(T, at, v_stages, rescaling, warps=1, k_stages=3, qk_waits=True):
+    """The same for the kernel of three softmax groups: a group leaves P in the columns of its scores, so that "P V of step i has
+    completed" (a barrier per group) frees the score buffer and the V slot, and Q K^T of step i + 3 waits for it.  Producers watch
+    the one barrier of the step that last used the slot.  `at`: slot and phase of a step in a ring of n slots, as 2 * slot + phase;
+    `rescaling`: P V of the step before is awaited behind the reference, in every step.
+
+    State: K tiles asked for, bits of those landed (in any order), the same for V, Q K^T issued / completed, P V issued / completed,
+    then per softmax warp (group-major) its operations done (three per step: scores there; reference taken over and published; P
+    handed over)."""
+    G, n_ops = 3, 3
+    slot, phase = lambda n, i: at(n, i) >> 1, lambda n, i: at(n, i) & 1
+
+    def passed(n, par, step, done, what):
+        """A wait with parity `par` for event `step` on a ring of n barriers; done(j): has event j happened?"""
+        c = sum(1 for j in range(step % n, T, n) if done(j))               # phases that this barrier has completed
+        ok = (c & 1) != par
+        if ok and not done(step):
+            raise Early(f"{what} {step}")
+        return ok
+
+    def moves(st):
+        ka, kl, va, vl, qi, qd, pi, pd = st[:8]
+        ops = lambda g, w: st[8 + g * warps + w]
+        below = lambda n: (lambda j: j < n)
+        landed = lambda bits: (lambda j: bool(bits >> j & 1))
+
+        def step(k, v=None):
+            n = list(st)
+            n[k] = st[k] + 1 if v is None else v
+            return tuple(n)
+        # producers: step u = i - stages, counted by Ring<3> from the first step that waits
+        if ka < T and (ka < k_stages or passed(G, phase(G, ka - k_stages), ka - k_stages, below(qd), "K slot of step")):
+            yield step(0)
+        if va < T and (va < v_stages or passed(G, phase(G, va - v_stages), va - v_stages, below(pd), "V slot of step")):
+            yield step(2)
+        for j in range(T):
+            if j < ka and not kl >> j & 1:
+                yield step(1, kl | 1 << j)
+            if j < va and not vl >> j & 1:
+                yield step(3, vl | 1 << j)
+        if qi < T and passed(k_stages, phase(k_stages, qi), qi, landed(kl), "K tile") and \
+                (qi < G or not qk_waits or passed(G, phase(G, qi) ^ 1, qi - G, below(pd), "P V")):
+            yield step(4)
+        if qd < qi:
+            yield step(5)
+        handed = lambda j: all(ops(j % G, w) >= n_ops * (j // G) + 3 for w in range(warps))
+        if pi < T and passed(v_stages, phase(v_stages, pi), pi, landed(vl), "V tile") and passed(G, phase(G, pi), pi, handed, "P"):
+            yield step(6)
+        if pd < pi:
+            yield step(7)
+        for g in range(G):
+            for w in range(warps):
+                o = ops(g, w)
+                i, op, ph = g + G * (o // n_ops), o % n_ops, o // n_ops & 1
+                if i >= T:
+                    continue
+                ph_prev = ph ^ 1 if g == 0 else ph                         # phase of step i - 1 on the barriers of its group
+                published = lambda j: ops(j % G, w) >= n_ops * (j // G) + 2
+                if op == 0:
+                    ok = passed(G, ph, i, below(qd), "Q K^T")
+                elif op == 1:
+                    ok = i == 0 or passed(G, ph_prev, i - 1, published, "reference")
+                else:
+                    ok = i == 0 or not rescaling or passed(G, ph_prev, i - 1, below(pd), "P V")
+                if ok:
+                    yield step(8 + g * warps + w)
+
+    start, full = (0,) * (8 + G * warps), (1 << T) - 1
+    end = (T, full, T, full, T, T, T, T) + tuple(n_ops * len(range(g, T, G)) for g in range(G) for _ in range(warps))
+    seen, todo = {start}, [start]
+    while todo:
+        st = todo.pop()
+        nxt = list(moves(st))
+        if not nxt and st != end:
+            raise Stuck(st)
+        for n in nxt:
+            if n not in seen:
+                seen.add(n)
+                todo.append(n)
+    assert end in seen
+    return len(seen)
+
+
+@pytest.mark.parametrize("form,T,warps", [("plain", 9, 1), ("rescaling", 9, 1), ("plain", 6, 2), ("rescaling", 6, 2)])
 def test_every_interleaving_ends_and_no_wait_is_passed_early(ring, form, T, warps):
     assert explore(T, ring.stages(), ring.bar, ring.parity, ring.slot_free, form, warps) > 1000
 
 
-@pytest.mark.parametrize("form", ["early", "late", "rescaling", "low"])
+@pytest.mark.parametrize("form", ["plain", "rescaling"])
 def test_a_producer_that_watches_one_barrier_can_miss_its_phase(ring, form):
     """The search finds the fault it is there for: a step and the one two steps on share a barrier."""
     one = lambda u, c0, c1: ((c1 if u & 1 else c0) & 1) != ((u >> 1) & 1)
     with pytest.raises(Stuck):
         explore(6, ring.stages(), ring.bar, ring.parity, one, form)
+
+
+@pytest.mark.parametrize("T,v_stages,rescaling,warps", [(8, 2, False, 1), (8, 2, True, 1), (8, 3, False, 1), (8, 3, True, 1), (5, 2, True, 2), (5, 3, False, 2)])
+def test_three_groups_every_interleaving_ends(ring, T, v_stages, rescaling, warps):
+    """V rings of the head dimensions 128 (two slots) and 64 (three)."""
+    assert explore_b64(T, ring.ring_at, v_stages, rescaling, warps) > 1000
+
+
+@pytest.mark.parametrize("change", [dict(v_stages=4), dict(k_stages=4), dict(qk_waits=False)])
+def test_three_groups_the_search_finds_faults(ring, change):
+    """A fourth slot lets the step that shares the awaited barrier run ahead of the producer (the kernel asserts that there are at
+    most as many slots as groups); without the wait for P V, Q K^T overtakes the group that reads its scores."""
+    with pytest.raises((Stuck, Early)):
+        explore_b64(8, ring.ring_at, **dict(dict(v_stages=3, rescaling=False), **change))
 
 
 def test_every_wait_that_orders_tensor_memory_is_followed_by_a_fence():
@@ -154,7 +252,7 @@ def test_every_wait_that_orders_tensor_memory_is_followed_by_a_fence():
     with open(os.path.join(build.CSRC, "attn_tcgen05.cuh")) as f:
         text = re.sub(r"//[^\n]*", "", f.read())
     text = text[text.index("attn_tcgen05_kernel("):text.index("wait_timeout_selftest_kernel")]
-    waits = [m.end() for m in re.finditer(r"mbar_wait_warp\((?:kLowInS \? )?bar_(?:sfull|sfree|pvdone|pfull|q\b|o\b)", text)]
+    waits = [m.end() for m in re.finditer(r"mbar_wait_warp\(bar_(?:sfull|sfree|pvdone|pfull|q\b|o\b)", text)]
     assert len(waits) >= 8
     for at in waits:
         access = re.compile(r"\b(?:tmem_ld|tmem_st|mma_ts_el|mma_ss_el)").search(text, at)
