@@ -130,14 +130,16 @@ carnator_status launch_score_select_r(const BuildWs& w, float* scores_opt, float
 // Sixteen rows a CTA, unless that leaves SMs without one (twice over, so that a CTA's loads run under another's selection).
 // Rows of more than 640 blocks (32 keys a lane) fill an SM's registers with one CTA of eight rows, so there eight only as long
 // as no SM gets a second CTA: 2 heads of 900 blocks, D = 128, top-k, eight rows 74.3 us, sixteen 63.2; 1 head 41.4 and 57.7.
-// Rows of 257 to 640 blocks leave room for one CTA of sixteen or two of eight, which spread better: 31 heads of 266 blocks, D = 64,
-// cumulative mass, eight rows 112.9 us, sixteen 122.4 (48 heads of 139 blocks: 55.6 and 53.3).
+// Rows of 257 to 640 blocks leave room for one CTA of sixteen or two of eight, which spread better whatever the number of heads: on
+// 80 layers of 4 to 64 heads, cumulative mass, sixteen rows took 1 to 16 % longer, none less (31 heads of 266 blocks, D = 64, 112.9 and 122.4 us;
+// 24 heads of 400 blocks 114.8 and 129.4; 48 heads of 640 383.9 and 409.7).
 template <int D, int NPL>
 carnator_status launch_score_select_d(const BuildWs& w, float* scores_opt, float scale, int B, const SelectArgs& sa, int sms, cudaStream_t stream) {
     const int64_t heads = int64_t(B) * sa.H;
-    if (NPL > 20 ? heads * ceil_div(sa.nqb, 8) <= sms : heads * ceil_div(sa.nqb, 16) < (NPL == 20 ? 4 : 2) * int64_t(sms))
-        return launch_score_select_r<D, 8, NPL>(w, scores_opt, scale, B, sa, stream);
-    return launch_score_select_r<D, 16, NPL>(w, scores_opt, scale, B, sa, stream);
+    if constexpr (NPL != 20)
+        if (!(NPL > 20 ? heads * ceil_div(sa.nqb, 8) <= sms : heads * ceil_div(sa.nqb, 16) < 2 * int64_t(sms)))
+            return launch_score_select_r<D, 16, NPL>(w, scores_opt, scale, B, sa, stream);
+    return launch_score_select_r<D, 8, NPL>(w, scores_opt, scale, B, sa, stream);
 }
 carnator_status launch_score_select(const BuildWs& w, float* scores_opt, float scale, int B, int D, const SelectArgs& sa, int sms, cudaStream_t stream) {
     // keys per lane: what a row needs costs instructions whether the row is that long or not
