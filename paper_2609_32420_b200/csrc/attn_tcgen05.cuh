@@ -393,8 +393,8 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
     // What the first step needs is on its way as early as it can be: the producers request the first ring of tiles as soon as the
     // list is known, and the query rows are asked into L2, while the block sets itself up.  Waiting for the list, the header and
     // the query rows one after the other behind the set-up, a block had its first scores 3.9 us later.  With the output in whole
-    // lines (write_rows): five-frame clip (10 blocks an SM) 384 -> 373 us, a region-restricted layer 564 -> 550, Wan-1.3B-shaped layer
-    // 2.19 -> 2.16 ms.
+    // lines (write_rows): five-frame clip (10 blocks an SM) 387 -> 375 us; a region-restricted layer and the Wan-1.3B-shaped one within
+    // what two runs differ by (552 -> 544 us, 2188 -> 2183 us).
     const uint32_t smem_base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
     const uint32_t sK = smem_base + C::kOffK;
     const uint32_t sV = smem_base + C::kOffV;
@@ -1452,7 +1452,8 @@ inline bool tcgen05_supported(const carnator_shape* s) {
 // head start when nearly everything else is done, and most SMs wait for them: five-frame clip (24 heads, 10 tiles per SM)
 // 406 -> 390 us.  Only for layers of up to 16 tiles per SM: on longer ones that wait is no longer seen.  At most as many heads as
 // keep K and V within 24 MB, so that they stay in either half of L2 (64 MB took 399 us), in groups of equal size: a short last
-// group leaves SMs idle at the end (15 heads of 3.1 MB in groups of 7, 7 and 1: 215 us, in three of 5: 198 us).
+// group leaves SMs idle at the end (15 heads of 3.1 MB in groups of 7, 7 and 1: 215 us, in three of 5: 198 us; on 38 layers of 7 to 25
+// heads of 3000 to 12000 tokens groups of unequal size took 1.4 % longer in the middle, at most 14 % longer and once 3 % less).
 constexpr int64_t kHeadGroupBytes = int64_t(24) << 20;
 constexpr int64_t kHeadGroupTiles = 16 * 148;
 inline int64_t head_group(const AttnArgs& a, int D, int tiles_per_head) {

@@ -540,7 +540,9 @@ __global__ void __launch_bounds__(256) select_rows_kernel(SelectArgs a, int rows
 // blocks with four rows a thread and a search down to the last bit 59.7: this kernel alone 31.2 -> 24.6 us).
 template <int D, int R, int NPL>
 struct ScoreSelect {
-    // key blocks per tile; eight rows of 160 key blocks: two tiles of 128, whose threads take four rows, are done sooner than one of 160
+    // key blocks per tile.  Eight rows of 129 to 160 key blocks: two tiles of 128, whose threads take four rows, are done sooner than one of
+    // 160 while an SM has one such CTA (9 heads of 139 blocks, D = 128, cumulative mass, 20.7 and 26.2 us; 24 heads 41.9 and 37.9).
+    // Sixteen rows: one tile of 160, of whose 512 threads 320 take eight rows each (48 heads 63.5 us, two tiles of 128 66.7).
     static constexpr int kKeys = R == 8 && NPL == 5 ? 128 : (32 * NPL < 256 ? 32 * NPL : 256);
     static constexpr int RG = kKeys <= 128 ? 4 : 8;                    // rows per thread
     static constexpr int kSlab = kKeys <= 128 ? 64 : 32, kLd = kSlab + 4;    // elements of the head dimension per step

@@ -127,7 +127,9 @@ carnator_status launch_score_select_r(const BuildWs& w, float* scores_opt, float
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return e == cudaSuccess ? CARNATOR_OK : cuda_fail(e, "score_select_kernel");
 }
-// Sixteen rows a CTA, unless that leaves SMs without one (twice over, so that a CTA's loads run under another's selection).
+// Sixteen rows a CTA, unless that leaves SMs without one (twice over, so that a CTA's loads run under another's selection).  Rows of up
+// to 64 blocks are right up to that line with eight (45 heads of 61 blocks, D = 64, cumulative mass, eight rows 19.1 us, sixteen 19.8);
+// longer ones want sixteen from about 1.6 CTAs an SM on (36 heads of 128 blocks 28.8 and 26.4, but 19 heads 18.7 and 20.5).
 // Rows of more than 640 blocks (32 keys a lane) fill an SM's registers with one CTA of eight rows, so there eight only as long
 // as no SM gets a second CTA: 2 heads of 900 blocks, D = 128, top-k, eight rows 74.3 us, sixteen 63.2; 1 head 41.4 and 57.7.
 // Rows of 257 to 640 blocks leave room for one CTA of sixteen or two of eight, which spread better whatever the number of heads: on
