@@ -14,7 +14,7 @@ LIB_PATH = os.path.join(PKG_DIR, "libcarnator.so")
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a",
     "-lineinfo", "-O3", "-std=c++17", "--shared",
-    "-Xcompiler", "-fPIC",
+    "-Xcompiler", "-fPIC,-fno-gnu-unique",       # two copies of the library in one process share no state
     "-I", INCLUDE, "-I", CSRC,
 ]
 

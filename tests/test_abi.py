@@ -3,6 +3,8 @@ workspace sizes, and rejects bad arguments before anything is launched."""
 import ctypes
 import os
 import re
+import shutil
+import subprocess
 
 import pytest
 
@@ -32,6 +34,16 @@ def test_exports_match_header():
         assert hasattr(L, name), name
     assert cn.version() >= 1
     assert cn.status_string(cn.OK) == "ok"
+
+
+@pytest.mark.skipif(shutil.which("nm") is None, reason="nm is not on PATH")
+def test_two_copies_in_one_process_share_no_state():
+    """The dynamic linker gives every copy of a library that is loaded one and the same instance of a "unique" symbol (what gcc makes
+    of statics in inline functions and templates).  A second copy then found its kernels' shared-memory limit on record as raised when
+    it had been raised for the first copy's kernels, and attention with 64-token blocks was refused ("invalid argument")."""
+    out = subprocess.run(["nm", "-D", "--defined-only", cn.LIB_PATH], capture_output=True, text=True, check=True).stdout
+    symbols = [line.split() for line in out.splitlines()]
+    assert any(s[1] == "T" for s in symbols) and not [s[2] for s in symbols if s[1] == "u"]
 
 
 def test_workspace_sizes():
