@@ -38,8 +38,10 @@ class Early(Exception):
 
 def explore(T, stages, bar, parity, slot_free, form, warps=1):
     """Walks all reachable states of one block of T steps.  `bar`, `parity`: barrier of a step for "scores there" and "P V
-    done"; `slot_free`: the producers' rule.  `form`: "plain" gives the scores' buffer back once the reference is published,
-    "rescaling" awaits P V of the step before in front of that, in every step.
+    done"; `slot_free`: the producers' rule.  `form`, the attn_tcgen05_kernel's own: "late" gives the scores' buffer back once the reference
+    is published, "rescaling" like "late" with P V of the step before awaited in front of the reference, in every step.  Two orders that
+    the same barriers allow and that no kernel has: "early" gives the buffer back on reading the scores, "low" with P V of the step
+    itself (the scores' columns hold a part of P until then).
 
     Counters of a state: K tiles asked for / landed, V tiles asked for / landed, Q K^T issued / completed, P V issued /
     completed, then per softmax warp (group-major) its operations done.  Each role's next operation follows from its counter."""
@@ -94,7 +96,9 @@ def explore(T, stages, bar, parity, slot_free, form, warps=1):
             yield step(2)
         if vl < va:
             yield step(3)
-        if qi < T and passed(kslot, kpar, kl, qi, "K tile") and (qi < 2 or group_wait(st, 1, qi - 2, "scores read")):
+        sfree_op = 0 if form == "early" else 1
+        if qi < T and passed(kslot, kpar, kl, qi, "K tile") and \
+                (qi < 2 or (passed(bar, parity, pd, qi - 2, "P V") if form == "low" else group_wait(st, sfree_op, qi - 2, "scores read"))):
             yield step(4)
         if qd < qi:
             yield step(5)
@@ -108,9 +112,9 @@ def explore(T, stages, bar, parity, slot_free, form, warps=1):
                 i, op = g + 2 * (st[k] // n_ops), st[k] % n_ops
                 if i >= T:
                     continue
-                if op == 0:          # scores of step i are there
+                if op == 0:          # scores of step i are there; "early": S given back
                     ok = passed(bar, parity, qd, i, "Q K^T")
-                elif op == 1:        # reference of step i - 1 (from the same warp of the other group), own one published, S given back
+                elif op == 1:        # reference of step i - 1 (from the same warp of the other group), own one published; "late": S given back
                     o = st[8 + (g ^ 1) * warps + w]
                     refs = (o + 1) // n_ops                                  # steps of the other group with the reference published
                     ok = i == 0 or (refs > 0 and (g ^ 1) + 2 * (refs - 1) >= i - 1)
@@ -219,12 +223,12 @@ def explore_b64(T, at, v_stages, rescaling, warps=1, k_stages=3, qk_waits=True):
     return len(seen)
 
 
-@pytest.mark.parametrize("form,T,warps", [("plain", 9, 1), ("rescaling", 9, 1), ("plain", 6, 2), ("rescaling", 6, 2)])
+@pytest.mark.parametrize("form,T,warps", [("early", 9, 1), ("late", 9, 1), ("rescaling", 9, 1), ("low", 9, 1), ("early", 6, 2), ("late", 6, 2), ("low", 6, 2), ("rescaling", 6, 2)])
 def test_every_interleaving_ends_and_no_wait_is_passed_early(ring, form, T, warps):
     assert explore(T, ring.stages(), ring.bar, ring.parity, ring.slot_free, form, warps) > 1000
 
 
-@pytest.mark.parametrize("form", ["plain", "rescaling"])
+@pytest.mark.parametrize("form", ["early", "late", "rescaling", "low"])
 def test_a_producer_that_watches_one_barrier_can_miss_its_phase(ring, form):
     """The search finds the fault it is there for: a step and the one two steps on share a barrier."""
     one = lambda u, c0, c1: ((c1 if u & 1 else c0) & 1) != ((u >> 1) & 1)
@@ -252,7 +256,7 @@ def test_every_wait_that_orders_tensor_memory_is_followed_by_a_fence():
     with open(os.path.join(build.CSRC, "attn_tcgen05.cuh")) as f:
         text = re.sub(r"//[^\n]*", "", f.read())
     text = text[text.index("attn_tcgen05_kernel("):text.index("wait_timeout_selftest_kernel")]
-    waits = [m.end() for m in re.finditer(r"mbar_wait_warp\(bar_(?:sfull|sfree|pvdone|pfull|q\b|o\b)", text)]
+    waits = [m.end() for m in re.finditer(r"mbar_wait_warp\((?:kLowInS \? )?bar_(?:sfull|sfree|pvdone|pfull|q\b|o\b)", text)]
     assert len(waits) >= 8
     for at in waits:
         access = re.compile(r"\b(?:tmem_ld|tmem_st|mma_ts_el|mma_ss_el)").search(text, at)
