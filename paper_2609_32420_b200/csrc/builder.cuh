@@ -544,7 +544,10 @@ struct ScoreSelect {
     // 160 while an SM has one such CTA (9 heads of 139 blocks, D = 128, cumulative mass, 20.7 and 26.2 us; 24 heads 41.9 and 37.9).
     // Sixteen rows: one tile of 160, of whose 512 threads 320 take eight rows each (48 heads 63.5 us, two tiles of 128 66.7).
     static constexpr int kKeys = R == 8 && NPL == 5 ? 128 : (32 * NPL < 256 ? 32 * NPL : 256);
-    static constexpr int RG = kKeys <= 128 ? 4 : 8;                    // rows per thread
+    // Rows per thread.  Four also where a row has up to 64 key blocks, although half of the threads are then left out of the product: with two
+    // (GPU time of whole builds) 12 heads of 61 blocks, D = 128, top-k, took 16.1 us against 15.3, 24 of 26 blocks 12.3 against 11.9, and 4
+    // heads of 13 blocks 5.8 against 5.9; only D = 64 with up to 26 blocks gained (24 heads of 13 blocks, cumulative mass, 8.9 against 9.7).
+    static constexpr int RG = kKeys <= 128 ? 4 : 8;
     static constexpr int kSlab = kKeys <= 128 ? 64 : 32, kLd = kSlab + 4;    // elements of the head dimension per step
     // CTAs that an SM is to hold, where that has to be said (0: the compiler's choice).  It has given sixteen rows of 161 to 256 blocks 64
     // registers or 76, and with 76 an SM holds one CTA instead of two: 48 heads of 256 blocks, D = 64, mass 0.9, 88.5 and 101.2 us.
